@@ -6,8 +6,11 @@
 // selected it, thousands of rows: the GEMM is bound by the tensor pipe, not
 // by the weight stream.  A work unit is one 128-row M-tile of X times one
 // 256-row weight tile over the whole K (no split); persistent CTAs (one per
-// SM) walk the units M-tile by M-tile, so the CTAs running at any time share
-// a few activation tiles and stream the weight tiles from L2.
+// SM) walk the units in groups of kPfGroup M-tiles, weight tile by weight
+// tile, so that the CTAs running at any time share about as many activation
+// tiles as weight tiles.  (M-tile by M-tile, every M-tile streams all the
+// weights: for a gate/up projection larger than L2 that is an HBM pass per
+// 128 tokens.)
 //
 // Warp 0 issues the TMA loads of a ring of stages ([X 128 x 64][X remainder
 // 128 x 64 with SPLIT][W 256 x 64], 128-byte swizzle); warp 1 issues
@@ -33,6 +36,7 @@ namespace buddy {
 
 constexpr int kPfThreads = 192;
 constexpr int kPfMaxStages = 8;
+constexpr int kPfGroup = 16;                  // M-tiles walked together
 constexpr uint32_t kPfABytes = 128u * 128u;   // one 128-row x 64-column bf16 tile
 constexpr uint32_t kPfWBytes = 256u * 128u;   // one 256-row weight tile
 
@@ -63,6 +67,16 @@ struct PfParams {
   int32_t* status;
   uint64_t wait_ns;        // limit of each pipeline wait (the drain waits keep kWaitLimitNs)
 };
+
+// M-tile and weight tile of unit u: groups of kPfGroup M-tiles, inside a group
+// the M-tile varies fastest.
+__device__ __forceinline__ void pf_unit(const PfParams& p, int u, int& mt, int& nt) {
+  const int per = kPfGroup * p.n_tiles;
+  const int g = u / per, r = u - g * per;
+  const int gm = min(kPfGroup, p.m_tiles - g * kPfGroup);
+  nt = r / gm;
+  mt = g * kPfGroup + (r - nt * gm);
+}
 
 template <int EPI>
 __device__ __forceinline__ void pf_load_w(uint8_t* st, const CUtensorMap* tw, uint64_t* bar, const PfParams& p,
@@ -233,7 +247,8 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       int issued = 0;
       bool ok = true;
       for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-        const int mt = u / p.n_tiles, nt = u - mt * p.n_tiles;
+        int mt, nt;
+        pf_unit(p, u, mt, nt);
         for (int kb = 0; kb < p.kb_total; ++kb) {
           if (!ptx::mbar_wait_bounded(&empty_bar[stage], ph ^ 1u, p.wait_ns, &abort_flag)) {
             ok = false;
@@ -314,7 +329,8 @@ __global__ void __launch_bounds__(kPfThreads, 1)
       const bool ok = ptx::mbar_wait_bounded(&tfull_bar[acc], acc_ph, p.wait_ns, &abort_flag);
       if (epi_bar_any(!ok)) break;
       ptx::tc_fence_after();
-      const int mt = u / p.n_tiles, nt = u - mt * p.n_tiles;
+      int mt, nt;
+      pf_unit(p, u, mt, nt);
       const int j = mt * 128 + q * 32 + lane;
       const uint32_t ta = tmem_base + (uint32_t)acc * 256u + ((uint32_t)(q * 32) << 16);
       pf_epilogue<EPI, SPLIT>(p, j, nt, ta);
