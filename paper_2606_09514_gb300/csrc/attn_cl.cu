@@ -60,27 +60,6 @@ __host__ __device__ constexpr size_t attn_cl_smem() {
          (size_t)kClMaxCtas * attn_cl_gstride<HD>() * 4;
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_size() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Address of the same shared-memory location in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t dsmem_addr(const void* p, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-               : "=r"(r)
-               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-  return r;
-}
 __device__ __forceinline__ void st_dsmem(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
@@ -111,7 +90,7 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
     pdl_trigger();
     return;
   }
-  const uint32_t rank = cluster_rank(), C = cluster_size();
+  const uint32_t rank = ptx::cluster_rank(), C = ptx::cluster_size();
   const int i = A.rows ? A.rows[j] : j;
   const int np = A.len[i] + 1;   // cached positions and the new token
   const int c0 = (int)((int64_t)np * rank / C), c1 = (int)((int64_t)np * (rank + 1) / C);
@@ -356,17 +335,17 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
     }
     const uint32_t own = (uint32_t)(x / SL);
     float* slot = gather + (size_t)rank * GS;
-    st_dsmem4(dsmem_addr(slot + 16 + (x - (int)own * SL), own), Ov);
+    st_dsmem4(ptx::dsmem_addr(slot + 16 + (x - (int)own * SL), own), Ov);
     // (m, l) of head hh to every owner whose slice holds one of its outputs
     if (ch == 0) {
       const uint32_t o1 = (uint32_t)(((hh + 1) * HD - 1) / SL);
       for (uint32_t o = own; o <= o1; ++o) {
-        st_dsmem(dsmem_addr(slot + hh, o), M);
-        st_dsmem(dsmem_addr(slot + 8 + hh, o), L);
+        st_dsmem(ptx::dsmem_addr(slot + hh, o), M);
+        st_dsmem(ptx::dsmem_addr(slot + 8 + hh, o), L);
       }
     }
   }
-  cluster_sync();   // every partial has landed in its owner's gather area
+  ptx::cluster_sync();   // every partial has landed in its owner's gather area
   const size_t obase = ((size_t)j * nq + (size_t)g * G) * HD;
   const int x0 = (int)rank * SL, x1 = min(G * HD, x0 + SL);
   for (int x = x0 + tid * 4; x < x1; x += kClThreads * 4) {

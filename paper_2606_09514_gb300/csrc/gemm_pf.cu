@@ -4,19 +4,29 @@
 //
 // A prefill block runs its projections on every token of the prompts that
 // selected it, thousands of rows: the GEMM is bound by the tensor pipe, not
-// by the weight stream.  A work unit is one 128-row M-tile of X times one
-// 256-row weight tile over the whole K (no split); persistent CTAs (one per
-// SM) walk the units in groups of kPfGroup M-tiles, weight tile by weight
-// tile, so that the CTAs running at any time share about as many activation
+// by the weight stream.  A work unit is a 256-row M-tile of X times one
+// 256-row weight tile over the whole K (no split), computed by a pair of CTAs
+// on two SMs (a cluster of 2, tcgen05 cta_group::2): each CTA holds 128 rows of
+// X and half of the weight tile, and 128 rows of the accumulator.  A K block
+// thus costs an SM 32 KiB of copies instead of the 48 KiB of a 128 x 256 tile
+// of its own, and the ring gets seven stages instead of four; a stage's four
+// MMAs run back to back at 128 cycles each, the tensor pipe's rate.  Qwen2.5-7B
+// gate/up at 8,000 tokens: 1.13 ms (1.92 PFLOP/s) against 2.38 ms with one-SM
+// tiles.  Persistent
+// pairs walk the units in groups of kPfGroup M-tiles, weight tile by weight
+// tile, so that the pairs running at any time share about as many activation
 // tiles as weight tiles.  (M-tile by M-tile, every M-tile streams all the
 // weights: for a gate/up projection larger than L2 that is an HBM pass per
-// 128 tokens.)
+// M-tile.)
 //
-// Warp 0 issues the TMA loads of a ring of stages ([X 128 x 64][X remainder
-// 128 x 64 with SPLIT][W 256 x 64], 128-byte swizzle); warp 1 issues
-// tcgen05.mma M = 128, N = 256, K = 16 into one of two TMEM accumulators
-// (512 columns); warps 2-5 drain the other accumulator and apply the
-// epilogue, each thread one row of the tile.  Every wait is bounded.
+// Warp 0 of each CTA issues the TMA loads of its part of a stage ([X 128 x 64]
+// [X remainder 128 x 64 with SPLIT][W 128 x 64], 128-byte swizzle; the bytes of
+// both CTAs are counted on CTA 0's barrier); warp 1 of CTA 0 issues tcgen05.mma
+// M = 256, N = 256, K = 16 into one of two TMEM accumulators (512 columns in
+// each CTA); warps 2-9 of each CTA drain the other accumulator and apply the
+// epilogue.  Every wait on a barrier is bounded; both CTAs reach the cluster
+// barriers at the end whatever happened before (they keep the pair alive while
+// MMAs read both CTAs' shared memory).
 //
 // Epilogues: residual add scattered to the token rows; SwiGLU (a tile holds
 // 128 gate rows and the matching 128 up rows); QKV (bias, rotate-half RoPE at
@@ -34,11 +44,11 @@
 
 namespace buddy {
 
-constexpr int kPfThreads = 192;
+constexpr int kPfEpiWarps = 8;               // two per TMEM lane quarter, half of the columns each
+constexpr int kPfThreads = 64 + 32 * kPfEpiWarps;
 constexpr int kPfMaxStages = 8;
-constexpr int kPfGroup = 16;                  // M-tiles walked together
-constexpr uint32_t kPfABytes = 128u * 128u;   // one 128-row x 64-column bf16 tile
-constexpr uint32_t kPfWBytes = 256u * 128u;   // one 256-row weight tile
+constexpr int kPfGroup = 8;                    // M-tiles (of 256 rows) walked together
+constexpr uint32_t kPfTileBytes = 128u * 128u; // one 128-row x 64-column bf16 tile
 
 struct PfParams {
   int N, K, m;
@@ -78,265 +88,372 @@ __device__ __forceinline__ void pf_unit(const PfParams& p, int u, int& mt, int& 
   mt = g * kPfGroup + (r - nt * gm);
 }
 
+// First row of the half of weight tile nt that CTA `rank` of the pair loads.
+// SwiGLU: CTA 0 the gate rows, CTA 1 the matching up rows (N + f0..).
 template <int EPI>
-__device__ __forceinline__ void pf_load_w(uint8_t* st, const CUtensorMap* tw, uint64_t* bar, const PfParams& p,
-                                          int tile, int kb) {
-  if (EPI == EPI_SWIGLU) {   // gate rows f0.., then the matching up rows N + f0..
-    ptx::tma_load_2d(st, tw, bar, kb * kTileK, tile * 128);
-    ptx::tma_load_2d(st + 128 * 128, tw, bar, kb * kTileK, p.N + tile * 128);
-  } else {
-    ptx::tma_load_2d(st, tw, bar, kb * kTileK, tile * 256);
-  }
+__device__ __forceinline__ int pf_w_row(const PfParams& p, int nt, uint32_t rank) {
+  return EPI == EPI_SWIGLU ? (int)rank * p.N + nt * 128 : nt * 256 + (int)rank * 128;
 }
 
-__device__ __forceinline__ void st_bf16x8(bf16* dst, const float* v) {
-  uint32_t w[4];
+// ---------------------------------------------------------------------------
+// Epilogues.  A warp takes 32 rows x 128 columns of the accumulator (columns
+// half * 128.., SwiGLU: gate columns half * 64.. and the matching up columns)
+// in mma-fragment form: thread t holds 2 neighbouring columns of rows t / 4
+// (+ 8, 16, 24), so that four threads read or write 32 contiguous bytes of an
+// fp32 row (16 bytes of a bf16 row, 32 after st_bf16_pair's exchange) and a
+// warp's access touches 8 whole sectors.  One row per thread touches 32
+// sectors for 16 bytes each: 25 us for a 256 x 256 tile's residual epilogue,
+// more than the tile's MMAs at K = 4096.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t pf_pack(float a, float b) {
+  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
+         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
+}
+__device__ __forceinline__ float pf_rest(float a) { return a - __bfloat162float(__float2bfloat16_rn(a)); }
+
+// Stores this thread's bf16 pairs of column groups g and g + 1 (8 columns
+// each) of one row: neighbouring threads exchange a pair, the even one stores
+// 4 columns of group g, the odd one 4 of group g + 1.  `row` points at column 0
+// of group g; all threads of the warp call, `ok` says which groups are stored.
+__device__ __forceinline__ void st_bf16_pair(bf16* row, uint32_t wg, uint32_t wg1, bool ok, bool ok1, int lane) {
+  const bool odd = lane & 1;
+  const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? wg : wg1, 1);
+  const uint2 v = odd ? make_uint2(got, wg1) : make_uint2(wg, got);
+  if (odd ? ok1 : ok) *reinterpret_cast<uint2*>(row + (odd ? 8 : 0) + (lane & 2) * 2) = v;
+}
+
+__device__ __forceinline__ void pf_resid(const PfParams& p, int j0, int nt, int half, uint32_t ta, int lane) {
+  const int gr = lane >> 2, tc = (lane & 3) * 2;
+  size_t off[4];
+  bool live[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    w[i] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * i])) |
-           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(v[2 * i + 1])) << 16);
-  *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-}
-
-// QKV epilogue of row j: the tile's 256 columns are 256 / HD whole heads;
-// bias, rotate-half RoPE at the token's position (pairs e, e + HD/2), q out in
-// fp32, K/V stored (bf16) at the token's position in the layer's cache.
-template <int HD>
-__device__ __forceinline__ void pf_qkv(const PfParams& p, int j, int nt, uint32_t ta) {
-  constexpr int half = HD / 2;
-  const bool live = j < p.m;
-  int seq = 0, pos = 0, cpos = 0;
-  if (live) {
-    const int row = p.rows ? p.rows[j] : j;
-    seq = p.tok_seq[row];
-    pos = p.tok_pos[row];
-    cpos = p.cache_len[seq] + (pos - p.len[seq]);
+  for (int i = 0; i < 4; ++i) {
+    const int j = j0 + gr + 8 * i;
+    live[i] = j < p.m;
+    off[i] = (size_t)(live[i] ? (p.rows ? p.rows[j] : j) : 0) * p.N;
   }
 #pragma unroll 1
-  for (int cb = 0; cb < 256; cb += HD) {
-    float x[HD];
-    ptx::tmem_ld64(ta + cb, x);
-    if (HD == 128) ptx::tmem_ld64(ta + cb + 64, x + 64);
-    const int n0 = nt * 256 + cb;   // first feature of this head
-    if (!live || n0 >= p.N) continue;
-    const int head = n0 / HD;
-    if (p.bias) {
+  for (int c0 = half * 128; c0 < half * 128 + 128; c0 += 64) {
+    const int n0 = nt * 256 + c0;
+    if (n0 >= p.N) break;   // N is a multiple of 64
+    float2 s[8][4];
 #pragma unroll
-      for (int e = 0; e < HD; ++e) x[e] += p.bias[n0 + e];
-    }
-    if (head < p.nq + p.nkv) {
-      const float* co = p.rope_cos + (size_t)pos * half;
-      const float* si = p.rope_sin + (size_t)pos * half;
+    for (int g = 0; g < 8; ++g)
 #pragma unroll
-      for (int e = 0; e < half; ++e) {
-        const float a = x[e], b = x[e + half];
-        x[e] = a * co[e] - b * si[e];
-        x[e + half] = b * co[e] + a * si[e];
-      }
-      if (head < p.nq) {
-        float4* q = reinterpret_cast<float4*>(p.q_out + (size_t)j * p.nq * HD + (size_t)head * HD);
+      for (int i = 0; i < 4; ++i)
+        if (live[i]) s[g][i] = *reinterpret_cast<const float2*>(p.resid_src + off[i] + n0 + 8 * g + tc);
+    __syncwarp();
+    uint32_t v[2][32];
+    ptx::tmem_ld_frag<8>(ta + c0, v[0]);
+    ptx::tmem_ld_frag<8>(ta + c0 + (16u << 16), v[1]);
+    ptx::tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < HD; e += 4) q[e >> 2] = make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
-      } else {
-        bf16* k = p.kc + kv_offset(p.seq_off, p.cap, seq, p.nkv, HD, head - p.nq, cpos);
+    for (int g = 0; g < 8; ++g)
 #pragma unroll
-        for (int e = 0; e < HD; e += 8) st_bf16x8(k + e, x + e);
-      }
-    } else {
-      bf16* v = p.vc + kv_offset(p.seq_off, p.cap, seq, p.nkv, HD, head - p.nq - p.nkv, cpos);
-#pragma unroll
-      for (int e = 0; e < HD; e += 8) st_bf16x8(v + e, x + e);
-    }
+      for (int i = 0; i < 4; ++i)
+        if (live[i])
+          *reinterpret_cast<float2*>(p.resid_dst + off[i] + n0 + 8 * g + tc) =
+              make_float2(s[g][i].x + __uint_as_float(v[i >> 1][4 * g + (i & 1) * 2]),
+                          s[g][i].y + __uint_as_float(v[i >> 1][4 * g + (i & 1) * 2 + 1]));
   }
 }
 
-// Epilogue of row j (lane of this warp's TMEM quarter) of unit tile nt.  All
-// lanes run the TMEM loads (warp-collective); only rows j < m store.
-template <int EPI, bool SPLIT>
-__device__ __forceinline__ void pf_epilogue(const PfParams& p, int j, int nt, uint32_t ta) {
-  const bool live = j < p.m;
-  if (EPI == EPI_RESID) {
-    const int row = live ? (p.rows ? p.rows[j] : j) : 0;
-    for (int c0 = 0; c0 < 256; c0 += 64) {
-      float v[64];
-      ptx::tmem_ld64(ta + c0, v);
-      const int n0 = nt * 256 + c0;
-      if (!live || n0 >= p.N) continue;   // N is a multiple of 64
-      const float4* src = reinterpret_cast<const float4*>(p.resid_src + (size_t)row * p.N + n0);
-      float4* dst = reinterpret_cast<float4*>(p.resid_dst + (size_t)row * p.N + n0);
+template <bool SPLIT>
+__device__ __forceinline__ void pf_swiglu(const PfParams& p, int j0, int nt, int half, uint32_t ta, int lane) {
+  const int gr = lane >> 2;
+  const int f0 = nt * 128 + half * 64;
+#pragma unroll 1
+  for (int h16 = 0; h16 < 2; ++h16) {
+    uint32_t g_[32], u_[32];
+    const uint32_t t16 = ta + ((uint32_t)(h16 * 16) << 16);
+    ptx::tmem_ld_frag<8>(t16 + half * 64, g_);
+    ptx::tmem_ld_frag<8>(t16 + 128 + half * 64, u_);
+    ptx::tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float4 s = src[i];
-        dst[i] = make_float4(s.x + v[4 * i], s.y + v[4 * i + 1], s.z + v[4 * i + 2], s.w + v[4 * i + 3]);
-      }
-    }
-  } else if (EPI == EPI_SWIGLU) {
-    for (int h = 0; h < 128; h += 64) {
-      float g[64], u[64];
-      ptx::tmem_ld64(ta + h, g);
-      ptx::tmem_ld64(ta + 128 + h, u);
-      if (!live) continue;
-      const int f0 = nt * 128 + h;
+    for (int i = 0; i < 2; ++i) {
+      const int j = j0 + h16 * 16 + gr + 8 * i;
+      const bool live = j < p.m;
+      const size_t at = (size_t)j * p.N + f0;
 #pragma unroll
-      for (int i = 0; i < 64; i += 8) {
-        if (f0 + i >= p.N) break;   // N is a multiple of 8
-        float a[8], lo[8];
+      for (int g = 0; g < 8; g += 2) {
+        float a[4];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          a[e] = silu_f(g[i + e]) * u[i + e];
-          lo[e] = a[e] - __bfloat162float(__float2bfloat16_rn(a[e]));
+        for (int e = 0; e < 4; ++e) {
+          const int k = 4 * (g + (e >> 1)) + 2 * i + (e & 1);
+          a[e] = silu_f(__uint_as_float(g_[k])) * __uint_as_float(u_[k]);
         }
-        st_bf16x8(p.out_act + (size_t)j * p.N + f0 + i, a);
-        if (SPLIT) st_bf16x8(p.out_act_lo + (size_t)j * p.N + f0 + i, lo);
+        const bool ok = live && f0 + 8 * g < p.N, ok1 = live && f0 + 8 * g + 8 < p.N;   // N is a multiple of 8
+        st_bf16_pair(p.out_act + at + 8 * g, pf_pack(a[0], a[1]), pf_pack(a[2], a[3]), ok, ok1, lane);
+        if (SPLIT)
+          st_bf16_pair(p.out_act_lo + at + 8 * g, pf_pack(pf_rest(a[0]), pf_rest(a[1])),
+                       pf_pack(pf_rest(a[2]), pf_rest(a[3])), ok, ok1, lane);
       }
     }
-  } else if (p.hd == 128) {
-    pf_qkv<128>(p, j, nt, ta);
-  } else {
-    pf_qkv<64>(p, j, nt, ta);
   }
 }
 
+// QKV: the tile's 256 columns are 256 / HD whole heads; bias, rotate-half RoPE
+// at the token's position (pairs e, e + HD/2), q out in fp32, K/V stored (bf16)
+// at the token's position in the layer's cache.
+template <int HD>
+__device__ __forceinline__ void pf_qkv(const PfParams& p, int j0, int nt, int half, uint32_t ta, int lane) {
+  constexpr int HH = HD / 2, G = HH / 8;
+  const int gr = lane >> 2, tc = (lane & 3) * 2;
+  int seq[4], pos[4], cpos[4];
+  bool live[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int j = j0 + gr + 8 * i;
+    live[i] = j < p.m;
+    const int row = live[i] ? (p.rows ? p.rows[j] : j) : 0;
+    seq[i] = p.tok_seq[row];
+    pos[i] = p.tok_pos[row];
+    cpos[i] = p.cache_len[seq[i]] + (pos[i] - p.len[seq[i]]);
+  }
+#pragma unroll 1
+  for (int cb = half * 128; cb < half * 128 + 128; cb += HD) {
+    const int n0 = nt * 256 + cb;   // first feature of this head
+    if (n0 >= p.N) break;
+    const int head = n0 / HD;
+#pragma unroll
+    for (int h16 = 0; h16 < 2; ++h16) {
+      __syncwarp();
+      uint32_t a_[4 * G], b_[4 * G];
+      const uint32_t t16 = ta + cb + ((uint32_t)(h16 * 16) << 16);
+      ptx::tmem_ld_frag<G>(t16, a_);
+      ptx::tmem_ld_frag<G>(t16 + HH, b_);
+      ptx::tmem_wait_ld();
+      float x[4 * G], y[4 * G];   // columns e and e + HD/2
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+        float ba[2] = {0.f, 0.f}, bb[2] = {0.f, 0.f};   // scalar loads: the bias may be 4-byte aligned
+        if (p.bias) {
+          const float* b = p.bias + n0 + 8 * g + tc;
+          ba[0] = b[0];
+          ba[1] = b[1];
+          bb[0] = b[HH];
+          bb[1] = b[HH + 1];
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int k = 4 * g + 2 * i;
+          x[k] = __uint_as_float(a_[k]) + ba[0];
+          x[k + 1] = __uint_as_float(a_[k + 1]) + ba[1];
+          y[k] = __uint_as_float(b_[k]) + bb[0];
+          y[k + 1] = __uint_as_float(b_[k + 1]) + bb[1];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int r = 2 * h16 + i;
+        if (head < p.nq + p.nkv) {
+          const float* co = p.rope_cos + (size_t)pos[r] * HH + tc;
+          const float* si = p.rope_sin + (size_t)pos[r] * HH + tc;
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            const float2 c2 = *reinterpret_cast<const float2*>(co + 8 * g);
+            const float2 s2 = *reinterpret_cast<const float2*>(si + 8 * g);
+            const int k = 4 * g + 2 * i;
+            const float u0 = x[k], v0 = y[k], u1 = x[k + 1], v1 = y[k + 1];
+            x[k] = u0 * c2.x - v0 * s2.x;
+            y[k] = v0 * c2.x + u0 * s2.x;
+            x[k + 1] = u1 * c2.y - v1 * s2.y;
+            y[k + 1] = v1 * c2.y + u1 * s2.y;
+          }
+        }
+        if (head < p.nq) {
+          if (live[r]) {
+            float* q = p.q_out + (size_t)(j0 + gr + 8 * r) * p.nq * HD + (size_t)head * HD + tc;
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+              const int k = 4 * g + 2 * i;
+              *reinterpret_cast<float2*>(q + 8 * g) = make_float2(x[k], x[k + 1]);
+              *reinterpret_cast<float2*>(q + HH + 8 * g) = make_float2(y[k], y[k + 1]);
+            }
+          }
+        } else {
+          const bool isk = head < p.nq + p.nkv;
+          bf16* c = (isk ? p.kc : p.vc) + kv_offset(p.seq_off, p.cap, seq[r], p.nkv, HD,
+                                                    head - p.nq - (isk ? 0 : p.nkv), cpos[r]);
+#pragma unroll
+          for (int g = 0; g < G; g += 2) {
+            const int k = 4 * g + 2 * i;
+            st_bf16_pair(c + 8 * g, pf_pack(x[k], x[k + 1]), pf_pack(x[k + 4], x[k + 5]), live[r], live[r], lane);
+            st_bf16_pair(c + HH + 8 * g, pf_pack(y[k], y[k + 1]), pf_pack(y[k + 4], y[k + 5]), live[r], live[r],
+                         lane);
+          }
+        }
+      }
+    }
+  }
+}
+
+// Epilogue of rows j0 .. j0 + 31 (this warp's TMEM quarter at ta) of unit tile
+// nt, one half of its columns.
 template <int EPI, bool SPLIT>
-__global__ void __launch_bounds__(kPfThreads, 1)
+__device__ __forceinline__ void pf_epilogue(const PfParams& p, int j0, int nt, int half, uint32_t ta, int lane) {
+  if (EPI == EPI_RESID) pf_resid(p, j0, nt, half, ta, lane);
+  else if (EPI == EPI_SWIGLU) pf_swiglu<SPLIT>(p, j0, nt, half, ta, lane);
+  else if (p.hd == 128) pf_qkv<128>(p, j0, nt, half, ta, lane);
+  else pf_qkv<64>(p, j0, nt, half, ta, lane);
+}
+
+// Whether `v` holds for any thread of the epilogue warps (a barrier for them).
+__device__ __forceinline__ bool pf_epi_any(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, 1, %2, p;\n"
+      " selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)v), "n"(32 * kPfEpiWarps)
+      : "memory");
+  return r != 0;
+}
+
+template <int EPI, bool SPLIT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
     gemm_pf_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tx,
                    const __grid_constant__ CUtensorMap txlo, const PfParams p) {
   extern __shared__ uint8_t smem_raw[];
+  // full, tempty and done are CTA 0's (its copies in CTA 1 stay unused);
+  // empty and tfull exist in both CTAs and are signalled together
   __shared__ __align__(8) uint64_t full_bar[kPfMaxStages], empty_bar[kPfMaxStages];
   __shared__ __align__(8) uint64_t tfull_bar[2], tempty_bar[2], done_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
-  __shared__ volatile int consumed;
+  __shared__ int issued_of[2];   // CTA 0: stages each CTA loaded
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = ptx::cluster_rank();
+  const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  if (call_aborted(p.status)) return;
+  if (call_aborted(p.status)) return;   // the same in both CTAs: the call's first kernel wrote it
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
-      ptx::mbar_init(&full_bar[s], 1);
+      ptx::mbar_init(&full_bar[s], 2);   // one expect_tx arrival per CTA
       ptx::mbar_init(&empty_bar[s], 1);
     }
     for (int a = 0; a < 2; ++a) {
       ptx::mbar_init(&tfull_bar[a], 1);
-      ptx::mbar_init(&tempty_bar[a], 4);
+      ptx::mbar_init(&tempty_bar[a], 2 * kPfEpiWarps);   // the epilogue warps of both CTAs
     }
     ptx::mbar_init(&done_bar, 1);
     abort_flag = 0;
-    consumed = 0;
     ptx::fence_mbar_init();
     ptx::tma_prefetch_desc(&tw);
     ptx::tma_prefetch_desc(&tx);
     if (SPLIT) ptx::tma_prefetch_desc(&txlo);
   }
-  if (warp == 1) {
-    ptx::tmem_alloc(&tmem_slot, 512);
-    ptx::tmem_relinquish();
-  }
+  if (warp == 1) ptx::tmem_alloc_pair(&tmem_slot, 512);
   ptx::tc_fence_before();
   __syncthreads();
+  ptx::cluster_sync();   // both CTAs' barriers are initialised
   ptx::tc_fence_after();
   const uint32_t tmem_base = tmem_slot;
 
+  int consumed = 0;   // CTA 0, MMA warp: stages waited for
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA
-    if (lane == 0) {
-      const uint32_t bytes = (SPLIT ? 2u : 1u) * kPfABytes + kPfWBytes;
-      int stage = 0;
-      uint32_t ph = 0;
-      int issued = 0;
-      bool ok = true;
-      for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-        int mt, nt;
-        pf_unit(p, u, mt, nt);
-        for (int kb = 0; kb < p.kb_total; ++kb) {
-          if (!ptx::mbar_wait_bounded(&empty_bar[stage], ph ^ 1u, p.wait_ns, &abort_flag)) {
-            ok = false;
-            break;
-          }
-          uint8_t* st = smem + (size_t)stage * p.stage_bytes;
-          ptx::mbar_arrive_expect_tx(&full_bar[stage], bytes);
-          ptx::tma_load_2d(st, &tx, &full_bar[stage], kb * kTileK, mt * 128);
-          if (SPLIT) ptx::tma_load_2d(st + kPfABytes, &txlo, &full_bar[stage], kb * kTileK, mt * 128);
-          pf_load_w<EPI>(st + p.w_off, &tw, &full_bar[stage], p, nt, kb);
-          ++issued;
-          if (++stage == p.stages) {
-            stage = 0;
-            ph ^= 1u;
-          }
+    const uint32_t bytes = (SPLIT ? 3u : 2u) * kPfTileBytes;
+    int stage = 0;
+    uint32_t ph = 0;
+    int issued = 0;
+    bool ok = true;
+    for (int u = pair; u < p.units && ok; u += pairs) {
+      int mt, nt;
+      pf_unit(p, u, mt, nt);
+      const int xrow = mt * 256 + (int)rank * 128, wrow = pf_w_row<EPI>(p, nt, rank);
+      for (int kb = 0; kb < p.kb_total; ++kb) {
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&empty_bar[stage], ph ^ 1u, p.wait_ns, &abort_flag));
+        if (!ok) break;
+        uint8_t* st = smem + (size_t)stage * p.stage_bytes;
+        const uint32_t bar = ptx::dsmem_addr(&full_bar[stage], 0);
+        if (ptx::elect_one()) {
+          ptx::mbar_arrive_expect_tx_cluster(bar, bytes);
+          ptx::tma_load_2d_pair(st, &tx, bar, kb * kTileK, xrow);
+          if (SPLIT) ptx::tma_load_2d_pair(st + kPfTileBytes, &txlo, bar, kb * kTileK, xrow);
+          ptx::tma_load_2d_pair(st + p.w_off, &tw, bar, kb * kTileK, wrow);
+        }
+        __syncwarp();
+        ++issued;
+        if (++stage == p.stages) {
+          stage = 0;
+          ph ^= 1u;
         }
       }
-      // never leave with copies in flight: wait for every issued stage to land
-      for (int it = consumed; it < issued; ++it) {
-        volatile int dummy = 0;
-        ptx::mbar_wait_bounded(&full_bar[it % p.stages], (uint32_t)((it / p.stages) & 1), kWaitLimitNs, &dummy);
-      }
     }
+    if (lane == 0)
+      asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(ptx::dsmem_addr(&issued_of[rank], 0)), "r"(issued)
+                   : "memory");
     __syncwarp();
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA
-    if (lane == 0) {
-      const uint32_t idesc = ptx::idesc_bf16(128u, 256u);
+    // ------------------------------------------------------- MMA (CTA 0 only)
+    if (rank == 0) {
+      const uint32_t idesc = ptx::idesc_bf16(256u, 256u);
       int stage = 0;
       uint32_t ph = 0;
       int acc = 0;
       uint32_t acc_ph = 0;
-      int n_consumed = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-        if (!ptx::mbar_wait_bounded(&tempty_bar[acc], acc_ph ^ 1u, p.wait_ns, &abort_flag)) break;
+      for (int u = pair; u < p.units && ok; u += pairs) {
+        ok = __all_sync(0xffffffffu,
+                        ptx::mbar_wait_bounded<true>(&tempty_bar[acc], acc_ph ^ 1u, p.wait_ns, &abort_flag));
+        if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t d = tmem_base + (uint32_t)acc * 256u;
         for (int kb = 0; kb < p.kb_total; ++kb) {
-          if (!ptx::mbar_wait_bounded(&full_bar[stage], ph, p.wait_ns, &abort_flag)) {
-            ok = false;
-            break;
-          }
-          consumed = ++n_consumed;
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&full_bar[stage], ph, p.wait_ns, &abort_flag));
+          if (!ok) break;
+          ++consumed;
           ptx::tc_fence_after();
           const uint8_t* st = smem + (size_t)stage * p.stage_bytes;
           const uint64_t da = ptx::smem_desc_sw128(st);
-          const uint64_t dl = ptx::smem_desc_sw128(st + kPfABytes);
+          const uint64_t dl = ptx::smem_desc_sw128(st + kPfTileBytes);
           const uint64_t dw = ptx::smem_desc_sw128(st + p.w_off);
+          if (ptx::elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kTileK / 16; ++k) {
-            ptx::mma_bf16(d, da + 2ull * k, dw + 2ull * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-            if (SPLIT) ptx::mma_bf16(d, dl + 2ull * k, dw + 2ull * k, idesc, 1u);
+            for (int k = 0; k < kTileK / 16; ++k) {
+              ptx::mma_bf16_pair(d, da + 2ull * k, dw + 2ull * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+              if (SPLIT) ptx::mma_bf16_pair(d, dl + 2ull * k, dw + 2ull * k, idesc, 1u);
+            }
+            ptx::mma_commit_pair(&empty_bar[stage]);
+            if (kb + 1 == p.kb_total) ptx::mma_commit_pair(&tfull_bar[acc]);
           }
-          ptx::mma_commit(&empty_bar[stage]);
+          __syncwarp();
           if (++stage == p.stages) {
             stage = 0;
             ph ^= 1u;
           }
         }
-        if (!ok) break;
-        ptx::mma_commit(&tfull_bar[acc]);
         acc ^= 1;
         if (acc == 0) acc_ph ^= 1u;
       }
-      // all issued MMAs complete before TMEM is released
-      ptx::mma_commit(&done_bar);
+      // all issued MMAs complete before TMEM is released and CTA 1 may leave
+      if (ptx::elect_one()) ptx::mma_commit_pair(&done_bar);
+      __syncwarp();
       volatile int dummy = 0;
       ptx::mbar_wait_bounded(&done_bar, 0, kWaitLimitNs, &dummy);
     }
     __syncwarp();
   } else {
     // ------------------------------------------------------------- epilogue
-    const int q = warp & 3;   // TMEM lane quarter this warp may access
+    const int q = warp & 3;            // TMEM lane quarter this warp may access
+    const int half = (warp - 2) >> 2;  // columns it takes
     int acc = 0;
     uint32_t acc_ph = 0;
-    for (int u = blockIdx.x; u < p.units; u += gridDim.x) {
+    for (int u = pair; u < p.units; u += pairs) {
       const bool ok = ptx::mbar_wait_bounded(&tfull_bar[acc], acc_ph, p.wait_ns, &abort_flag);
-      if (epi_bar_any(!ok)) break;
+      if (pf_epi_any(!ok)) break;
       ptx::tc_fence_after();
       int mt, nt;
       pf_unit(p, u, mt, nt);
-      const int j = mt * 128 + q * 32 + lane;
+      const int j0 = mt * 256 + (int)rank * 128 + q * 32;
       const uint32_t ta = tmem_base + (uint32_t)acc * 256u + ((uint32_t)(q * 32) << 16);
-      pf_epilogue<EPI, SPLIT>(p, j, nt, ta);
+      pf_epilogue<EPI, SPLIT>(p, j0, nt, half, ta, lane);
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&tempty_bar[acc]);
+      if (lane == 0) ptx::mbar_arrive_cluster(ptx::dsmem_addr(&tempty_bar[acc], 0));
       acc ^= 1;
       if (acc == 0) acc_ph ^= 1u;
     }
@@ -344,9 +461,24 @@ __global__ void __launch_bounds__(kPfThreads, 1)
 
   ptx::tc_fence_before();
   __syncthreads();
+  ptx::cluster_sync();   // neither CTA loads, multiplies or drains any more
   ptx::tc_fence_after();
+  if (rank == 0 && threadIdx.x == 32) {
+    // Never leave with copies in flight: after a wait that ran out, stages may
+    // have been loaded that no MMA waited for.  A CTA that did not get to load
+    // its part of such a stage is arrived for here.
+    for (int it = consumed; it < max(issued_of[0], issued_of[1]); ++it) {
+      uint64_t* bar = &full_bar[it % p.stages];
+      if (it >= issued_of[0]) ptx::mbar_arrive(bar);
+      if (it >= issued_of[1]) ptx::mbar_arrive(bar);
+      volatile int dummy = 0;
+      ptx::mbar_wait_bounded(bar, (uint32_t)((it / p.stages) & 1), kWaitLimitNs, &dummy);
+    }
+  }
   if (threadIdx.x == 0 && abort_flag) atomicOr(p.status, BUDDY_DEV_TIMEOUT);
-  if (warp == 1) ptx::tmem_dealloc(tmem_base, 512);
+  __syncwarp();
+  if (warp == 1) ptx::tmem_dealloc_pair(tmem_base, 512);
+  ptx::cluster_sync();   // CTA 1's copies have landed before it leaves
 }
 
 // ---------------------------------------------------------------------------
@@ -355,7 +487,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
 int gemm_pf_prepare(Ctx& c) {
   const int limit = 227 * 1024 - 2 * 1024;
   for (int v = 0; v < 2; ++v) {
-    const uint32_t sb = (v ? 2u : 1u) * kPfABytes + kPfWBytes;
+    const uint32_t sb = (v ? 3u : 2u) * kPfTileBytes;
     c.pf_stages[v] = std::min(kPfMaxStages, (int)((limit - 1024) / sb));
     c.pf_smem[v] = (int)(c.pf_stages[v] * sb) + 1024;
   }
@@ -382,13 +514,13 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
   p.K = K;
   p.m = m;
   p.n_tiles = tiles;
-  p.m_tiles = (m + 127) / 128;
+  p.m_tiles = (m + 255) / 256;
   p.kb_total = (K + kTileK - 1) / kTileK;
   p.units = p.n_tiles * p.m_tiles;
   const int v = split ? 1 : 0;
   p.stages = c.pf_stages[v];
-  p.stage_bytes = (split ? 2u : 1u) * kPfABytes + kPfWBytes;
-  p.w_off = (split ? 2u : 1u) * kPfABytes;
+  p.stage_bytes = (split ? 3u : 2u) * kPfTileBytes;
+  p.w_off = (split ? 2u : 1u) * kPfTileBytes;
   p.rows = e.rows;
   p.resid_src = e.resid_src;
   p.resid_dst = e.resid_dst;
@@ -411,10 +543,10 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
   p.hd = c.hd;
   p.status = c.status;
   p.wait_ns = c.wait_ns;
-  const CUtensorMap& tw = c.tmaps_host[(size_t)layer * 4 + which];
+  const CUtensorMap& tw = c.pf_wmaps[(size_t)layer * 4 + which];
   const CUtensorMap& tx = c.pf_tmaps[xi];
   const CUtensorMap& txlo = c.pf_tmaps[3 + xi];
-  const int grid = std::min(p.units, c.num_sms);
+  const int grid = 2 * std::min(p.units, c.num_sms / 2);
   const size_t smem = c.pf_smem[v];
   if (split) {
     switch (epi) {

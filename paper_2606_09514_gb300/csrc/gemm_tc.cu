@@ -490,7 +490,15 @@ int gemm_tc_prepare(Ctx& c) {
   // them over all SMs.
   c.tc_defer = c.maxB > kTcDeferRows;
   if (c.pf_max > 0) {
-    // prefill activations: 128-row boxes (one M-tile per copy)
+    // prefill weights and activations: 128-row boxes (one CTA's part of a tile)
+    c.pf_wmaps.assign((size_t)c.L * 4, CUtensorMap{});
+    for (int l = 0; l < c.L; ++l) {
+      const buddy_layer_weights& w = c.layers[l];
+      CUtensorMap* M = &c.pf_wmaps[(size_t)l * 4];
+      if (!make_map(&M[0], w.w_qkv, c.qkvN, c.d, 128) || !make_map(&M[1], w.w_o, c.d, c.qd, 128) ||
+          !make_map(&M[2], w.w_gate_up, 2ull * c.F, c.d, 128) || !make_map(&M[3], w.w_down, c.d, c.F, 128))
+        return BUDDY_ERR_ARG;
+    }
     if (!make_map(&c.pf_tmaps[0], c.pf_xn, c.pf_max, c.d, 128) ||
         !make_map(&c.pf_tmaps[1], c.pf_attn, c.pf_max, c.qd, 128) ||
         !make_map(&c.pf_tmaps[2], c.pf_act, c.pf_max, c.F, 128) ||

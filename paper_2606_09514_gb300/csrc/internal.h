@@ -245,6 +245,7 @@ struct Ctx {
   int32_t* pf_tok_end = nullptr;  // [maxB] one past the last token row of each prompt
   int32_t* pf_cnt = nullptr;      // [maxB] positions the pooled context covers
   float* pf_hlast = nullptr;      // [maxB, d] last prompt token's hidden state
+  std::vector<CUtensorMap> pf_wmaps;   // per layer 4 weight maps, 128-row boxes
   CUtensorMap pf_tmaps[6];        // pf_xn, pf_attn, pf_act, then their remainder terms
   int pf_stages[2] = {1, 1}, pf_smem[2] = {0, 0};
 
