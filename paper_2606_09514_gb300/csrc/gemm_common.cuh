@@ -40,7 +40,12 @@
 
 namespace buddy {
 
+// TMA warp, MMA warp and four epilogue warps; eight with a deferred fixup (two
+// per TMEM lane quarter, half of the columns each): with two M-tiles, whose one
+// accumulator the next unit waits for, draining 256 x 256 values and their
+// SwiGLU took four warps 15 us of the 70 us of a Qwen2.5-7B gate/up GEMM.
 constexpr int kTcThreads = 192;
+constexpr int kTcDeferThreads = 320;
 constexpr int kTcMaxStages = 16;
 constexpr int kTileK = 64;                       // K columns per stage (128 B of bf16)
 constexpr uint32_t kXTileMax = 128 * 128;        // bytes one M-tile operand spans
@@ -60,7 +65,6 @@ struct TcParams {
   const int32_t* rows;
   const int32_t* count;
   int n;
-  float* out_f32;
   bf16* out_act;
   bf16* out_act_lo;       // SPLIT: bf16 remainder of the SwiGLU output
   const float* resid_src;
@@ -95,20 +99,18 @@ struct TcParams {
   uint32_t panel_bytes;   // bytes of one panel (hi, then lo for SPLIT)
   int panel_kb;           // K blocks one panel holds (hi part)
   uint32_t gstage_off;    // byte offset of the first unit's RMSNorm gains (fp32, panel_kb x 64)
-  // Deferred fixup: units only stage their partials; a second kernel
-  // (gemm_fix_kernel) sums the splits and applies the epilogue on every SM.
-  int defer;
   uint64_t wait_ns;       // limit of each pipeline wait (the drain waits keep kWaitLimitNs)
 };
 
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-__device__ __forceinline__ bool epi_bar_any(bool v) {
+// Whether `v` holds for any of the `n` epilogue threads (a barrier for them).
+__device__ __forceinline__ bool epi_bar_any(bool v, uint32_t n) {
   uint32_t r;
   asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, 1, 128, p;\n"
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, 1, %2, p;\n"
       " selp.u32 %0, 1, 0, q;\n}\n"
       : "=r"(r)
-      : "r"((uint32_t)v)
+      : "r"((uint32_t)v), "r"(n)
       : "memory");
   return r != 0;
 }
@@ -137,16 +139,23 @@ __device__ __forceinline__ uint32_t tc_x_bytes(int m, bool split) {
   return (split ? 2u : 1u) * (uint32_t)round16(m) * 128u;
 }
 
-// Activation rows 0..round16(m)-1 at K block kb, 16 rows per copy.
+// Activation rows 0..round16(m)-1 at K block kb in as few copies as the box
+// sizes allow (128, 64, 32 and 16 rows): issuing a copy takes its thread about
+// 85 cycles, so that at 256 rows sixteen 16-row copies took longer than the
+// stage's MMAs (1540 cycles against 1024 a stage; 220 with two 128-row ones).
 template <bool SPLIT>
-__device__ __forceinline__ void tc_load_x(uint8_t* st, const CUtensorMap* tx, const CUtensorMap* txlo, uint64_t* bar,
+__device__ __forceinline__ void tc_load_x(uint8_t* st, const XMaps& tx, const XMaps& txlo, uint64_t* bar,
                                           const TcParams& p, int m, int kb) {
   uint8_t* x0 = st;
   uint8_t* l0 = x0 + p.mt * p.xr;
-  for (int r0 = 0; r0 < m; r0 += 16) {
+  const int mr = round16(m);
+  for (int r0 = 0; r0 < mr;) {
+    const int left = mr - r0;   // r0 is a multiple of the box below: a box never crosses an M-tile
+    const int b = left >= 128 ? 3 : (left >= 64 ? 2 : (left >= 32 ? 1 : 0));
     const uint32_t off = (uint32_t)(r0 >> 7) * p.xr + (uint32_t)(r0 & 127) * 128u;
-    ptx::tma_load_2d(x0 + off, tx, bar, kb * kTileK, r0);
-    if (SPLIT) ptx::tma_load_2d(l0 + off, txlo, bar, kb * kTileK, r0);
+    ptx::tma_load_2d(x0 + off, &tx.box[b], bar, kb * kTileK, r0);
+    if (SPLIT) ptx::tma_load_2d(l0 + off, &txlo.box[b], bar, kb * kTileK, r0);
+    r0 += 16 << b;
   }
 }
 
@@ -431,18 +440,11 @@ __device__ __forceinline__ void tc_apply4(const TcParams& p, int tile, int j, in
     }
   } else {
     const int n0 = tile * p.bw + c;
-    float* dst;
     float w[4];
-    if (EPI == EPI_STORE_F32) {
-      dst = p.out_f32 + (size_t)j * p.N + n0;
+    const int seq = p.rows ? p.rows[j] : j;
+    float* dst = p.resid_dst + (size_t)seq * p.N + n0;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) w[i] = v[i];
-    } else {
-      const int seq = p.rows ? p.rows[j] : j;
-      dst = p.resid_dst + (size_t)seq * p.N + n0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) w[i] = rs[i] + v[i];
-    }
+    for (int i = 0; i < 4; ++i) w[i] = rs[i] + v[i];
     if (n0 + 4 <= p.N) {   // one 16-byte store (N % 4 == 0, c % 4 == 0)
       *reinterpret_cast<float4*>(dst) = make_float4(w[0], w[1], w[2], w[3]);
     } else {
@@ -508,23 +510,26 @@ __device__ __forceinline__ void tc_fix_item(const TcParams& p, int tile, int j, 
 }
 
 // ---------------------------------------------------------------------------
-// Epilogue of one unit by the four epilogue warps (128 threads).  Warp w reads
-// TMEM lanes 32*(w%4).. (rows of each M-tile) and writes the unit's
+// Epilogue of one unit by the epilogue warps (four, or eight with DEFER, then
+// two per lane quarter with half of the columns each).  Warp w reads TMEM lanes
+// 32*(w%4).. (rows of each M-tile) and writes the unit's
 // accumulator rows j < m to its workspace slot; the accumulator is released
 // (tempty) right after.  The CTA that completes a tile (the last of its K
 // splits, or the only one) then applies the epilogue with all 128 threads over
 // (row, 4-column group) items, summing the splits' slots in split order
-// (deterministic).  With p.defer every unit stops after staging its slot,
+// (deterministic).  With DEFER every unit stops after staging its slot,
 // except a SwiGLU GEMM with a single K split, which applies its epilogue
 // directly.
 // ---------------------------------------------------------------------------
-template <int EPI, bool SPLIT>
+template <int EPI, bool SPLIT, bool DEFER>
 __device__ __forceinline__ void tc_epilogue_unit(const TcParams& p, int u, int m, uint32_t tacc, uint64_t* tempty,
                                                  int* last_flag) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = warp & 3;   // TMEM lane quarter this warp may access
+  constexpr int parts = DEFER ? 2 : 1;
+  const int part = DEFER ? (warp - 2) >> 2 : 0;   // this warp's share of the columns
   const int tile = u % p.n_tiles;
-  if (EPI == EPI_SWIGLU && p.defer && p.splits == 1) {
+  if (EPI == EPI_SWIGLU && DEFER && p.splits == 1) {
     // One K split (larger batches): SwiGLU straight from the accumulator, gate
     // column c and up column c + bw/2 of the same row, with no workspace and no
     // fixup kernel (the same arithmetic as tc_apply4 on a single partial).
@@ -533,7 +538,7 @@ __device__ __forceinline__ void tc_epilogue_unit(const TcParams& p, int u, int m
       if (t * 128 + q * 32 >= m) continue;   // warp-uniform
       const int j = t * 128 + q * 32 + lane;
       const uint32_t ta = tacc + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * p.bw);
-      for (int c0 = 0; c0 < h; c0 += 16) {
+      for (int c0 = part * h / parts; c0 < (part + 1) * h / parts; c0 += 16) {
         float g[16], up[16];
         ptx::tmem_ld16(ta + c0, g);
         ptx::tmem_ld16(ta + h + c0, up);
@@ -577,7 +582,7 @@ __device__ __forceinline__ void tc_epilogue_unit(const TcParams& p, int u, int m
     if (t * 128 + q * 32 >= m) continue;   // warp-uniform
     const int j = t * 128 + q * 32 + lane;
     const uint32_t ta = tacc + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * p.bw);
-    for (int c0 = 0; c0 < p.bw; c0 += 64) {
+    for (int c0 = part * p.bw / parts; c0 < (part + 1) * p.bw / parts; c0 += 64) {
       float v[64];
       ptx::tmem_ld64(ta + c0, v);
       if (j < m) {
@@ -589,7 +594,7 @@ __device__ __forceinline__ void tc_epilogue_unit(const TcParams& p, int u, int m
   }
   ptx::tc_fence_before();
   if (lane == 0) ptx::mbar_arrive(tempty);
-  if (p.defer) return;   // gemm_fix_kernel sums the splits
+  if (DEFER) return;   // gemm_fix_kernel sums the splits
   epi_bar();
   const int et = threadIdx.x & 127;
   if (et == 0) {

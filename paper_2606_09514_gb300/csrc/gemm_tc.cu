@@ -6,13 +6,13 @@
 // tile geometry, the ring stage layout and the epilogues are described in
 // gemm_common.cuh.  Persistent CTAs (one per SM) walk work units (weight tile,
 // K split); warp 0 issues TMA loads into a ring of stages, warp 1 issues the
-// tcgen05 MMAs (accumulating fp32 in TMEM), warps 2-5 drain TMEM and run the
-// epilogue.  A tile split over K is finished by the last CTA to arrive, which
+// tcgen05 MMAs (accumulating fp32 in TMEM), the other warps drain TMEM and run
+// the epilogue.  A tile split over K is finished by the last CTA to arrive, which
 // sums the partials in split order (deterministic).
 //
-// Epilogues: fp32 store; residual add into the (row-gathered) hidden state;
-// SwiGLU (a tile holds 128 gate rows and the matching 128 up rows); QKV
-// finalisation (bias, RoPE, q, K/V cache append, pooled first-layer V).
+// Epilogues: residual add into the (row-gathered) hidden state; SwiGLU (a tile
+// holds 128 gate rows and the matching 128 up rows); QKV finalisation (bias,
+// RoPE, q, K/V cache append, pooled first-layer V).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -30,10 +30,14 @@ namespace buddy {
 // SPLIT: the activations are given as two bf16 terms hi + lo (hi = bf16(x),
 // lo = bf16(x - hi)); every K step issues one MMA per term into the same
 // accumulator, so the product carries ~16 mantissa bits of the activations.
-template <int EPI, bool SPLIT>
-__global__ void __launch_bounds__(kTcThreads, 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tx,
-                   const __grid_constant__ CUtensorMap txlo, const TcParams p) {
+// DEFER (more than kTcDeferRows rows): the units only stage their partials, a
+// second kernel (gemm_fix_kernel) sums the splits and applies the epilogue on
+// every SM; without it (up to that many rows) the kernel can run in panel mode
+// and the last split of a tile applies the epilogue.
+template <int EPI, bool SPLIT, bool DEFER>
+__global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
+    gemm_tc_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ XMaps tx,
+                   const __grid_constant__ XMaps txlo, const TcParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[kTcMaxStages], empty_bar[kTcMaxStages];
   __shared__ __align__(8) uint64_t tfull_bar[2], tempty_bar[2], done_bar, pfull_bar[2];
@@ -73,7 +77,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     for (int a = 0; a < 2; ++a) {
       ptx::mbar_init(&tfull_bar[a], 1);
-      ptx::mbar_init(&tempty_bar[a], 4);
+      ptx::mbar_init(&tempty_bar[a], DEFER ? 8 : 4);
     }
     ptx::mbar_init(&done_bar, 1);
     ptx::mbar_init(&pfull_bar[0], 1);
@@ -82,8 +86,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     consumed = 0;
     ptx::fence_mbar_init();
     ptx::tma_prefetch_desc(&tw);
-    ptx::tma_prefetch_desc(&tx);
-    if (SPLIT) ptx::tma_prefetch_desc(&txlo);
+    if (DEFER || !p.nsrc)
+      for (int b = 0; b < 4; ++b) {
+        ptx::tma_prefetch_desc(&tx.box[b]);
+        if (SPLIT) ptx::tma_prefetch_desc(&txlo.box[b]);
+      }
   }
   if (warp == 1) {
     ptx::tmem_alloc(&tmem_slot, p.tmem_cols);
@@ -110,7 +117,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
   }
-  const bool panel = p.nsrc != nullptr;
+  const bool panel = !DEFER && p.nsrc != nullptr;
   const bool first_pass = panel && p.K <= kPanelFirstMaxK;
   if (first_pass && warp >= 2 && blockIdx.x < p.units) {
     // Before the wait: the RMSNorm gains of the first unit's K range (weights,
@@ -171,7 +178,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             ptx::mbar_arrive_expect_tx(&full_bar[stage], w_bytes + x_bytes);
             tc_load_w<EPI>(st, &tw, &full_bar[stage], p, tile, kb, pol);
           }
-          if (!panel) tc_load_x<SPLIT>(st, &tx, &txlo, &full_bar[stage], p, m, kb);
+          if (!panel) tc_load_x<SPLIT>(st, tx, txlo, &full_bar[stage], p, m, kb);
           ++issued;
           if (++stage == p.stages) {
             stage = 0;
@@ -273,9 +280,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         if (et == 0) ptx::mbar_arrive(&pfull_bar[(ui + 1) & 1]);
       }
       const bool ok = ptx::mbar_wait_bounded(&tfull_bar[acc], acc_ph, p.wait_ns, &abort_flag);
-      if (epi_bar_any(!ok)) break;
+      if (epi_bar_any(!ok, DEFER ? 256 : 128)) break;
       ptx::tc_fence_after();
-      tc_epilogue_unit<EPI, SPLIT>(p, u, m, tmem_base + (uint32_t)acc * acc_cols, &tempty_bar[acc], &last_flag);
+      tc_epilogue_unit<EPI, SPLIT, DEFER>(p, u, m, tmem_base + (uint32_t)acc * acc_cols, &tempty_bar[acc], &last_flag);
       if (p.acc_bufs == 2) {
         acc ^= 1;
         if (acc == 0) acc_ph ^= 1u;
@@ -436,12 +443,12 @@ int gemm_tc_prepare(Ctx& c) {
     max_tiles = std::max(max_tiles, tiles);
   }
   // tensor maps: activations (fixed scratch) and per-layer weights
-  c.tmaps_host.assign((size_t)c.L * 4 + 6, CUtensorMap{});
-  CUtensorMap* X = &c.tmaps_host[(size_t)c.L * 4];
-  if (!make_map(&X[0], c.xn, c.maxB, c.d, 16) || !make_map(&X[1], c.attn_out, c.maxB, c.qd, 16) ||
-      !make_map(&X[2], c.act, c.maxB, c.F, 16) || !make_map(&X[3], c.xn_lo, c.maxB, c.d, 16) ||
-      !make_map(&X[4], c.attn_lo, c.maxB, c.qd, 16) || !make_map(&X[5], c.act_lo, c.maxB, c.F, 16))
-    return BUDDY_ERR_CUDA;
+  c.tmaps_host.assign((size_t)c.L * 4, CUtensorMap{});
+  const struct { const void* p; int k; } xs[6] = {{c.xn, c.d},    {c.attn_out, c.qd}, {c.act, c.F},
+                                                  {c.xn_lo, c.d}, {c.attn_lo, c.qd},  {c.act_lo, c.F}};
+  for (int i = 0; i < 6; ++i)
+    for (int b = 0; b < 4; ++b)
+      if (!make_map(&c.tc_xmaps[i].box[b], xs[i].p, c.maxB, xs[i].k, 16u << b)) return BUDDY_ERR_CUDA;
   for (int l = 0; l < c.L; ++l) {
     const buddy_layer_weights& w = c.layers[l];
     CUtensorMap* M = &c.tmaps_host[(size_t)l * 4];
@@ -512,15 +519,22 @@ int gemm_tc_prepare(Ctx& c) {
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
   const int qs0 = std::max(c.tc_smem[0], c.tc_panel ? c.tc_psmem[0] : 0);
   const int qs1 = std::max(c.tc_smem[1], c.tc_panel ? c.tc_psmem[1] : 0);
-  if (cudaFuncSetAttribute(gemm_tc_kernel<EPI_STORE_F32, false>, A, c.tc_smem[0]) ||
-      cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false>, A, c.tc_smem[0]) ||
-      cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false>, A, qs0) ||
-      cudaFuncSetAttribute(gemm_tc_kernel<EPI_STORE_F32, true>, A, c.tc_smem[1]) ||
-      cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true>, A, c.tc_smem[1]) ||
-      cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true>, A, qs1) ||
-      cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false>, A, qs0) ||
-      cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, true>, A, qs1))
-    return BUDDY_ERR_CUDA;
+  bool bad = false;
+  if (c.tc_defer)
+    bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, true>, A, c.tc_smem[0]) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, true>, A, c.tc_smem[0]) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, true>, A, c.tc_smem[0]) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, true, true>, A, c.tc_smem[1]) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true, true>, A, c.tc_smem[1]) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true, true>, A, c.tc_smem[1]);
+  else
+    bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, false>, A, qs0) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, false>, A, c.tc_smem[0]) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, false>, A, qs0) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, true, false>, A, qs1) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true, false>, A, c.tc_smem[1]) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true, false>, A, qs1);
+  if (bad) return BUDDY_ERR_CUDA;
   return BUDDY_OK;
 }
 
@@ -550,7 +564,6 @@ static TcParams tc_params(const Ctx& c, const GemmArgs& a, size_t* smem_out) {
   p.rows = a.sel.rows;
   p.count = a.sel.count;
   p.n = a.sel.n;
-  p.out_f32 = a.out_f32;
   p.out_act = (bf16*)a.out_act;
   p.out_act_lo = (bf16*)a.out_act_lo;
   p.resid_src = a.resid_src;
@@ -584,7 +597,6 @@ static TcParams tc_params(const Ctx& c, const GemmArgs& a, size_t* smem_out) {
     smem = c.tc_psmem[v];
   }
   p.count_late = a.count_late ? 1 : 0;
-  p.defer = c.tc_defer ? 1 : 0;
   p.wait_ns = c.wait_ns;
   p.nq = c.nq;
   p.nkv = c.nkv;
@@ -593,67 +605,38 @@ static TcParams tc_params(const Ctx& c, const GemmArgs& a, size_t* smem_out) {
   return p;
 }
 
-void launch_gemm_tc(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s) {
-  const int which = a.which;
+template <int EPI, bool SPLIT>
+static void launch_tc(const Ctx& c, const GemmArgs& a, cudaStream_t s) {
   size_t smem = 0;
   const TcParams p = tc_params(c, a, &smem);
-  const CUtensorMap& tw = c.tmaps_host[(size_t)a.layer * 4 + which];
-  const int xi = which == 0 || which == 2 ? 0 : (which == 1 ? 1 : 2);
-  const CUtensorMap& tx = c.tmaps_host[(size_t)c.L * 4 + xi];
-  const CUtensorMap& txlo = c.tmaps_host[(size_t)c.L * 4 + 3 + xi];
+  const CUtensorMap& tw = c.tmaps_host[(size_t)a.layer * 4 + a.which];
+  const int xi = a.which == 0 || a.which == 2 ? 0 : (a.which == 1 ? 1 : 2);
+  const XMaps& tx = c.tc_xmaps[xi];
+  const XMaps& txlo = c.tc_xmaps[3 + xi];
   const int grid = std::min(p.units, c.num_sms);
+  if (c.tc_defer)
+    launch_k(gemm_tc_kernel<EPI, SPLIT, true>, grid, kTcDeferThreads, smem, s, c.pdl, tw, tx, txlo, p);
+  else
+    launch_k(gemm_tc_kernel<EPI, SPLIT, false>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
+}
 
-  if (a.split) {
-    switch (epi) {
-      case EPI_QKV:
-        launch_k(gemm_tc_kernel<EPI_QKV, true>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-        break;
-      case EPI_STORE_F32:
-        launch_k(gemm_tc_kernel<EPI_STORE_F32, true>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-        break;
-      case EPI_RESID:
-        launch_k(gemm_tc_kernel<EPI_RESID, true>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-        break;
-      default:
-        launch_k(gemm_tc_kernel<EPI_SWIGLU, true>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-    }
-  } else {
-    switch (epi) {
-      case EPI_QKV:
-        launch_k(gemm_tc_kernel<EPI_QKV, false>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-        break;
-      case EPI_STORE_F32:
-        launch_k(gemm_tc_kernel<EPI_STORE_F32, false>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-        break;
-      case EPI_RESID:
-        launch_k(gemm_tc_kernel<EPI_RESID, false>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-        break;
-      default:
-        launch_k(gemm_tc_kernel<EPI_SWIGLU, false>, grid, kTcThreads, smem, s, c.pdl, tw, tx, txlo, p);
-    }
-  }
+void launch_gemm_tc(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s) {
+  if (epi == EPI_QKV) a.split ? launch_tc<EPI_QKV, true>(c, a, s) : launch_tc<EPI_QKV, false>(c, a, s);
+  else if (epi == EPI_RESID) a.split ? launch_tc<EPI_RESID, true>(c, a, s) : launch_tc<EPI_RESID, false>(c, a, s);
+  else a.split ? launch_tc<EPI_SWIGLU, true>(c, a, s) : launch_tc<EPI_SWIGLU, false>(c, a, s);
+}
+
+template <int EPI, bool SPLIT>
+static void launch_fix(const Ctx& c, const GemmArgs& a, cudaStream_t s) {
+  size_t smem = 0;
+  const TcParams p = tc_params(c, a, &smem);
+  launch_k(gemm_fix_kernel<EPI, SPLIT>, c.num_sms * (2048 / kTcFixThreads), kTcFixThreads, 0, s, c.pdl, p);
 }
 
 void launch_gemm_fix(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s) {
-  size_t smem = 0;
-  const TcParams p = tc_params(c, a, &smem);
-  const int fgrid = c.num_sms * (2048 / kTcFixThreads);
-  if (a.split) {
-    switch (epi) {
-      case EPI_QKV: launch_k(gemm_fix_kernel<EPI_QKV, true>, fgrid, kTcFixThreads, 0, s, c.pdl, p); break;
-      case EPI_STORE_F32: launch_k(gemm_fix_kernel<EPI_STORE_F32, true>, fgrid, kTcFixThreads, 0, s, c.pdl, p); break;
-      case EPI_RESID: launch_k(gemm_fix_kernel<EPI_RESID, true>, fgrid, kTcFixThreads, 0, s, c.pdl, p); break;
-      default: launch_k(gemm_fix_kernel<EPI_SWIGLU, true>, fgrid, kTcFixThreads, 0, s, c.pdl, p);
-    }
-  } else {
-    switch (epi) {
-      case EPI_QKV: launch_k(gemm_fix_kernel<EPI_QKV, false>, fgrid, kTcFixThreads, 0, s, c.pdl, p); break;
-      case EPI_STORE_F32: launch_k(gemm_fix_kernel<EPI_STORE_F32, false>, fgrid, kTcFixThreads, 0, s, c.pdl, p); break;
-      case EPI_RESID: launch_k(gemm_fix_kernel<EPI_RESID, false>, fgrid, kTcFixThreads, 0, s, c.pdl, p); break;
-      default: launch_k(gemm_fix_kernel<EPI_SWIGLU, false>, fgrid, kTcFixThreads, 0, s, c.pdl, p);
-    }
-  }
+  if (epi == EPI_QKV) a.split ? launch_fix<EPI_QKV, true>(c, a, s) : launch_fix<EPI_QKV, false>(c, a, s);
+  else if (epi == EPI_RESID) a.split ? launch_fix<EPI_RESID, true>(c, a, s) : launch_fix<EPI_RESID, false>(c, a, s);
+  else a.split ? launch_fix<EPI_SWIGLU, true>(c, a, s) : launch_fix<EPI_SWIGLU, false>(c, a, s);
 }
-
 
 }  // namespace buddy

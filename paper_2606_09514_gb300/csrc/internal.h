@@ -70,6 +70,11 @@ struct GemmArgs {
 
 struct Ctx;
 
+// Tensor maps of one activation matrix with boxes of 16, 32, 64 and 128 rows.
+struct XMaps {
+  CUtensorMap box[4];
+};
+
 // Epilogue pointers of a prefill GEMM (gemm_pf.cu); unused ones stay null.
 struct PfEpi {
   const int32_t* rows;      // compact row -> token row (nullptr: identity)
@@ -209,7 +214,8 @@ struct Ctx {
 
   // tcgen05 GEMM resources
   bool use_tc = false;
-  std::vector<CUtensorMap> tmaps_host;    // per layer 4 weight maps, then 3 activation maps
+  std::vector<CUtensorMap> tmaps_host;    // per layer 4 weight maps
+  XMaps tc_xmaps[6];                      // xn, attn_out, act, then their remainder terms
   int tc_bw = 256, tc_mt = 1, tc_rows_max = 16, tc_acc_bufs = 2;   // tile geometry (gemm_common.cuh)
   int tc_stages[2] = {1, 1}, tc_smem[2] = {0, 0};                   // [plain, split activations]
   uint32_t tc_stage_bytes[2] = {0, 0}, tc_w_off[2] = {0, 0}, tc_xr = 0, tc_tmem_cols = 512;
