@@ -3,41 +3,63 @@
 // c0 + t of the block's cache (c0 = the positions it held before the
 // prompt), attends to cache positions 0 .. c0 + t.
 //
-// A CTA takes one work item: 64 query tokens of one sequence and one query
-// head (4 warps x 16 tokens).  It walks the key/value positions of the KV
-// head in tiles of 64, copied with 16-byte cp.async into two shared-memory
-// buffers (one tile in flight while the other is used; rows padded by 16
-// bytes so that ldmatrix is conflict-free).  Per tile and warp:
-//   S = Q K^T      mma.sync m16n8k16, the 16 tokens as A (from registers),
-//                  K rows through ldmatrix as B; 8 position tiles x HD/16
-//                  k-steps;
-//   online softmax per token in base 2 (queries pre-scaled by
-//                  log2(e) / sqrt(d_h)), causal and range masks;
-//   O += P V       the probabilities re-packed from the S fragments as A,
-//                  V through ldmatrix.trans as B; HD/8 channel tiles x 4
-//                  k-steps.
-// With SPLIT (the blocks that feed the router) the queries and the
-// probabilities are each given as bf16 hi + lo and every product is issued
-// for both terms.
+// The query heads of a KV head share its keys and values, so the rows of a tile
+// are (token, head of the group) pairs: row R of a (sequence, KV head) is token
+// R / G, head R % G.  A work item is NQ tiles of 128 such rows that walk the
+// same key/value tiles of 128 positions: two tiles, or one where the queries
+// and probabilities are bf16 hi + lo pairs (SPLIT, the blocks that feed the
+// router), whose queries take twice the shared memory.
+//
+// On the 5th-generation tensor cores:
+//   S = Q K^T   tcgen05.mma M = 128, N = 128, K = HD: queries (pre-scaled by
+//               log2(e) / sqrt(d_h)) and keys from shared memory, S in TMEM;
+//   softmax     four warps per tile, a row per thread: running reference m,
+//               p = 2^(s - m) written back as bf16 over S's columns.  m follows
+//               the row's maximum only when that rises by more than 8 (p stays
+//               below 2^8), so that the output is rescaled a few times per row
+//               instead of once per key tile; the final division makes the
+//               choice of m immaterial;
+//   O += P V    M = 128, N = HD, K = 128: P from TMEM, V from shared memory
+//               (MN-major), O in TMEM.
+// With SPLIT every product is issued for both terms.
+//
+// Warps: 4 NQ softmax warps, one MMA warp, two copy warps (16-byte cp.async
+// into the 128-byte-swizzled layout, two buffers each for K and V; rows past
+// the range are zero).  With two tiles the MMAs of one overlap the softmax of
+// the other; with one tile S has two buffers and the next S overlaps the
+// softmax of this one.  Every wait is bounded.
+//
+// Bound by the MMA issue (about 100 cycles for the 64 cycles of an N = 128 MMA)
+// and the softmax chain.  Two prompts of 2,999 and 5,000 tokens, 28 heads of 128
+// over 4 KV heads: 0.30 ms (0.9 PFLOP/s of the visible positions), 0.57 ms with
+// SPLIT, against 1.16 and 1.55 ms on mma.sync with 64-row tiles of one head.
 #include <cuda_runtime.h>
 
 #include "attn_tc.cuh"
 #include "common.cuh"
+#include "gemm_common.cuh"
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace buddy {
 
-constexpr int kPfaThreads = 128;
-constexpr int kPfaRows = 64;    // query tokens per work item
-constexpr int kPfaKeys = 64;    // key positions per tile
+constexpr int kPfaRows = 128;    // rows of a tile (MMA M)
+constexpr int kPfaKeys = 128;    // positions of a key/value tile
+constexpr int kPfaLoadThreads = 64;
+constexpr uint32_t kPfaRegion = 128u * 128u;   // 128 rows x 64 channels of bf16
 
-template <int HD>
-__host__ __device__ constexpr size_t attn_pf_smem() {
-  return (size_t)2 * 2 * kPfaKeys * (HD + 8) * sizeof(bf16);   // 2 buffers x (K, V)
+template <bool SPLIT>
+__host__ __device__ constexpr int pfa_tiles() { return SPLIT ? 1 : 2; }
+template <bool SPLIT>
+__host__ __device__ constexpr int pfa_threads() { return 128 * pfa_tiles<SPLIT>() + 32 + kPfaLoadThreads; }
+template <int HD, bool SPLIT>
+__host__ __device__ constexpr size_t pfa_smem() {
+  // queries (hi, and lo with SPLIT), two K and two V buffers, alignment slack
+  return (size_t)(HD / 64) * kPfaRegion * (pfa_tiles<SPLIT>() * (SPLIT ? 2 : 1) + 4) + 1024;
 }
 
 struct PfaArgs {
-  const int4* items;        // (sequence, query head, first compact row, first prompt token)
+  const int4* items;        // (sequence, KV head, first compact row of the sequence, first tile row)
   const int32_t* n_tok;     // sequence -> prompt tokens
   const int32_t* base;      // sequence -> positions the layer's cache held before the prompt
   const float* q;           // [m, nq * hd] compact rows
@@ -48,234 +70,363 @@ struct PfaArgs {
   bf16* out;                // [m, nq * hd]
   bf16* out_lo;
   int nq, nkv;
-  const int32_t* status;
+  int32_t* status;
+  uint64_t wait_ns;
 };
 
+// 16 bytes from global to shared memory, or zeros.
+__device__ __forceinline__ void cp_async16_or_zero(uint32_t dst, const void* src, bool real) {
+  const uint32_t n = real ? 16u : 0u;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+
+// Byte offset of 16-byte piece c of row r in a tile of 64-channel regions
+// (128-byte rows, 128-byte swizzle).
+__device__ __forceinline__ uint32_t pfa_piece(int r, int c) {
+  return (uint32_t)(c >> 3) * kPfaRegion + (uint32_t)r * 128u + (uint32_t)(((c ^ r) & 7) << 4);
+}
+
 template <int HD, bool SPLIT>
-__global__ void __launch_bounds__(kPfaThreads) attn_pf_kernel(PfaArgs A) {
-  extern __shared__ __align__(16) uint8_t smraw[];
-  constexpr int KROW = HD + 8;
-  constexpr int KSTEPS = HD / 16;
-  constexpr int NT = kPfaKeys / 8;    // position tiles of the logits
-  constexpr int DT = HD / 8;          // channel tiles of the output
-  constexpr int V16 = HD / 8;         // 16-byte pieces per row
+__global__ void __launch_bounds__(pfa_threads<SPLIT>(), 1) attn_pf_kernel(const PfaArgs A) {
+  extern __shared__ uint8_t smem_raw[];
+  constexpr int NQ = pfa_tiles<SPLIT>();
+  constexpr int V16 = HD / 8;                           // 16-byte pieces per row
+  constexpr uint32_t TILE = (HD / 64) * kPfaRegion;     // bytes of a 128-row tile
+  // TMEM columns: S slots at 0 and 128 (P over their first half); O of tile q at
+  // 256 + 128 q; with SPLIT (one tile) P's remainders of the two slots at 384
+  constexpr uint32_t kO = 256, kPLo = 384;
+  __shared__ __align__(8) uint64_t q_ready, k_full[2], k_empty[2], v_full[2], v_empty[2];
+  __shared__ __align__(8) uint64_t s_full[2], p_ready[2], pv_done, o_full[2], drained;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int abort_flag;
   if (call_aborted(A.status)) return;
+
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sQ = smem;                                   // [tile][hi, lo]
+  uint8_t* sK = smem + NQ * (SPLIT ? 2 : 1) * TILE;     // [2]
+  uint8_t* sV = sK + 2 * TILE;                          // [2]
+
   const int4 it = A.items[blockIdx.x];
-  const int seq = it.x, h = it.y, j0 = it.z, t0 = it.w;
-  const int G = A.nq / A.nkv, g = h / G;
-  const int ntok = A.n_tok[seq];
+  const int seq = it.x, g = it.y, row0 = it.w;
+  const int G = A.nq / A.nkv;
   const int c0 = A.base[seq];
-  const int nrow = min(kPfaRows, ntok - t0);
-  const int kmax = c0 + t0 + nrow;    // positions the last query of the item sees
-  const int64_t kvbase = (A.seq_off[seq] * A.nkv + (int64_t)g * A.cap[seq]) * HD;
-  bf16* sK[2];
-  bf16* sV[2];
-  sK[0] = reinterpret_cast<bf16*>(smraw);
-  sV[0] = sK[0] + kPfaKeys * KROW;
-  sK[1] = sV[0] + kPfaKeys * KROW;
-  sV[1] = sK[1] + kPfaKeys * KROW;
+  const int R = A.n_tok[seq] * G;                       // rows of this (sequence, KV head)
+  const int nq = NQ == 2 && R - row0 > kPfaRows ? 2 : 1;   // tiles with rows
+  const int last = min(R, row0 + nq * kPfaRows) - 1;
+  const int kmax = c0 + last / G + 1;                   // positions the last row sees
+  const int n = (kmax + kPfaKeys - 1) / kPfaKeys;
 
-  auto issue = [&](int kt, int buf) {
-    const int p0 = kt * kPfaKeys;
-    const int cnt = min(kPfaKeys, kmax - p0);
-    for (int x = tid; x < kPfaKeys * V16; x += kPfaThreads) {
-      const int r = x / V16, q16 = x - r * V16;
-      bf16* kd = sK[buf] + r * KROW + q16 * 8;
-      bf16* vd = sV[buf] + r * KROW + q16 * 8;
-      if (r < cnt) {
-        const size_t off = (size_t)(kvbase + (int64_t)(p0 + r) * HD + q16 * 8);
-        cp_async16(kd, A.Kc + off);
-        cp_async16(vd, A.Vc + off);
-      } else {   // rows past the range: zero (their probabilities are 0; 0 * stale could be NaN)
-        *reinterpret_cast<uint4*>(kd) = make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(vd) = make_uint4(0u, 0u, 0u, 0u);
-      }
+  if (tid == 0) {
+    ptx::mbar_init(&q_ready, 128 * nq);
+    for (int b = 0; b < 2; ++b) {
+      ptx::mbar_init(&k_full[b], kPfaLoadThreads);
+      ptx::mbar_init(&v_full[b], kPfaLoadThreads);
+      ptx::mbar_init(&k_empty[b], 1);
+      ptx::mbar_init(&v_empty[b], 1);
+      ptx::mbar_init(&s_full[b], 1);
+      ptx::mbar_init(&p_ready[b], 128);
+      ptx::mbar_init(&o_full[b], 1);
     }
-  };
-
-  const int ntiles = (kmax + kPfaKeys - 1) / kPfaKeys;
-  issue(0, 0);
-  cp_async_commit();
-
-  // queries of this warp's 16 tokens as A fragments: row r = lane / 4 (+ 8),
-  // columns 2 (lane % 4) (+ 1) (+ 8) of each k-step; pre-scaled
-  const float scale = 1.4426950408889634f * rsqrtf((float)HD);
-  const int gr = lane >> 2, tc = (lane & 3) * 2;
-  const int rA = warp * 16 + gr, rB = rA + 8;          // rows within the item
-  const bool vA = rA < nrow, vB = rB < nrow;
-  const float* qA = A.q + ((size_t)(j0 + rA) * A.nq + h) * HD;
-  const float* qB = A.q + ((size_t)(j0 + rB) * A.nq + h) * HD;
-  uint32_t qh[KSTEPS][4], ql[KSTEPS][4];
-#pragma unroll
-  for (int kk = 0; kk < KSTEPS; ++kk) {
-    float2 a0 = vA ? *reinterpret_cast<const float2*>(qA + kk * 16 + tc) : make_float2(0.f, 0.f);
-    float2 a1 = vB ? *reinterpret_cast<const float2*>(qB + kk * 16 + tc) : make_float2(0.f, 0.f);
-    float2 a2 = vA ? *reinterpret_cast<const float2*>(qA + kk * 16 + 8 + tc) : make_float2(0.f, 0.f);
-    float2 a3 = vB ? *reinterpret_cast<const float2*>(qB + kk * 16 + 8 + tc) : make_float2(0.f, 0.f);
-    const float2 f[4] = {a0, a1, a2, a3};
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      if (SPLIT) tca::split_pack(f[r].x * scale, f[r].y * scale, qh[kk][r], ql[kk][r]);
-      else qh[kk][r] = tca::pack_bf16(f[r].x * scale, f[r].y * scale);
-    }
+    ptx::mbar_init(&pv_done, 1);
+    ptx::mbar_init(&drained, 1);
+    abort_flag = 0;
+    ptx::fence_mbar_init();
   }
-  const int qposA = c0 + t0 + rA, qposB = c0 + t0 + rB;   // cache positions of the two rows
-  float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;
-  float o[DT][4];
-#pragma unroll
-  for (int t = 0; t < DT; ++t) o[t][0] = o[t][1] = o[t][2] = o[t][3] = 0.f;
+  constexpr int kMmaWarp = 4 * NQ;
+  if (warp == kMmaWarp) {
+    ptx::tmem_alloc(&tmem_slot, 512);
+    ptx::tmem_relinquish();
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = tmem_slot;
 
-  for (int kt = 0; kt < ntiles; ++kt) {
-    const int buf = kt & 1;
-    if (kt + 1 < ntiles) issue(kt + 1, buf ^ 1);
-    cp_async_commit();
-    cp_async_wait<1>();
-    __syncthreads();
-    const bf16* Ks = sK[buf];
-    const bf16* Vs = sV[buf];
-    const int p0 = kt * kPfaKeys;
-    // ---- S = Q K^T: 16 tokens x 64 positions
-    float s[NT][4];
+  if (warp < kMmaWarp) {
+    const int q = warp >> 2;                            // this warp's tile
+    if (q < nq) {
+      // ------------------------------------------------------------- softmax
+      const int rt = (warp & 3) * 32 + lane;            // row of the tile
+      const bool live = row0 + q * kPfaRows + rt < R;
+      const int row = min(R - 1, row0 + q * kPfaRows + rt);
+      const int t = row / G, h = g * G + row - t * G;
+      const size_t at = ((size_t)(it.z + t) * A.nq + h) * HD;
+      {   // the row's query, scaled, as bf16 (hi, lo) in the swizzled K-major layout
+        const float scale = 1.4426950408889634f * rsqrtf((float)HD);
+        const float4* src = reinterpret_cast<const float4*>(A.q + at);
+        uint8_t* dst = sQ + (size_t)q * (SPLIT ? 2 : 1) * TILE;
+#pragma unroll 8
+        for (int c = 0; c < V16; ++c) {
+          const float4 a = src[2 * c], b = src[2 * c + 1];
+          const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+          uint32_t hi[4], lo[4];
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+          for (int i = 0; i < 4; ++i) tca::split_pack(f[2 * i] * scale, f[2 * i + 1] * scale, hi[i], lo[i]);
+          *reinterpret_cast<uint4*>(dst + pfa_piece(rt, c)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          if (SPLIT) *reinterpret_cast<uint4*>(dst + TILE + pfa_piece(rt, c)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        ptx::mbar_arrive(&q_ready);
+      }
+      const uint32_t tq = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+      const uint32_t to = tq + kO + (uint32_t)q * 128u;
+      const int seen = c0 + t + 1;                      // positions this row sees
+      float m = -INFINITY, l = 0.f;
+      bool ok = true;
+      for (int j = 0; j < n; ++j) {
+        const int slot = NQ == 2 ? q : (j & 1);
+        const uint32_t ph = (uint32_t)(NQ == 2 ? j & 1 : (j >> 1) & 1);
+        ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&s_full[slot], ph, A.wait_ns, &abort_flag));
+        if (!ok) break;
+        ptx::tc_fence_after();
+        const uint32_t ts = tq + (uint32_t)slot * 128u;
+        const int lim = seen - j * kPfaKeys;            // visible columns of this tile (may be <= 0)
+        const bool cut = __any_sync(0xffffffffu, lim < kPfaKeys);
+        uint32_t s[kPfaKeys];   // the row, read once (P overwrites its columns)
 #pragma unroll
-    for (int np = 0; np < NT; np += 2) {
-      // ldmatrix x4: positions 8 np.. / 8 (np + 1).., dims +0 / +8 of a k-step
-      const int m4 = lane >> 3, r8 = lane & 7;
-      const bf16* kr = Ks + (size_t)(8 * np + 8 * (m4 >> 1) + r8) * KROW + 8 * (m4 & 1);
+        for (int c = 0; c < kPfaKeys; c += 32) ptx::tmem_ld32(ts + c, s + c);
+        ptx::tmem_wait_ld();
+        if (cut) {
 #pragma unroll
-      for (int kk = 0; kk < KSTEPS; ++kk) {
-        uint32_t b0, b1, b2, b3;
-        tca::ldsm_x4(kr + kk * 16, b0, b1, b2, b3);
-        tca::mma16816(s[np], qh[kk][0], qh[kk][1], qh[kk][2], qh[kk][3], b0, b1);
-        tca::mma16816(s[np + 1], qh[kk][0], qh[kk][1], qh[kk][2], qh[kk][3], b2, b3);
-        if (SPLIT) {
-          tca::mma16816(s[np], ql[kk][0], ql[kk][1], ql[kk][2], ql[kk][3], b0, b1);
-          tca::mma16816(s[np + 1], ql[kk][0], ql[kk][1], ql[kk][2], ql[kk][3], b2, b3);
+          for (int i = 0; i < kPfaKeys; ++i)
+            if (i >= lim) s[i] = 0xff800000u;   // -inf: p = 0
+        }
+        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int i = 0; i < kPfaKeys; ++i) mx4[i & 3] = fmaxf(mx4[i & 3], __uint_as_float(s[i]));
+        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+        // position 0 is visible to every row: m is finite from tile 0 on
+        const bool raise = mx > m + 8.f;
+        if (__any_sync(0xffffffffu, raise)) {
+          const float al = raise ? tca::exp2a(m - mx) : 1.f;
+          if (raise) m = mx;
+          l *= al;
+          if (j > 0) {
+            if (NQ == 1) {   // S of this tile was computed before the previous tile's O += P V ended
+              ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&pv_done, (uint32_t)((j - 1) & 1), A.wait_ns,
+                                                                  &abort_flag));
+              if (!ok) break;
+              ptx::tc_fence_after();
+            }
+#pragma unroll 1
+            for (int c = 0; c < HD; c += 32) {
+              uint32_t o[32];
+              ptx::tmem_ld32(to + c, o);
+              ptx::tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * al);
+              ptx::tmem_st32(to + c, o);
+            }
+          }
+        }
+        float ls[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < kPfaKeys; c += 32) {
+          uint32_t hi[16], lo[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float p0 = tca::exp2a(__uint_as_float(s[c + 2 * i]) - m);
+            const float p1 = tca::exp2a(__uint_as_float(s[c + 2 * i + 1]) - m);
+            ls[i & 3] += p0 + p1;
+            if (SPLIT) tca::split_pack(p0, p1, hi[i], lo[i]);
+            else hi[i] = tca::pack_bf16(p0, p1);
+          }
+          ptx::tmem_st16(ts + c / 2, hi);
+          if (SPLIT) ptx::tmem_st16(tq + kPLo + (uint32_t)slot * 64u + c / 2, lo);
+        }
+        l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        ptx::tmem_wait_st();
+        ptx::tc_fence_before();
+        ptx::mbar_arrive(&p_ready[slot]);
+      }
+      if (ok) ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&o_full[q], 0, A.wait_ns, &abort_flag));
+      if (ok) {
+        ptx::tc_fence_after();
+        const float inv = 1.f / l;
+#pragma unroll 1
+        for (int c = 0; c < HD; c += 32) {
+          uint32_t o[32];
+          ptx::tmem_ld32(to + c, o);
+          ptx::tmem_wait_ld();
+          if (!live) continue;
+#pragma unroll
+          for (int i = 0; i < 32; i += 8) {
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              tca::split_pack(__uint_as_float(o[i + 2 * e]) * inv, __uint_as_float(o[i + 2 * e + 1]) * inv, hi[e],
+                              lo[e]);
+            *reinterpret_cast<uint4*>(A.out + at + c + i) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            if (SPLIT) *reinterpret_cast<uint4*>(A.out_lo + at + c + i) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          }
         }
       }
     }
-    // ---- masks and online softmax (rows A = gr, B = gr + 8)
-    float cmA = -INFINITY, cmB = -INFINITY;
+  } else if (warp == kMmaWarp) {
+    // -------------------------------------------------------------------- MMA
+    if (lane == 0) {
+      const uint32_t id_s = ptx::idesc_bf16(128u, (uint32_t)kPfaKeys);
+      const uint32_t id_o = ptx::idesc_bf16(128u, (uint32_t)HD) | ptx::kIdescBMnMajor;
+      auto wait = [&](uint64_t* bar, int phase) {
+        return ptx::mbar_wait_bounded(bar, (uint32_t)(phase & 1), A.wait_ns, &abort_flag);
+      };
+      auto qk = [&](int q, int slot, int j) {   // S slot = Q_q K_j^T
+        const uint8_t* Q = sQ + (size_t)q * (SPLIT ? 2 : 1) * TILE;
+        const uint8_t* K = sK + (size_t)(j & 1) * TILE;
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const int pp = p0 + nt * 8 + tc;
-      if (pp > qposA) s[nt][0] = -INFINITY;
-      if (pp + 1 > qposA) s[nt][1] = -INFINITY;
-      if (pp > qposB) s[nt][2] = -INFINITY;
-      if (pp + 1 > qposB) s[nt][3] = -INFINITY;
-      cmA = fmaxf(cmA, fmaxf(s[nt][0], s[nt][1]));
-      cmB = fmaxf(cmB, fmaxf(s[nt][2], s[nt][3]));
-    }
+        for (int k = 0; k < HD / 16; ++k) {
+          const uint64_t dk = ptx::smem_desc_sw128(K + (k >> 2) * kPfaRegion) + 2ull * (k & 3);
+          const uint64_t dq = ptx::smem_desc_sw128(Q + (k >> 2) * kPfaRegion) + 2ull * (k & 3);
+          ptx::mma_bf16(tmem + (uint32_t)slot * 128u, dq, dk, id_s, k > 0 ? 1u : 0u);
+          if (SPLIT) {
+            const uint64_t dl = ptx::smem_desc_sw128(Q + TILE + (k >> 2) * kPfaRegion) + 2ull * (k & 3);
+            ptx::mma_bf16(tmem + (uint32_t)slot * 128u, dl, dk, id_s, 1u);
+          }
+        }
+        ptx::mma_commit(&s_full[slot]);
+      };
+      auto pv = [&](int q, int slot, int j) {   // O_q += P V_j
+        const uint8_t* V = sV + (size_t)(j & 1) * TILE;
+        const uint32_t d = tmem + kO + (uint32_t)q * 128u, a = tmem + (uint32_t)slot * 128u;
 #pragma unroll
-    for (int off = 1; off < 4; off <<= 1) {
-      cmA = fmaxf(cmA, __shfl_xor_sync(0xffffffffu, cmA, off));
-      cmB = fmaxf(cmB, __shfl_xor_sync(0xffffffffu, cmB, off));
-    }
-    // position 0 of tile 0 is visible to every row, so the running max is
-    // finite from the first tile on
-    const float nmA = fmaxf(mA, cmA), nmB = fmaxf(mB, cmB);
-    const float alA = tca::exp2a(mA - nmA), alB = tca::exp2a(mB - nmB);
-    mA = nmA;
-    mB = nmB;
-    float psA = 0.f, psB = 0.f;
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      s[nt][0] = tca::exp2a(s[nt][0] - mA);
-      s[nt][1] = tca::exp2a(s[nt][1] - mA);
-      s[nt][2] = tca::exp2a(s[nt][2] - mB);
-      s[nt][3] = tca::exp2a(s[nt][3] - mB);
-      psA += s[nt][0] + s[nt][1];
-      psB += s[nt][2] + s[nt][3];
-    }
-    lA = lA * alA + psA;   // per-thread partial sums; the quad is reduced at the end
-    lB = lB * alB + psB;
-#pragma unroll
-    for (int t = 0; t < DT; ++t) {
-      o[t][0] *= alA;
-      o[t][1] *= alA;
-      o[t][2] *= alB;
-      o[t][3] *= alB;
-    }
-    // ---- O += P V: k-steps of 16 positions (two position tiles)
-#pragma unroll
-    for (int kk = 0; kk < NT / 2; ++kk) {
-      uint32_t ah[4], al[4] = {0u, 0u, 0u, 0u};
-      if (SPLIT) {
-        tca::split_pack(s[2 * kk][0], s[2 * kk][1], ah[0], al[0]);
-        tca::split_pack(s[2 * kk][2], s[2 * kk][3], ah[1], al[1]);
-        tca::split_pack(s[2 * kk + 1][0], s[2 * kk + 1][1], ah[2], al[2]);
-        tca::split_pack(s[2 * kk + 1][2], s[2 * kk + 1][3], ah[3], al[3]);
-      } else {
-        ah[0] = tca::pack_bf16(s[2 * kk][0], s[2 * kk][1]);
-        ah[1] = tca::pack_bf16(s[2 * kk][2], s[2 * kk][3]);
-        ah[2] = tca::pack_bf16(s[2 * kk + 1][0], s[2 * kk + 1][1]);
-        ah[3] = tca::pack_bf16(s[2 * kk + 1][2], s[2 * kk + 1][3]);
+        for (int k = 0; k < kPfaKeys / 16; ++k) {
+          const uint64_t dv = ptx::smem_desc_sw128_mn(V + k * 2048, kPfaRegion);   // 16 positions: two 1 KiB groups
+          ptx::mma_bf16_ts(d, a + 8u * k, dv, id_o, (j > 0 || k > 0) ? 1u : 0u);
+          if (SPLIT) ptx::mma_bf16_ts(d, tmem + kPLo + (uint32_t)slot * 64u + 8u * k, dv, id_o, 1u);
+        }
+      };
+      bool ok = wait(&q_ready, 0) && wait(&k_full[0], 0);
+      if (ok) {
+        ptx::tc_fence_after();
+        for (int q = 0; q < nq; ++q) qk(q, q, 0);
+        ptx::mma_commit(&k_empty[0]);
       }
-      // ldmatrix.trans x4: positions 16 kk + 0..7 / + 8..15, channels +0 / +8
-      const int m4 = lane >> 3, r8 = lane & 7;
-      const bf16* vr = Vs + (size_t)(16 * kk + 8 * (m4 & 1) + r8) * KROW + 8 * (m4 >> 1);
-#pragma unroll
-      for (int t = 0; t < DT; t += 2) {
-        uint32_t b0, b1, b2, b3;
-        tca::ldsm_x4_t(vr + t * 8, b0, b1, b2, b3);
-        tca::mma16816(o[t], ah[0], ah[1], ah[2], ah[3], b0, b1);
-        tca::mma16816(o[t + 1], ah[0], ah[1], ah[2], ah[3], b2, b3);
-        if (SPLIT) {
-          tca::mma16816(o[t], al[0], al[1], al[2], al[3], b0, b1);
-          tca::mma16816(o[t + 1], al[0], al[1], al[2], al[3], b2, b3);
+      for (int j = 0; j < n && ok; ++j) {
+        const bool more = j + 1 < n;
+        if (NQ == 2) {
+          for (int q = 0; q < nq && ok; ++q) {
+            ok = wait(&p_ready[q], j) && (q > 0 || wait(&v_full[j & 1], j >> 1)) &&
+                 (q > 0 || !more || wait(&k_full[(j + 1) & 1], (j + 1) >> 1));
+            if (!ok) break;
+            ptx::tc_fence_after();
+            pv(q, q, j);
+            if (q == nq - 1) ptx::mma_commit(&v_empty[j & 1]);
+            if (more) {
+              qk(q, q, j + 1);   // in issue order after the P V that reads P from the same columns
+              if (q == nq - 1) ptx::mma_commit(&k_empty[(j + 1) & 1]);
+            } else {
+              ptx::mma_commit(&o_full[q]);
+            }
+          }
+        } else {
+          if (more) {
+            ok = wait(&k_full[(j + 1) & 1], (j + 1) >> 1);
+            if (!ok) break;
+            ptx::tc_fence_after();
+            qk(0, (j + 1) & 1, j + 1);
+            ptx::mma_commit(&k_empty[(j + 1) & 1]);
+          }
+          ok = wait(&p_ready[j & 1], j >> 1) && wait(&v_full[j & 1], j >> 1);
+          if (!ok) break;
+          ptx::tc_fence_after();
+          pv(0, j & 1, j);
+          ptx::mma_commit(&v_empty[j & 1]);
+          ptx::mma_commit(more ? &pv_done : &o_full[0]);
         }
       }
     }
-    __syncthreads();   // the buffer is refilled by the next iteration's issue
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------ K, V copies
+    const int lt = tid - 32 * (kMmaWarp + 1);
+    const int64_t kvbase = (A.seq_off[seq] * A.nkv + (int64_t)g * A.cap[seq]) * HD;
+    constexpr int RPI = kPfaLoadThreads / V16;   // rows per round
+    const int c = lt % V16, r0 = lt / V16;
+    auto copy = [&](uint8_t* dst, const bf16* src, int j) {
+      const int p0 = j * kPfaKeys;
+      const uint32_t d = ptx::smem_u32(dst);
+      const bf16* s = src + kvbase + (int64_t)p0 * HD + c * 8;
+#pragma unroll 8
+      for (int r = r0; r < kPfaKeys; r += RPI) {
+        const bool real = p0 + r < kmax;
+        cp_async16_or_zero(d + pfa_piece(r, c), real ? s + (int64_t)r * HD : A.Kc, real);
+      }
+      cp_async_commit();
+    };
+    // loads K0 V0 K1 V1 ..: a load is announced once the next one is issued
+    uint64_t* pending = nullptr;
+    bool ok = true;
+    for (int x = 0; x < 2 * n && ok; ++x) {
+      const int j = x >> 1, b = j & 1;
+      const bool isk = (x & 1) == 0;
+      ok = ptx::mbar_wait_bounded(isk ? &k_empty[b] : &v_empty[b], (uint32_t)(((j >> 1) & 1) ^ 1), A.wait_ns,
+                                  &abort_flag);
+      if (!ok) break;
+      copy((isk ? sK : sV) + (size_t)b * TILE, isk ? A.Kc : A.Vc, j);
+      if (pending) {
+        cp_async_wait<1>();
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        ptx::mbar_arrive(pending);
+      }
+      pending = isk ? &k_full[b] : &v_full[b];
+    }
+    cp_async_wait<0>();
+    if (ok && pending) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      ptx::mbar_arrive(pending);
+    }
   }
-  cp_async_wait<0>();
 
-#pragma unroll
-  for (int off = 1; off < 4; off <<= 1) {
-    lA += __shfl_xor_sync(0xffffffffu, lA, off);
-    lB += __shfl_xor_sync(0xffffffffu, lB, off);
-  }
-  const float iA = 1.f / lA, iB = 1.f / lB;
-  const size_t qd = (size_t)A.nq * HD;
-#pragma unroll
-  for (int t = 0; t < DT; ++t) {
-    const int ch = h * HD + t * 8 + tc;
-    if (vA) {
-      store_out(A.out, A.out_lo, (size_t)(j0 + rA) * qd + ch, o[t][0] * iA);
-      store_out(A.out, A.out_lo, (size_t)(j0 + rA) * qd + ch + 1, o[t][1] * iA);
+  // every issued MMA completes before TMEM is freed: normally all have (o_full),
+  // after a wait that ran out the MMA warp waits for its own
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    if (abort_flag) {
+      if (lane == 0) {
+        ptx::mma_commit(&drained);
+        volatile int dummy = 0;
+        ptx::mbar_wait_bounded(&drained, 0, kWaitLimitNs, &dummy);
+        atomicOr(A.status, BUDDY_DEV_TIMEOUT);
+      }
+      __syncwarp();
     }
-    if (vB) {
-      store_out(A.out, A.out_lo, (size_t)(j0 + rB) * qd + ch, o[t][2] * iB);
-      store_out(A.out, A.out_lo, (size_t)(j0 + rB) * qd + ch + 1, o[t][3] * iB);
-    }
+    ptx::tc_fence_after();
+    ptx::tmem_dealloc(tmem, 512);
   }
+}
+
+template <int HD, bool SPLIT>
+static int pfa_prepare() {
+  return cudaFuncSetAttribute(attn_pf_kernel<HD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)pfa_smem<HD, SPLIT>()) == cudaSuccess
+             ? BUDDY_OK
+             : BUDDY_ERR_CUDA;
+}
+int attention_pf_prepare(const Ctx& c) {
+  const int a = c.hd == 128 ? pfa_prepare<128, false>() : pfa_prepare<64, false>();
+  return a != BUDDY_OK ? a : (c.hd == 128 ? pfa_prepare<128, true>() : pfa_prepare<64, true>());
+}
+
+// Rows (tokens x heads of a group) of one work item.
+int attention_pf_rows(bool split) { return kPfaRows * (split ? pfa_tiles<true>() : pfa_tiles<false>()); }
+
+template <int HD, bool SPLIT>
+static void pfa_launch(const PfaArgs& A, int n_items, cudaStream_t s) {
+  attn_pf_kernel<HD, SPLIT><<<n_items, pfa_threads<SPLIT>(), pfa_smem<HD, SPLIT>(), s>>>(A);
 }
 
 void launch_attention_pf(const Ctx& c, int n_items, const int4* items, const int32_t* n_tok, const int32_t* base,
                          const buddy_kv_state& kv, int layer, const float* q, void* out, void* out_lo,
                          cudaStream_t s) {
-  PfaArgs A{items, n_tok, base, q, kv.seq_off, kv.cap, (const bf16*)kv.k_cache[layer],
-            (const bf16*)kv.v_cache[layer], (bf16*)out, (bf16*)out_lo, c.nq, c.nkv, c.status};
+  const PfaArgs A{items, n_tok, base, q, kv.seq_off, kv.cap, (const bf16*)kv.k_cache[layer],
+                  (const bf16*)kv.v_cache[layer], (bf16*)out, (bf16*)out_lo, c.nq, c.nkv, c.status, c.wait_ns};
   if (c.hd == 128) {
-    const size_t smem = attn_pf_smem<128>();
-    if (out_lo) {
-      cudaFuncSetAttribute(attn_pf_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      attn_pf_kernel<128, true><<<n_items, kPfaThreads, smem, s>>>(A);
-    } else {
-      cudaFuncSetAttribute(attn_pf_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      attn_pf_kernel<128, false><<<n_items, kPfaThreads, smem, s>>>(A);
-    }
+    if (out_lo) pfa_launch<128, true>(A, n_items, s);
+    else pfa_launch<128, false>(A, n_items, s);
   } else {
-    const size_t smem = attn_pf_smem<64>();
-    if (out_lo) {
-      cudaFuncSetAttribute(attn_pf_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      attn_pf_kernel<64, true><<<n_items, kPfaThreads, smem, s>>>(A);
-    } else {
-      cudaFuncSetAttribute(attn_pf_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      attn_pf_kernel<64, false><<<n_items, kPfaThreads, smem, s>>>(A);
-    }
+    if (out_lo) pfa_launch<64, true>(A, n_items, s);
+    else pfa_launch<64, false>(A, n_items, s);
   }
 }
 

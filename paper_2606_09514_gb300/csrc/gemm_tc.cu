@@ -513,7 +513,8 @@ int gemm_tc_prepare(Ctx& c) {
         !make_map(&c.pf_tmaps[4], c.pf_attn_lo, c.pf_max, c.qd, 128) ||
         !make_map(&c.pf_tmaps[5], c.pf_act_lo, c.pf_max, c.F, 128))
       return BUDDY_ERR_CUDA;
-    const int rc = gemm_pf_prepare(c);
+    int rc = gemm_pf_prepare(c);
+    if (rc == BUDDY_OK) rc = attention_pf_prepare(c);
     if (rc != BUDDY_OK) return rc;
   }
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;

@@ -155,6 +155,8 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
 void launch_attention_pf(const Ctx& c, int n_items, const int4* items, const int32_t* n_tok, const int32_t* base,
                          const buddy_kv_state& kv, int layer, const float* q, void* out, void* out_lo,
                          cudaStream_t s);
+int attention_pf_prepare(const Ctx& c);
+int attention_pf_rows(bool split);       // (token, query head of a group) rows per work item
 void launch_pool_refresh_n(const Ctx& c, const buddy_kv_state& kv, int n_seq, const int32_t* n_new,
                            cudaStream_t s);
 int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_host, const float* x,

@@ -208,26 +208,36 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
                                     c.masked ? kv.layer_len : nullptr, c.L, kv.batch, c.status);
   pf_tokens_kernel<<<(T + 255) / 256, 256, 0, s>>>(T, c.pf_tok_seq, c.pf_tok_t, kv.len, c.pf_tok_pos, c.status);
 
-  // attention work items for a set of sequences: 64 query tokens x one head
-  auto items_for = [&](const std::vector<int>& seqs, std::vector<int4>& out) {
+  // attention work items for a set of sequences: (token, head of a group) rows
+  // of one KV head, those that see the most positions first (the last to start
+  // are then the shortest)
+  const int G = c.nq / c.nkv;
+  auto items_for = [&](const std::vector<int>& seqs, bool split, std::vector<int4>& out) {
+    const int rows = attention_pf_rows(split);
+    const size_t at = out.size();
     int j = 0;
     for (int i : seqs) {
-      for (int t0 = 0; t0 < n_tok_host[i]; t0 += 64)
-        for (int h = 0; h < c.nq; ++h) out.push_back(make_int4(i, h, j + t0, t0));
+      for (int r0 = 0; r0 < n_tok_host[i] * G; r0 += rows)
+        for (int g = 0; g < c.nkv; ++g) out.push_back(make_int4(i, g, j, r0));
       j += n_tok_host[i];
     }
+    std::stable_sort(out.begin() + at, out.end(), [](const int4& a, const int4& b) { return a.w > b.w; });
   };
   std::vector<int> all(B);
   for (int i = 0; i < B; ++i) all[i] = i;
+  // the item buffer: every sequence for the blocks that feed the router, every
+  // sequence for the last block, then the routed layers
   std::vector<int4> items_all;
-  items_for(all, items_all);
-  if ((int64_t)items_all.size() > c.pf_items_max) return BUDDY_ERR_RANGE;
-  // slot 0 of the item buffer: every sequence; slots 1.. : the routed layers
+  items_for(all, true, items_all);
+  const int n_split = (int)items_all.size();
+  items_for(all, false, items_all);
+  if ((int64_t)items_all.size() > 2 * c.pf_items_max) return BUDDY_ERR_RANGE;
   PCK(cudaMemcpyAsync(c.pf_items, items_all.data(), sizeof(int4) * items_all.size(), cudaMemcpyHostToDevice, s));
-  const PfLayerWork every{nullptr, T, c.pf_items, (int)items_all.size()};
+  const PfLayerWork feed{nullptr, T, c.pf_items, n_split};
+  const PfLayerWork every{nullptr, T, c.pf_items + n_split, (int)items_all.size() - n_split};
 
   // blocks 0..c on every token, then the router per prompt
-  for (int l = 0; l <= c.cl; ++l) pf_block(c, kv, l, every, l == 0 ? x : h_out, h_out, s, prof);
+  for (int l = 0; l <= c.cl; ++l) pf_block(c, kv, l, feed, l == 0 ? x : h_out, h_out, s, prof);
   {
     ProfScope p(c, s, BUDDY_PROF_ROUTE, 1, prof);
     launch_pool_refresh_n(c, kv, B, c.pf_n_tok, s);
@@ -271,7 +281,7 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
     item_at[l] = items_l.size();
     for (int i : seqs)
       for (int t = off[i]; t < off[i + 1]; ++t) rows_all.push_back(t);
-    items_for(seqs, items_l);
+    items_for(seqs, false, items_l);
     work[l].m = (int)(rows_all.size() - row_at[l]);
     work[l].n_items = (int)(items_l.size() - item_at[l]);
   }
