@@ -57,7 +57,7 @@ static void free_ctx(buddy_ctx* x) {
                   c.count, c.h_in_stage, c.h_out_stage, c.k_stage, c.mask_stage, c.xn_lo, c.act_lo, c.attn_lo,
                   c.gemm_ws, c.gemm_ctr, c.pf_xn, c.pf_xn_lo, c.pf_q, c.pf_attn, c.pf_attn_lo,
                   c.pf_act, c.pf_act_lo, c.pf_tok_seq, c.pf_tok_t, c.pf_tok_pos, c.pf_rows, c.pf_items,
-                  c.pf_n_tok, c.pf_tok_end, c.pf_cnt, c.pf_hlast};
+                  c.pf_n_tok, c.pf_tok_end, c.pf_cnt, c.pf_hlast, c.pf_ws, c.pf_ctr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (x->cap_stream) cudaStreamDestroy(x->cap_stream);
@@ -269,6 +269,7 @@ extern "C" int buddy_device_status(buddy_ctx* ctx, void* stream, int32_t* flags)
   if (h[0] & BUDDY_DEV_TIMEOUT) {
     // a GEMM that gave up left split-K arrival counters mid-count: re-arm them
     if (c.gemm_ctr) CK(cudaMemsetAsync(c.gemm_ctr, 0, c.gemm_ctr_n * sizeof(int32_t), s));
+    if (c.pf_ctr) CK(cudaMemsetAsync(c.pf_ctr, 0, c.pf_ctr_n * sizeof(int32_t), s));
     CK(cudaMemsetAsync(c.attn_ctr, 0, (size_t)c.maxB * c.nkv * sizeof(int32_t), s));
   }
   CK(cudaStreamSynchronize(s));

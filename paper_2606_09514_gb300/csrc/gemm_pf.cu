@@ -19,6 +19,14 @@
 // weights: for a gate/up projection larger than L2 that is an HBM pass per
 // M-tile.)
 //
+// Units that do not fill a last wave of pairs are cut along K (pf_bound): each
+// pair takes an equal, contiguous share of their K blocks, first of all its work,
+// stages the accumulator of a part in a workspace slot, and the pair that
+// completes a unit sums the parts in K order and applies the epilogue.  With one
+// short prompt every unit is such a unit: Llama-3-8B's O projection has 16, which
+// kept 16 of the 76 pairs busy for 64 K blocks (61 tokens on a 4-block
+// Llama-3-8B: 0.85 -> 0.73 ms; 5 prompts, 2,878 tokens: 4.06 -> 3.93 ms).
+//
 // Warp 0 of each CTA issues the TMA loads of its part of a stage ([X 128 x 64]
 // [X remainder 128 x 64 with SPLIT][W 128 x 64], 128-byte swizzle; the bytes of
 // both CTAs are counted on CTA 0's barrier); warp 1 of CTA 0 issues tcgen05.mma
@@ -52,7 +60,12 @@ constexpr uint32_t kPfTileBytes = 128u * 128u; // one 128-row x 64-column bf16 t
 
 struct PfParams {
   int N, K, m;
-  int n_tiles, m_tiles, kb_total, units;
+  int n_tiles, m_tiles, kb_total;
+  int units;               // units computed whole, by pair u % pairs
+  int sk_units;            // units after them, cut along K over sk_pairs pairs
+  int sk_pairs, sk_gran;   // cuts fall on multiples of sk_gran K blocks of a unit
+  float4* ws;              // sk: [pair][part 0, 1][CTA] accumulators in fragment form
+  int32_t* ctr;            // sk: [unit][CTA] K blocks that have arrived
   int stages;
   uint32_t stage_bytes, w_off;
   // epilogue
@@ -88,6 +101,46 @@ __device__ __forceinline__ void pf_unit(const PfParams& p, int u, int& mt, int& 
   mt = g * kPfGroup + (r - nt * gm);
 }
 
+// Start of pair i's share of the cut units' K blocks, laid end to end.  A share
+// is at least sk_gran blocks (sk_pairs is chosen so) and shorter than a unit: it
+// touches one unit or two.
+__device__ __forceinline__ int pf_bound(const PfParams& p, int i) {
+  const int T = p.sk_units * p.kb_total;
+  if (i >= p.sk_pairs) return T;
+  const int x = i * T / p.sk_pairs, u = x / p.kb_total;
+  return u * p.kb_total + (x - u * p.kb_total) / p.sk_gran * p.sk_gran;
+}
+
+// A piece of a pair's work: K blocks [kb0, kb1) of unit u; part >= 0 of a cut unit.
+struct PfSeg {
+  int u, kb0, kb1, part;
+};
+struct PfWork {
+  int a, b, a0, u;   // cut K blocks left [a, b) (a0: where they began), next whole unit
+  __device__ __forceinline__ PfWork(const PfParams& p, int pair) : u(pair) {
+    a = a0 = pair < p.sk_pairs ? pf_bound(p, pair) : 0;
+    b = pair < p.sk_pairs ? pf_bound(p, pair + 1) : 0;
+  }
+  __device__ __forceinline__ bool next(const PfParams& p, int pairs, PfSeg& s) {
+    if (a < b) {
+      const int r = a / p.kb_total;
+      s.u = p.units + r;
+      s.kb0 = a - r * p.kb_total;
+      s.kb1 = min(p.kb_total, s.kb0 + b - a);
+      s.part = r == a0 / p.kb_total ? 0 : 1;
+      a += s.kb1 - s.kb0;
+      return true;
+    }
+    if (u >= p.units) return false;
+    s.u = u;
+    s.kb0 = 0;
+    s.kb1 = p.kb_total;
+    s.part = -1;
+    u += pairs;
+    return true;
+  }
+};
+
 // First row of the half of weight tile nt that CTA `rank` of the pair loads.
 // SwiGLU: CTA 0 the gate rows, CTA 1 the matching up rows (N + f0..).
 template <int EPI>
@@ -105,6 +158,87 @@ __device__ __forceinline__ int pf_w_row(const PfParams& p, int nt, uint32_t rank
 // sectors for 16 bytes each: 25 us for a 256 x 256 tile's residual epilogue,
 // more than the tile's MMAs at K = 4096.
 // ---------------------------------------------------------------------------
+// Parts of cut units.  A part is stored as the epilogue threads hold it: blocks
+// of 16 rows x 64 columns, 8 float4 per thread, a warp's 32 threads side by side.
+__device__ __forceinline__ size_t pf_slot(int pair, int part, uint32_t rank) {
+  return ((size_t)(pair * 2 + part) * 2 + rank) * (32 * 8 * 32);   // float4
+}
+__device__ __forceinline__ size_t pf_block(int q, int h16, int col) {
+  return (size_t)((q * 2 + h16) * 4 + (col >> 6)) * (8 * 32);
+}
+
+// Stages this warp's accumulators (rows of its quarter at ta, its half of the
+// columns).
+__device__ __noinline__ void pf_stage(float4* slot, uint32_t ta, int q, int half, int lane) {
+#pragma unroll 1
+  for (int h16 = 0; h16 < 2; ++h16)
+#pragma unroll 1
+    for (int c = half * 128; c < half * 128 + 128; c += 64) {
+      uint32_t r[32];
+      ptx::tmem_ld_frag<8>(ta + c + ((uint32_t)(h16 * 16) << 16), r);
+      ptx::tmem_wait_ld();
+      float4* d = slot + pf_block(q, h16, c) + lane;
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        __stcg(d + k * 32, make_float4(__uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1]),
+                                       __uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3])));
+    }
+}
+
+// The sum of the parts that pairs i0 .. i1 staged (part s0 of pair i0, part 0 of
+// the others), in that order, back into the accumulator; two parts' loads in
+// flight.
+__device__ __noinline__ void pf_gather(const float4* ws, int i0, int i1, int s0, uint32_t rank, uint32_t ta, int q,
+                                          int half, int lane) {
+#pragma unroll 1
+  for (int h16 = 0; h16 < 2; ++h16)
+#pragma unroll 1
+    for (int c = half * 128; c < half * 128 + 128; c += 64) {
+      const float4* base = ws + pf_block(q, h16, c) + lane;
+      float4 v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+      for (int i = i0; i <= i1; i += 2) {
+        float4 x[8], y[8];
+        const float4* bx = base + pf_slot(i, i == i0 ? s0 : 0, rank);
+        const float4* by = base + pf_slot(i + 1, 0, rank);
+        const bool two = i < i1;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) x[k] = __ldcg(bx + k * 32);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (two) y[k] = __ldcg(by + k * 32);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          v[k].x += x[k].x;
+          v[k].y += x[k].y;
+          v[k].z += x[k].z;
+          v[k].w += x[k].w;
+        }
+        if (two) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            v[k].x += y[k].x;
+            v[k].y += y[k].y;
+            v[k].z += y[k].z;
+            v[k].w += y[k].w;
+          }
+        }
+      }
+      uint32_t r[32];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        r[4 * k] = __float_as_uint(v[k].x);
+        r[4 * k + 1] = __float_as_uint(v[k].y);
+        r[4 * k + 2] = __float_as_uint(v[k].z);
+        r[4 * k + 3] = __float_as_uint(v[k].w);
+      }
+      ptx::tmem_st_frag8(ta + c + ((uint32_t)(h16 * 16) << 16), r);
+    }
+  ptx::tmem_wait_st();
+}
+
 __device__ __forceinline__ uint32_t pf_pack(float a, float b) {
   return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
          ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
@@ -124,37 +258,36 @@ __device__ __forceinline__ void st_bf16_pair(bf16* row, uint32_t wg, uint32_t wg
 
 __device__ __forceinline__ void pf_resid(const PfParams& p, int j0, int nt, int half, uint32_t ta, int lane) {
   const int gr = lane >> 2, tc = (lane & 3) * 2;
-  size_t off[4];
-  bool live[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int j = j0 + gr + 8 * i;
-    live[i] = j < p.m;
-    off[i] = (size_t)(live[i] ? (p.rows ? p.rows[j] : j) : 0) * p.N;
-  }
 #pragma unroll 1
-  for (int c0 = half * 128; c0 < half * 128 + 128; c0 += 64) {
+  for (int x = 0; x < 4; ++x) {
+    const int h16 = x >> 1, c0 = half * 128 + (x & 1) * 64;
     const int n0 = nt * 256 + c0;
-    if (n0 >= p.N) break;   // N is a multiple of 64
-    float2 s[8][4];
+    if (n0 >= p.N) continue;   // N is a multiple of 64
+    bool live[2];
+    size_t at[2];
+    float2 s[8][2];
 #pragma unroll
-    for (int g = 0; g < 8; ++g)
+    for (int i = 0; i < 2; ++i) {
+      const int j = j0 + h16 * 16 + gr + 8 * i;
+      live[i] = j < p.m;
+      at[i] = (size_t)(live[i] ? (p.rows ? p.rows[j] : j) : 0) * p.N + n0 + tc;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (live[i]) s[g][i] = *reinterpret_cast<const float2*>(p.resid_src + off[i] + n0 + 8 * g + tc);
+      for (int g = 0; g < 8; ++g)
+        if (live[i]) s[g][i] = *reinterpret_cast<const float2*>(p.resid_src + at[i] + 8 * g);
+    }
     __syncwarp();
-    uint32_t v[2][32];
-    ptx::tmem_ld_frag<8>(ta + c0, v[0]);
-    ptx::tmem_ld_frag<8>(ta + c0 + (16u << 16), v[1]);
+    uint32_t v[32];
+    ptx::tmem_ld_frag<8>(ta + c0 + ((uint32_t)(h16 * 16) << 16), v);
     ptx::tmem_wait_ld();
 #pragma unroll
-    for (int g = 0; g < 8; ++g)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int g = 0; g < 8; ++g)
         if (live[i])
-          *reinterpret_cast<float2*>(p.resid_dst + off[i] + n0 + 8 * g + tc) =
-              make_float2(s[g][i].x + __uint_as_float(v[i >> 1][4 * g + (i & 1) * 2]),
-                          s[g][i].y + __uint_as_float(v[i >> 1][4 * g + (i & 1) * 2 + 1]));
+          *reinterpret_cast<float2*>(p.resid_dst + at[i] + 8 * g) =
+              make_float2(s[g][i].x + __uint_as_float(v[4 * g + 2 * i]),
+                          s[g][i].y + __uint_as_float(v[4 * g + 2 * i + 1]));
+    __syncwarp();
   }
 }
 
@@ -288,8 +421,8 @@ __device__ __forceinline__ void pf_qkv(const PfParams& p, int j0, int nt, int ha
   }
 }
 
-// Epilogue of rows j0 .. j0 + 31 (this warp's TMEM quarter at ta) of unit tile
-// nt, one half of its columns.
+// Epilogue of rows j0 .. j0 + 31 (this warp's quarter) of unit tile nt, one half
+// of its columns.
 template <int EPI, bool SPLIT>
 __device__ __forceinline__ void pf_epilogue(const PfParams& p, int j0, int nt, int half, uint32_t ta, int lane) {
   if (EPI == EPI_RESID) pf_resid(p, j0, nt, half, ta, lane);
@@ -322,6 +455,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
   __shared__ int issued_of[2];   // CTA 0: stages each CTA loaded
+  __shared__ int last_part;      // the part just staged completed its unit
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_rank();
@@ -360,11 +494,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
     uint32_t ph = 0;
     int issued = 0;
     bool ok = true;
-    for (int u = pair; u < p.units && ok; u += pairs) {
+    PfWork work(p, pair);
+    PfSeg sg;
+    while (ok && work.next(p, pairs, sg)) {
       int mt, nt;
-      pf_unit(p, u, mt, nt);
+      pf_unit(p, sg.u, mt, nt);
       const int xrow = mt * 256 + (int)rank * 128, wrow = pf_w_row<EPI>(p, nt, rank);
-      for (int kb = 0; kb < p.kb_total; ++kb) {
+      for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
         ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&empty_bar[stage], ph ^ 1u, p.wait_ns, &abort_flag));
         if (!ok) break;
         uint8_t* st = smem + (size_t)stage * p.stage_bytes;
@@ -396,13 +532,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
       int acc = 0;
       uint32_t acc_ph = 0;
       bool ok = true;
-      for (int u = pair; u < p.units && ok; u += pairs) {
+      PfWork work(p, pair);
+      PfSeg sg;
+      while (ok && work.next(p, pairs, sg)) {
         ok = __all_sync(0xffffffffu,
                         ptx::mbar_wait_bounded<true>(&tempty_bar[acc], acc_ph ^ 1u, p.wait_ns, &abort_flag));
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t d = tmem_base + (uint32_t)acc * 256u;
-        for (int kb = 0; kb < p.kb_total; ++kb) {
+        for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
           ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&full_bar[stage], ph, p.wait_ns, &abort_flag));
           if (!ok) break;
           ++consumed;
@@ -414,11 +552,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
           if (ptx::elect_one()) {
 #pragma unroll
             for (int k = 0; k < kTileK / 16; ++k) {
-              ptx::mma_bf16_pair(d, da + 2ull * k, dw + 2ull * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+              ptx::mma_bf16_pair(d, da + 2ull * k, dw + 2ull * k, idesc, (kb > sg.kb0 || k > 0) ? 1u : 0u);
               if (SPLIT) ptx::mma_bf16_pair(d, dl + 2ull * k, dw + 2ull * k, idesc, 1u);
             }
             ptx::mma_commit_pair(&empty_bar[stage]);
-            if (kb + 1 == p.kb_total) ptx::mma_commit_pair(&tfull_bar[acc]);
+            if (kb + 1 == sg.kb1) ptx::mma_commit_pair(&tfull_bar[acc]);
           }
           __syncwarp();
           if (++stage == p.stages) {
@@ -442,15 +580,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
     const int half = (warp - 2) >> 2;  // columns it takes
     int acc = 0;
     uint32_t acc_ph = 0;
-    for (int u = pair; u < p.units; u += pairs) {
+    PfWork work(p, pair);
+    PfSeg sg;
+    while (work.next(p, pairs, sg)) {
       const bool ok = ptx::mbar_wait_bounded(&tfull_bar[acc], acc_ph, p.wait_ns, &abort_flag);
       if (pf_epi_any(!ok)) break;
       ptx::tc_fence_after();
       int mt, nt;
-      pf_unit(p, u, mt, nt);
+      pf_unit(p, sg.u, mt, nt);
       const int j0 = mt * 256 + (int)rank * 128 + q * 32;
       const uint32_t ta = tmem_base + (uint32_t)acc * 256u + ((uint32_t)(q * 32) << 16);
-      pf_epilogue<EPI, SPLIT>(p, j0, nt, half, ta, lane);
+      bool finish = true;
+      if (sg.kb1 - sg.kb0 < p.kb_total) {   // a part of a cut unit
+        pf_stage(p.ws + pf_slot(pair, sg.part, rank), ta, q, half, lane);
+        pf_epi_any(false);   // every thread's part is stored before the arrival is counted
+        const int r = sg.u - p.units;
+        if (threadIdx.x == 64) {
+          int32_t* ctr = p.ctr + r * 2 + rank;
+          const int had = ptx::atom_add_acq_rel(ctr, sg.kb1 - sg.kb0);
+          last_part = had + sg.kb1 - sg.kb0 == p.kb_total;
+          if (last_part) *ctr = 0;   // re-armed for a later launch
+        }
+        pf_epi_any(false);
+        finish = last_part;
+        if (finish) {
+          // the pairs whose shares meet this unit
+          const int k0 = r * p.kb_total, k1 = k0 + p.kb_total;
+          int i0 = min(p.sk_pairs - 1, r * p.sk_pairs / p.sk_units);
+          while (i0 > 0 && pf_bound(p, i0) > k0) --i0;
+          while (i0 + 1 < p.sk_pairs && pf_bound(p, i0 + 1) <= k0) ++i0;
+          int i1 = i0;
+          while (i1 + 1 < p.sk_pairs && pf_bound(p, i1 + 1) < k1) ++i1;
+          pf_gather(p.ws, i0, i1, pf_bound(p, i0) < k0 ? 1 : 0, rank, ta, q, half, lane);
+          ptx::tc_fence_before();
+          pf_epi_any(false);   // SwiGLU reads columns that the other warp of the quarter gathered
+          ptx::tc_fence_after();
+        }
+      }
+      if (finish) pf_epilogue<EPI, SPLIT>(p, j0, nt, half, ta, lane);
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive_cluster(ptx::dsmem_addr(&tempty_bar[acc], 0));
@@ -485,6 +652,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
 // Host side
 // ---------------------------------------------------------------------------
 int gemm_pf_prepare(Ctx& c) {
+  // parts of cut units: two accumulators of 256 x 256 fp32 per pair; arrival
+  // counters per cut unit (fewer than pairs) and CTA
+  const size_t pairs = c.num_sms / 2;
+  if (!c.pf_ws && cudaMalloc(&c.pf_ws, pairs * 2 * 256 * 256 * sizeof(float)) != cudaSuccess) return BUDDY_ERR_CUDA;
+  c.pf_ctr_n = (int)pairs * 2;
+  if (!c.pf_ctr && cudaMalloc(&c.pf_ctr, c.pf_ctr_n * sizeof(int32_t)) != cudaSuccess) return BUDDY_ERR_CUDA;
+  if (cudaMemset(c.pf_ctr, 0, c.pf_ctr_n * sizeof(int32_t)) != cudaSuccess) return BUDDY_ERR_CUDA;
   const int limit = 227 * 1024 - 2 * 1024;
   for (int v = 0; v < 2; ++v) {
     const uint32_t sb = (v ? 3u : 2u) * kPfTileBytes;
@@ -516,7 +690,21 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
   p.n_tiles = tiles;
   p.m_tiles = (m + 255) / 256;
   p.kb_total = (K + kTileK - 1) / kTileK;
-  p.units = p.n_tiles * p.m_tiles;
+  // Whole waves of units, then the rest cut along K where that saves more than
+  // staging and summing the parts costs (about 10 us; a K block takes 0.26 us,
+  // twice that with SPLIT): R units left for P pairs end a fraction (P - R) / P
+  // of a unit's time earlier.  Cuts at multiples of 4 K blocks, at most 8 parts.
+  const int P = c.num_sms / 2, units = p.n_tiles * p.m_tiles, R = units % P;
+  const bool cut = (int64_t)(P - R) * p.kb_total * (split ? 52 : 26) > (int64_t)1000 * P;
+  p.sk_units = R > 0 && cut ? R : 0;
+  p.units = units - p.sk_units;
+  if (p.sk_units) {
+    const int T = p.sk_units * p.kb_total;
+    p.sk_gran = std::max(4, P <= 6 * R ? 4 : (p.kb_total + 7) / 8);
+    p.sk_pairs = std::max(1, std::min(P, T / p.sk_gran));
+    p.ws = c.pf_ws;
+    p.ctr = c.pf_ctr;
+  }
   const int v = split ? 1 : 0;
   p.stages = c.pf_stages[v];
   p.stage_bytes = (split ? 3u : 2u) * kPfTileBytes;
@@ -546,7 +734,7 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
   const CUtensorMap& tw = c.pf_wmaps[(size_t)layer * 4 + which];
   const CUtensorMap& tx = c.pf_tmaps[xi];
   const CUtensorMap& txlo = c.pf_tmaps[3 + xi];
-  const int grid = 2 * std::min(p.units, c.num_sms / 2);
+  const int grid = 2 * (p.units ? std::min(std::max(p.units, p.sk_pairs), P) : p.sk_pairs);
   const size_t smem = c.pf_smem[v];
   if (split) {
     switch (epi) {

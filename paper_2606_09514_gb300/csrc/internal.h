@@ -256,6 +256,9 @@ struct Ctx {
   std::vector<CUtensorMap> pf_wmaps;   // per layer 4 weight maps, 128-row boxes
   CUtensorMap pf_tmaps[6];        // pf_xn, pf_attn, pf_act, then their remainder terms
   int pf_stages[2] = {1, 1}, pf_smem[2] = {0, 0};
+  float4* pf_ws = nullptr;        // parts of units cut along K
+  int32_t* pf_ctr = nullptr;      // K blocks that have arrived, per cut unit and CTA
+  int pf_ctr_n = 0;
 
   // profiler: event pairs around kernel launches (direct-launch mode only)
   int profiling = 0;
