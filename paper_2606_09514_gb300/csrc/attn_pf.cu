@@ -99,7 +99,12 @@ __global__ void __launch_bounds__(pfa_threads<SPLIT>(), 1) attn_pf_kernel(const 
   __shared__ __align__(8) uint64_t s_full[2], p_ready[2], pv_done, o_full[2], drained;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
-  if (call_aborted(A.status)) return;
+  // (written by the call's first kernel, complete before the preceding kernel let
+  // this one launch, as were the items, the token counts and the positions)
+  if (call_aborted(A.status)) {
+    pdl_wait();
+    return;
+  }
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -142,6 +147,8 @@ __global__ void __launch_bounds__(pfa_threads<SPLIT>(), 1) attn_pf_kernel(const 
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = tmem_slot;
+  pdl_wait();   // the queries, keys and values of the preceding kernel
+  pdl_trigger();
 
   if (warp < kMmaWarp) {
     const int q = warp >> 2;                            // this warp's tile
@@ -412,8 +419,8 @@ int attention_pf_prepare(const Ctx& c) {
 int attention_pf_rows(bool split) { return kPfaRows * (split ? pfa_tiles<true>() : pfa_tiles<false>()); }
 
 template <int HD, bool SPLIT>
-static void pfa_launch(const PfaArgs& A, int n_items, cudaStream_t s) {
-  attn_pf_kernel<HD, SPLIT><<<n_items, pfa_threads<SPLIT>(), pfa_smem<HD, SPLIT>(), s>>>(A);
+static void pfa_launch(const PfaArgs& A, int n_items, bool pdl, cudaStream_t s) {
+  launch_k(attn_pf_kernel<HD, SPLIT>, n_items, pfa_threads<SPLIT>(), pfa_smem<HD, SPLIT>(), s, pdl, A);
 }
 
 void launch_attention_pf(const Ctx& c, int n_items, const int4* items, const int32_t* n_tok, const int32_t* base,
@@ -422,11 +429,11 @@ void launch_attention_pf(const Ctx& c, int n_items, const int4* items, const int
   const PfaArgs A{items, n_tok, base, q, kv.seq_off, kv.cap, (const bf16*)kv.k_cache[layer],
                   (const bf16*)kv.v_cache[layer], (bf16*)out, (bf16*)out_lo, c.nq, c.nkv, c.status, c.wait_ns};
   if (c.hd == 128) {
-    if (out_lo) pfa_launch<128, true>(A, n_items, s);
-    else pfa_launch<128, false>(A, n_items, s);
+    if (out_lo) pfa_launch<128, true>(A, n_items, c.pdl, s);
+    else pfa_launch<128, false>(A, n_items, c.pdl, s);
   } else {
-    if (out_lo) pfa_launch<64, true>(A, n_items, s);
-    else pfa_launch<64, false>(A, n_items, s);
+    if (out_lo) pfa_launch<64, true>(A, n_items, c.pdl, s);
+    else pfa_launch<64, false>(A, n_items, c.pdl, s);
   }
 }
 

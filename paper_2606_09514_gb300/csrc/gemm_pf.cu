@@ -461,7 +461,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
   const uint32_t rank = ptx::cluster_rank();
   const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  if (call_aborted(p.status)) return;   // the same in both CTAs: the call's first kernel wrote it
+  // The call's first kernel wrote the abort word: it completed before the
+  // preceding kernel let this one launch, and both CTAs read the same.
+  if (call_aborted(p.status)) {
+    pdl_wait();
+    return;
+  }
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
@@ -489,7 +494,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
   int consumed = 0;   // CTA 0, MMA warp: stages waited for
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA
-    const uint32_t bytes = (SPLIT ? 3u : 2u) * kPfTileBytes;
+    // The first ring of weight tiles, which no earlier kernel writes, is on its
+    // way before the dependency wait.
+    int pre = 0;
+    {
+      PfWork work(p, pair);
+      PfSeg sg;
+      while (pre < p.stages && work.next(p, pairs, sg)) {
+        int mt, nt;
+        pf_unit(p, sg.u, mt, nt);
+        const int wrow = pf_w_row<EPI>(p, nt, rank);
+        for (int kb = sg.kb0; kb < sg.kb1 && pre < p.stages; ++kb, ++pre) {
+          const uint32_t bar = ptx::dsmem_addr(&full_bar[pre], 0);
+          if (ptx::elect_one()) {
+            ptx::mbar_expect_tx_cluster(bar, kPfTileBytes);
+            ptx::tma_load_2d_pair(smem + (size_t)pre * p.stage_bytes + p.w_off, &tw, bar, kb * kTileK, wrow);
+          }
+          __syncwarp();
+        }
+      }
+    }
+    pdl_wait();
+    pdl_trigger();
+    constexpr uint32_t x_bytes = (SPLIT ? 2u : 1u) * kPfTileBytes;
     int stage = 0;
     uint32_t ph = 0;
     int issued = 0;
@@ -501,15 +528,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
       pf_unit(p, sg.u, mt, nt);
       const int xrow = mt * 256 + (int)rank * 128, wrow = pf_w_row<EPI>(p, nt, rank);
       for (int kb = sg.kb0; kb < sg.kb1; ++kb) {
-        ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&empty_bar[stage], ph ^ 1u, p.wait_ns, &abort_flag));
-        if (!ok) break;
+        const bool have_w = issued < pre;
+        if (!have_w) {
+          ok = __all_sync(0xffffffffu, ptx::mbar_wait_bounded(&empty_bar[stage], ph ^ 1u, p.wait_ns, &abort_flag));
+          if (!ok) break;
+        }
         uint8_t* st = smem + (size_t)stage * p.stage_bytes;
         const uint32_t bar = ptx::dsmem_addr(&full_bar[stage], 0);
         if (ptx::elect_one()) {
-          ptx::mbar_arrive_expect_tx_cluster(bar, bytes);
+          ptx::mbar_arrive_expect_tx_cluster(bar, x_bytes + (have_w ? 0u : kPfTileBytes));
           ptx::tma_load_2d_pair(st, &tx, bar, kb * kTileK, xrow);
           if (SPLIT) ptx::tma_load_2d_pair(st + kPfTileBytes, &txlo, bar, kb * kTileK, xrow);
-          ptx::tma_load_2d_pair(st + p.w_off, &tw, bar, kb * kTileK, wrow);
+          if (!have_w) ptx::tma_load_2d_pair(st + p.w_off, &tw, bar, kb * kTileK, wrow);
         }
         __syncwarp();
         ++issued;
@@ -525,6 +555,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA (CTA 0 only)
+    pdl_wait();
     if (rank == 0) {
       const uint32_t idesc = ptx::idesc_bf16(256u, 256u);
       int stage = 0;
@@ -578,6 +609,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
     // ------------------------------------------------------------- epilogue
     const int q = warp & 3;            // TMEM lane quarter this warp may access
     const int half = (warp - 2) >> 2;  // columns it takes
+    pdl_wait();
     int acc = 0;
     uint32_t acc_ph = 0;
     PfWork work(p, pair);
@@ -738,15 +770,15 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
   const size_t smem = c.pf_smem[v];
   if (split) {
     switch (epi) {
-      case EPI_QKV: launch_k(gemm_pf_kernel<EPI_QKV, true>, grid, kPfThreads, smem, s, false, tw, tx, txlo, p); break;
-      case EPI_RESID: launch_k(gemm_pf_kernel<EPI_RESID, true>, grid, kPfThreads, smem, s, false, tw, tx, txlo, p); break;
-      default: launch_k(gemm_pf_kernel<EPI_SWIGLU, true>, grid, kPfThreads, smem, s, false, tw, tx, txlo, p);
+      case EPI_QKV: launch_k(gemm_pf_kernel<EPI_QKV, true>, grid, kPfThreads, smem, s, c.pdl, tw, tx, txlo, p); break;
+      case EPI_RESID: launch_k(gemm_pf_kernel<EPI_RESID, true>, grid, kPfThreads, smem, s, c.pdl, tw, tx, txlo, p); break;
+      default: launch_k(gemm_pf_kernel<EPI_SWIGLU, true>, grid, kPfThreads, smem, s, c.pdl, tw, tx, txlo, p);
     }
   } else {
     switch (epi) {
-      case EPI_QKV: launch_k(gemm_pf_kernel<EPI_QKV, false>, grid, kPfThreads, smem, s, false, tw, tx, txlo, p); break;
-      case EPI_RESID: launch_k(gemm_pf_kernel<EPI_RESID, false>, grid, kPfThreads, smem, s, false, tw, tx, txlo, p); break;
-      default: launch_k(gemm_pf_kernel<EPI_SWIGLU, false>, grid, kPfThreads, smem, s, false, tw, tx, txlo, p);
+      case EPI_QKV: launch_k(gemm_pf_kernel<EPI_QKV, false>, grid, kPfThreads, smem, s, c.pdl, tw, tx, txlo, p); break;
+      case EPI_RESID: launch_k(gemm_pf_kernel<EPI_RESID, false>, grid, kPfThreads, smem, s, c.pdl, tw, tx, txlo, p); break;
+      default: launch_k(gemm_pf_kernel<EPI_SWIGLU, false>, grid, kPfThreads, smem, s, c.pdl, tw, tx, txlo, p);
     }
   }
 }

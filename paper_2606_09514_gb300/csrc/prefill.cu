@@ -26,6 +26,8 @@ namespace buddy {
 // ---------------------------------------------------------------------------
 __global__ void pf_tokens_kernel(int T, const int32_t* tok_seq, const int32_t* tok_t, const int32_t* len,
                                  int32_t* tok_pos, const int32_t* status) {
+  pdl_wait();
+  pdl_trigger();
   if (call_aborted(status)) return;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r < T) tok_pos[r] = len[tok_seq[r]] + tok_t[r];
@@ -37,6 +39,8 @@ __global__ void pf_tokens_kernel(int T, const int32_t* tok_seq, const int32_t* t
 __global__ void pf_check_kernel(int B, const int32_t* k, int Lm, int k_min, const int32_t* n_tok,
                                 const int32_t* len, const int32_t* cap, int max_pos, const int32_t* layer_len, int L,
                                 int kv_batch, int32_t* status) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ int bad;
   if (threadIdx.x == 0) bad = 0;
   __syncthreads();
@@ -64,6 +68,8 @@ __global__ void pf_check_kernel(int B, const int32_t* k, int Lm, int k_min, cons
 // the number of positions the pooled context covers (len + n_tok).
 __global__ void pf_gather_kernel(int B, int d, const int32_t* tok_end, const float* H, const int32_t* len,
                                  const int32_t* n_tok, float* hlast, int32_t* cnt, const int32_t* status) {
+  pdl_wait();
+  pdl_trigger();
   if (call_aborted(status)) return;
   const int i = blockIdx.x;
   const float* src = H + (size_t)(tok_end[i] - 1) * d;
@@ -75,17 +81,18 @@ __global__ void pf_gather_kernel(int B, int d, const int32_t* tok_end, const flo
 // CTA per (block, prompt, KV head), 16 bytes at a time (5 prompts of 128..1023
 // tokens, 2 routed blocks: 11 us, against 92 us with a CTA per block and prompt
 // storing elements).
-template <typename T>
 __global__ void pf_zero_kernel(int B, int L, int first, int nkv, int hd, const uint8_t* mask, LayerPtrs ptrs,
                                const int32_t* len, const int32_t* n_tok, const int64_t* seq_off,
                                const int32_t* cap, const int32_t* status) {
+  pdl_wait();
+  pdl_trigger();
   if (call_aborted(status)) return;
   const int l = first + blockIdx.x, i = blockIdx.y, g = blockIdx.z;
   if (l >= L - 1 || mask[(size_t)i * L + l]) return;
   const int64_t base = kv_offset(seq_off, cap, i, nkv, hd, g, len[i]);
-  uint4* Kc = reinterpret_cast<uint4*>((T*)ptrs.k[l] + base);
-  uint4* Vc = reinterpret_cast<uint4*>((T*)ptrs.v[l] + base);
-  const int64_t n = (int64_t)n_tok[i] * hd * (int)sizeof(T) / 16;
+  uint4* Kc = reinterpret_cast<uint4*>((bf16*)ptrs.k[l] + base);
+  uint4* Vc = reinterpret_cast<uint4*>((bf16*)ptrs.v[l] + base);
+  const int64_t n = (int64_t)n_tok[i] * hd / 8;
   for (int64_t x = threadIdx.x; x < n; x += blockDim.x) {
     Kc[x] = make_uint4(0u, 0u, 0u, 0u);
     Vc[x] = make_uint4(0u, 0u, 0u, 0u);
@@ -96,6 +103,8 @@ __global__ void pf_zero_kernel(int B, int L, int first, int nkv, int hd, const u
 // prompt executed layer l.
 __global__ void pf_advance_kernel(int B, int L, const int32_t* n_tok, const uint8_t* mask, int32_t* len,
                                   int32_t* layer_len, int kv_batch, const int32_t* status) {
+  pdl_wait();
+  pdl_trigger();
   if (call_aborted(status)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B) return;
@@ -204,9 +213,11 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
   PCK(cudaMemcpyAsync(c.pf_n_tok, n_tok_host, sizeof(int32_t) * B, cudaMemcpyHostToDevice, s));
   PCK(cudaMemcpyAsync(c.pf_tok_end, ends.data(), sizeof(int32_t) * B, cudaMemcpyHostToDevice, s));
   const int k_min = c.have_pred ? 0 : 1;
-  pf_check_kernel<<<1, 256, 0, s>>>(B, k, c.Lm, k_min, c.pf_n_tok, kv.len, kv.cap, c.max_pos,
-                                    c.masked ? kv.layer_len : nullptr, c.L, kv.batch, c.status);
-  pf_tokens_kernel<<<(T + 255) / 256, 256, 0, s>>>(T, c.pf_tok_seq, c.pf_tok_t, kv.len, c.pf_tok_pos, c.status);
+  launch_k(pf_check_kernel, 1, 256, 0, s, c.pdl, B, k, c.Lm, k_min, (const int32_t*)c.pf_n_tok,
+           (const int32_t*)kv.len, kv.cap, c.max_pos, (const int32_t*)(c.masked ? kv.layer_len : nullptr), c.L,
+           kv.batch, c.status);
+  launch_k(pf_tokens_kernel, (T + 255) / 256, 256, 0, s, c.pdl, T, (const int32_t*)c.pf_tok_seq,
+           (const int32_t*)c.pf_tok_t, (const int32_t*)kv.len, c.pf_tok_pos, (const int32_t*)c.status);
 
   // attention work items for a set of sequences: (token, head of a group) rows
   // of one KV head, those that see the most positions first (the last to start
@@ -241,8 +252,8 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
   {
     ProfScope p(c, s, BUDDY_PROF_ROUTE, 1, prof);
     launch_pool_refresh_n(c, kv, B, c.pf_n_tok, s);
-    pf_gather_kernel<<<B, 256, 0, s>>>(B, c.d, c.pf_tok_end, h_out, kv.len, c.pf_n_tok, c.pf_hlast, c.pf_cnt,
-                                       c.status);
+    launch_k(pf_gather_kernel, B, 256, 0, s, c.pdl, B, c.d, (const int32_t*)c.pf_tok_end, (const float*)h_out,
+             (const int32_t*)kv.len, (const int32_t*)c.pf_n_tok, c.pf_hlast, c.pf_cnt, (const int32_t*)c.status);
     launch_route(c, B, c.pf_hlast, kv.pool_sum, c.pf_cnt, 0, k, c.mask, c.sel, c.scores, s);
   }
   // the routes come back to the host, which sizes every later launch
@@ -261,12 +272,8 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
     }
     ProfScope ps(c, s, BUDDY_PROF_PF_OTHER, 1, prof);
     dim3 g(std::max(1, c.Lm), B, c.nkv);
-    if (c.dtype == BUDDY_DTYPE_BF16)
-      pf_zero_kernel<bf16><<<g, 256, 0, s>>>(B, c.L, c.cl + 1, c.nkv, c.hd, c.mask, p, kv.len, c.pf_n_tok,
-                                             kv.seq_off, kv.cap, c.status);
-    else
-      pf_zero_kernel<float><<<g, 256, 0, s>>>(B, c.L, c.cl + 1, c.nkv, c.hd, c.mask, p, kv.len, c.pf_n_tok,
-                                              kv.seq_off, kv.cap, c.status);
+    launch_k(pf_zero_kernel, g, 256, 0, s, c.pdl, B, c.L, c.cl + 1, c.nkv, c.hd, (const uint8_t*)c.mask, p,
+             (const int32_t*)kv.len, (const int32_t*)c.pf_n_tok, kv.seq_off, kv.cap, (const int32_t*)c.status);
   }
   // row lists and work items of the routed layers
   std::vector<int32_t> rows_all;
@@ -302,8 +309,8 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
   pf_block(c, kv, c.L - 1, every, h_out, h_out, s, prof);
   {
     ProfScope p(c, s, BUDDY_PROF_PF_OTHER, 1, prof);
-    pf_advance_kernel<<<(B + 255) / 256, 256, 0, s>>>(B, c.L, c.pf_n_tok, c.mask, kv.len,
-                                                      c.masked ? kv.layer_len : nullptr, kv.batch, c.status);
+    launch_k(pf_advance_kernel, (B + 255) / 256, 256, 0, s, c.pdl, B, c.L, (const int32_t*)c.pf_n_tok,
+             (const uint8_t*)c.mask, kv.len, c.masked ? kv.layer_len : nullptr, kv.batch, (const int32_t*)c.status);
   }
   if (mask_out) PCK(cudaMemcpyAsync(mask_out, c.mask, (size_t)B * c.L, cudaMemcpyDeviceToDevice, s));
   if (scores_out)
