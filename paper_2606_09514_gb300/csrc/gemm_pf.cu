@@ -187,7 +187,8 @@ __device__ __noinline__ void pf_stage(float4* slot, uint32_t ta, int q, int half
 
 // The sum of the parts that pairs i0 .. i1 staged (part s0 of pair i0, part 0 of
 // the others), in that order, back into the accumulator; two parts' loads in
-// flight.
+// flight (four spill the kernel's registers, which costs every launch more than
+// the shorter sums give).
 __device__ __noinline__ void pf_gather(const float4* ws, int i0, int i1, int s0, uint32_t rank, uint32_t ta, int q,
                                           int half, int lane) {
 #pragma unroll 1
@@ -624,7 +625,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
       const uint32_t ta = tmem_base + (uint32_t)acc * 256u + ((uint32_t)(q * 32) << 16);
       bool finish = true;
       if (sg.kb1 - sg.kb0 < p.kb_total) {   // a part of a cut unit
-        pf_stage(p.ws + pf_slot(pair, sg.part, rank), ta, q, half, lane);
+        const bool any = j0 < p.m;   // rows past the last token are neither staged nor summed
+        if (any) pf_stage(p.ws + pf_slot(pair, sg.part, rank), ta, q, half, lane);
         pf_epi_any(false);   // every thread's part is stored before the arrival is counted
         const int r = sg.u - p.units;
         if (threadIdx.x == 64) {
@@ -643,7 +645,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPfThreads, 1)
           while (i0 + 1 < p.sk_pairs && pf_bound(p, i0 + 1) <= k0) ++i0;
           int i1 = i0;
           while (i1 + 1 < p.sk_pairs && pf_bound(p, i1 + 1) < k1) ++i1;
-          pf_gather(p.ws, i0, i1, pf_bound(p, i0) < k0 ? 1 : 0, rank, ta, q, half, lane);
+          if (any) pf_gather(p.ws, i0, i1, pf_bound(p, i0) < k0 ? 1 : 0, rank, ta, q, half, lane);
           ptx::tc_fence_before();
           pf_epi_any(false);   // SwiGLU reads columns that the other warp of the quarter gathered
           ptx::tc_fence_after();
@@ -723,16 +725,18 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
   p.m_tiles = (m + 255) / 256;
   p.kb_total = (K + kTileK - 1) / kTileK;
   // Whole waves of units, then the rest cut along K where that saves more than
-  // staging and summing the parts costs (about 10 us; a K block takes 0.26 us,
+  // staging and summing the parts costs (about 8 us; a K block takes 0.26 us,
   // twice that with SPLIT): R units left for P pairs end a fraction (P - R) / P
-  // of a unit's time earlier.  Cuts at multiples of 4 K blocks, at most 8 parts.
+  // of a unit's time earlier.  With few units a part is a quarter of a unit (a
+  // sum of more parts takes as long as the shorter parts save), else cuts fall on
+  // multiples of 4 K blocks.
   const int P = c.num_sms / 2, units = p.n_tiles * p.m_tiles, R = units % P;
-  const bool cut = (int64_t)(P - R) * p.kb_total * (split ? 52 : 26) > (int64_t)1000 * P;
+  const bool cut = (int64_t)(P - R) * p.kb_total * (split ? 52 : 26) > (int64_t)800 * P;
   p.sk_units = R > 0 && cut ? R : 0;
   p.units = units - p.sk_units;
   if (p.sk_units) {
     const int T = p.sk_units * p.kb_total;
-    p.sk_gran = std::max(4, P <= 6 * R ? 4 : (p.kb_total + 7) / 8);
+    p.sk_gran = std::max(4, P <= 4 * R ? 4 : (p.kb_total + 3) / 4);
     p.sk_pairs = std::max(1, std::min(P, T / p.sk_gran));
     p.ws = c.pf_ws;
     p.ctr = c.pf_ctr;
