@@ -14,7 +14,7 @@
 namespace buddy {
 
 constexpr int kMaxLayers = 128;
-constexpr int kRouteZSlots = 16;  // K-split slots of the router's hidden-unit partial sums
+constexpr int kRouteZSlots = 32;  // K-split slots of the router's hidden-unit partial sums
 constexpr int kMaxBatch = 1024;
 
 // Per-layer K/V base pointers passed by value to kernels that touch many layers.
@@ -131,6 +131,7 @@ bool attention_tc(const Ctx& c);         // tensor-core loop over the whole GPU
 bool attention_cl(const Ctx& c);         // small batches: one cluster per stream (attn_cl.cu)
 void launch_attention_cl(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int layer, const float* q, void* out,
                          void* out_lo, cudaStream_t s);
+cudaError_t route_prepare();
 void launch_route(const Ctx& c, int B, const float* h1, const float* pool, const int32_t* len,
                   int len_bias, const int32_t* k, uint8_t* mask, int32_t* sel, float* scores,
                   cudaStream_t s);
@@ -202,7 +203,6 @@ struct Ctx {
   float* attn_acc = nullptr;   // [maxB, nq, max_chunks, hd]
   int32_t* attn_ctr = nullptr; // [maxB, nkv] chunk arrivals (self-resetting)
   float* dm_u = nullptr;       // [kRouteZSlots, maxB, r + predictor hidden] partial sums
-  float* dm_x = nullptr;       // [maxB, 2d] router inputs (larger batches)
   uint8_t* mask = nullptr;     // [maxB, L]
   int32_t* sel = nullptr;      // [maxB, Lm]
   float* scores = nullptr;     // [maxB, Lm]

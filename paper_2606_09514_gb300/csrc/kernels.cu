@@ -323,12 +323,14 @@ void launch_pool_update(const Ctx& c, int B, const buddy_kv_state& kv, cudaStrea
 // Small batches: one CTA per hidden unit and up to 8 sequences; its 8 warps
 // take 8 contiguous slices of the 2d-long dot product (four float4 loads of
 // W1 in flight per lane), then reduce through shared memory.  Larger batches
-// (route_hidden_tiled_kernel): a tiled fp32 GEMM whose K splits leave
+// (route_gemm_kernel): a tiled fp32 GEMM whose K splits leave
 // partial sums that part 2 adds in split order.
 // ---------------------------------------------------------------------------
 constexpr int kRouteRows = 8;
 constexpr int kRouteTiledMin = 16;    // batches above this take the tiled router GEMM
 constexpr int kRtBM = 64, kRtBN = 64, kRtBK = 32;
+constexpr int kRtStages = 4, kRtRow = kRtBK + 4;   // buffers, floats from one row to the next
+constexpr int kRtSmem = kRtStages * (kRtBM + kRtBN) * kRtRow * 4;
 
 __global__ void __launch_bounds__(256) route_hidden_kernel(
     int B, int d, int hd, int group, int nkv, const float* __restrict__ h1,
@@ -392,105 +394,115 @@ __global__ void __launch_bounds__(256) route_hidden_kernel(
   }
 }
 
-// Router part 1 for larger batches, step 1: the router input of every row,
-// X[i] = [pool_sum[i] / (len[i] + len_bias) expanded over query heads ; h1[i]]
-// ([B, 2d] fp32), so that the GEMM below reads plain rows.
-__global__ void __launch_bounds__(256) route_pack_kernel(int d, int hd, int group, int nkv,
+// Router part 1 for larger batches: Z[i][unit] = X[i] . W[unit] over one K split,
+// a split lying in one half of the router input: the pooled half (read from the
+// pooled sums of the KV head that query head k / hd shares; the division by the
+// positions is applied to the split's sums) or the hidden half.  Tiles of 64 rows
+// x 64 units, K in steps of 32 through a ring of kRtStages shared-memory buffers
+// (16-byte cp.async, three steps in flight; the weights of the first three before
+// the dependency wait); rows are 36 floats apart, so that the 16 threads that
+// read 16 units' float4 meet no bank twice in a phase.  Each of the 256 threads
+// accumulates 4 rows x 4 units.  Split s writes slot s of z ([splits, B, r +
+// rp]); part 2 adds the slots in split order.  Bound by latency at few tiles and
+// by shared-memory reads and fp32 FMA at many: a whole routing call of 250 rows x
+// 256 units x 7168 takes 39.6 us, against 66.8 us with one step in flight and a
+// kernel that packed the rows first.
+__global__ void __launch_bounds__(256) route_gemm_kernel(int B, int d, int hd, int group, int nkv,
                                                          const float* __restrict__ h1,
                                                          const float* __restrict__ pool, const int32_t* len,
-                                                         int len_bias, float* __restrict__ X,
-                                                         const int32_t* status) {
-  pdl_wait();
-  pdl_trigger();
-  if (call_aborted(status)) return;
-  const int i = blockIdx.x;
-  const float inv = 1.0f / (float)(len[i] + len_bias);
-  const int kvd = nkv * hd;
-  float4* xo = reinterpret_cast<float4*>(X + (size_t)i * 2 * d);
-  for (int k = threadIdx.x * 4; k < 2 * d; k += blockDim.x * 4) {
-    float4 v;
-    if (k < d) {
-      const int qh = k / hd, e = k - qh * hd;
-      v = *reinterpret_cast<const float4*>(pool + (size_t)i * kvd + (qh / group) * hd + e);
-      v.x *= inv; v.y *= inv; v.z *= inv; v.w *= inv;
-    } else {
-      v = *reinterpret_cast<const float4*>(h1 + (size_t)i * d + (k - d));
-    }
-    xo[k >> 2] = v;
-  }
-}
-
-// Router part 1 for larger batches, step 2: Z[i][unit] = X[i] . W[unit] over
-// one K split.  Tiles of 64 rows x 64 units, K in steps of 32 staged in
-// shared memory (transposed: the inner loop reads 4 consecutive rows and 4
-// consecutive units as float4) with the next step's float4 loads in
-// registers while the current one is consumed; each of the 256 threads
-// accumulates 4 rows x 4 units.  Split s writes slot s of z ([splits, B,
-// r + rp]); part 2 adds the slots in split order.
-__global__ void __launch_bounds__(256) route_gemm_kernel(int B, int K2, const float* __restrict__ X,
-                                                         const float* __restrict__ w1, int r,
+                                                         int len_bias, const float* __restrict__ w1, int r,
                                                          const float* __restrict__ pw1, int rp, int k_per_split,
                                                          float* __restrict__ z, const int32_t* status) {
-  pdl_wait();
-  pdl_trigger();
-  if (call_aborted(status)) return;
-  __shared__ __align__(16) float xs[kRtBK][kRtBM + 4];
-  __shared__ __align__(16) float ws[kRtBK][kRtBN + 4];
+  extern __shared__ __align__(16) float rt_smem[];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int u0 = blockIdx.x * kRtBN, i0 = blockIdx.y * kRtBM;
   const int cols = r + rp;
-  const int ka = blockIdx.z * k_per_split, kb = min(K2, ka + k_per_split);
+  const int half = gridDim.z >> 1;
+  const bool hidden = (int)blockIdx.z >= half;
+  const int ka = ((int)blockIdx.z - (hidden ? half : 0)) * k_per_split, kb = min(d, ka + k_per_split);
+  const int steps = kb > ka ? (kb - ka + kRtBK - 1) / kRtBK : 0;
+  auto xbuf = [&](int s) { return rt_smem + (size_t)s * (kRtBM + kRtBN) * kRtRow; };
   // this thread's two float4 of each tile: (row or unit) = e / 8, k4 = e % 8
-  float4 xr[2], wr[2];
-  auto fetch = [&](int k0) {
+  auto load = [&](int step, bool weights) {
+    const int k0 = ka + step * kRtBK;
+    float* dst = xbuf(step % kRtStages) + (weights ? kRtBM * kRtRow : 0);
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int e = tid + q * 256, rr = e >> 3, k = k0 + (e & 7) * 4;
-      const int i = i0 + rr, unit = u0 + rr;
-      xr[q] = (i < B && k < kb) ? *reinterpret_cast<const float4*>(X + (size_t)i * K2 + k)
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float* wp = unit < r ? w1 + (size_t)unit * K2 : pw1 + (size_t)(unit - r) * K2;
-      wr[q] = (unit < cols && k < kb) ? __ldg(reinterpret_cast<const float4*>(wp + k))
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int row = (weights ? u0 : i0) + rr;
+      const bool real = row < (weights ? cols : B) && k < kb;
+      const float* src = w1;
+      if (real) {
+        if (weights)
+          src = (row < r ? w1 + (size_t)row * 2 * d : pw1 + (size_t)(row - r) * 2 * d) + (hidden ? d : 0) + k;
+        else if (hidden)
+          src = h1 + (size_t)row * d + k;
+        else
+          src = pool + (size_t)row * nkv * hd + (k / hd) / group * hd + k % hd;
+      }
+      const uint32_t n = real ? 16u : 0u;   // else zeros
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(dst + rr * kRtRow + (e & 7) * 4)),
+                   "l"(src), "r"(n)
+                   : "memory");
     }
   };
-  auto stash = [&]() {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int e = tid + q * 256, rr = e >> 3, kk = (e & 7) * 4;
-      xs[kk][rr] = xr[q].x; xs[kk + 1][rr] = xr[q].y; xs[kk + 2][rr] = xr[q].z; xs[kk + 3][rr] = xr[q].w;
-      ws[kk][rr] = wr[q].x; ws[kk + 1][rr] = wr[q].y; ws[kk + 2][rr] = wr[q].z; ws[kk + 3][rr] = wr[q].w;
-    }
-  };
+  auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+  for (int s = 0; s < kRtStages - 1; ++s)
+    if (s < steps) load(s, true);
+  pdl_wait();
+  pdl_trigger();
+  if (call_aborted(status)) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return;
+  }
+  for (int s = 0; s < kRtStages - 1; ++s) {
+    if (s < steps) load(s, false);
+    commit();
+  }
   float acc[4][4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) acc[a][0] = acc[a][1] = acc[a][2] = acc[a][3] = 0.f;
-  fetch(ka);
-  for (int k0 = ka; k0 < kb; k0 += kRtBK) {
-    __syncthreads();   // the previous step's tiles are consumed
-    stash();
-    __syncthreads();
-    if (k0 + kRtBK < kb) fetch(k0 + kRtBK);   // in flight while this step computes
-#pragma unroll 8
-    for (int kk = 0; kk < kRtBK; ++kk) {
-      const float4 a = *reinterpret_cast<const float4*>(&xs[kk][ty * 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&ws[kk][tx * 4]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+  for (int p = 0; p < 4; ++p) acc[p][0] = acc[p][1] = acc[p][2] = acc[p][3] = 0.f;
+  for (int s = 0; s < steps; ++s) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRtStages - 2) : "memory");
+    __syncthreads();   // step s has landed for every thread, step s - 1 is consumed
+    if (s + kRtStages - 1 < steps) {
+      load(s + kRtStages - 1, true);
+      load(s + kRtStages - 1, false);
+    }
+    commit();
+    const float* xs = xbuf(s % kRtStages) + ty * kRtRow;
+    const float* ws = xbuf(s % kRtStages) + (kRtBM + tx) * kRtRow;
+#pragma unroll
+    for (int kk = 0; kk < kRtBK; kk += 4) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        a[p] = *reinterpret_cast<const float4*>(xs + p * 16 * kRtRow + kk);
+        b[p] = *reinterpret_cast<const float4*>(ws + p * 16 * kRtRow + kk);
+      }
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] += av[p] * bv[q];
+        for (int q = 0; q < 4; ++q) {
+          acc[p][q] += a[p].x * b[q].x;
+          acc[p][q] += a[p].y * b[q].y;
+          acc[p][q] += a[p].z * b[q].z;
+          acc[p][q] += a[p].w * b[q].w;
+        }
     }
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   float* zs = z + (size_t)blockIdx.z * B * cols;
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
-    const int i = i0 + ty * 4 + p;
+    const int i = i0 + ty + 16 * p;
     if (i >= B) continue;
+    const float inv = hidden ? 1.f : 1.0f / (float)(len[i] + len_bias);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int unit = u0 + tx * 4 + q;
-      if (unit < cols) zs[(size_t)i * cols + unit] = acc[p][q];
+      const int unit = u0 + tx + 16 * q;
+      if (unit < cols) zs[(size_t)i * cols + unit] = acc[p][q] * inv;
     }
   }
 }
@@ -520,6 +532,7 @@ __global__ void __launch_bounds__(1024) route_select_kernel(
   // hidden units: K-split partial sums in split order, bias, SiLU
   for (int c = threadIdx.x; c < r + rp; c += blockDim.x) {
     float v = 0.f;
+#pragma unroll 8
     for (int sp = 0; sp < splits; ++sp) v += z[((size_t)sp * B + i) * (r + rp) + c];
     ui[c] = silu_f(v + (c < r ? b1[c] : pb1[c - r]));
   }
@@ -579,12 +592,17 @@ __global__ void __launch_bounds__(1024) route_select_kernel(
   if (threadIdx.x == 0 && mask) mask[(size_t)i * L + L - 1] = 1;
 }
 
-// K splits of the tiled router GEMM: about 256 CTAs, at most kRouteZSlots.
+// K splits of the tiled router GEMM (half of them for each half of the input):
+// about two CTAs per SM, at most kRouteZSlots.
 static int route_splits(const Ctx& c, int B) {
   if (B <= kRouteTiledMin) return 1;
   const int cols = c.r + (c.have_pred ? c.pred.hidden : 0);
   const int tiles = ((cols + kRtBN - 1) / kRtBN) * ((B + kRtBM - 1) / kRtBM);
-  return std::max(1, std::min(kRouteZSlots, 256 / std::max(1, tiles)));
+  return 2 * std::max(1, std::min(kRouteZSlots / 2, c.num_sms / tiles));
+}
+
+cudaError_t route_prepare() {
+  return cudaFuncSetAttribute(route_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRtSmem);
 }
 
 void launch_route(const Ctx& c, int B, const float* h1, const float* pool, const int32_t* len,
@@ -599,12 +617,11 @@ void launch_route(const Ctx& c, int B, const float* h1, const float* pool, const
              len_bias, c.dm.w1, c.dm.b1, c.r, c.have_pred ? c.pred.w1 : nullptr, c.have_pred ? c.pred.b1 : nullptr,
              rp, c.dm_u, (const int32_t*)c.status);
   } else {
-    launch_k(route_pack_kernel, B, 256, 0, s, c.pdl, c.d, c.hd, c.nq / c.nkv, c.nkv, h1, pool, len, len_bias,
-             c.dm_x, (const int32_t*)c.status);
-    const int kps = ((2 * c.d + splits - 1) / splits + kRtBK - 1) / kRtBK * kRtBK;
+    const int half = splits / 2;
+    const int kps = ((c.d + half - 1) / half + kRtBK - 1) / kRtBK * kRtBK;
     dim3 g1((cols + kRtBN - 1) / kRtBN, (B + kRtBM - 1) / kRtBM, splits);
-    launch_k(route_gemm_kernel, g1, 256, 0, s, c.pdl, B, 2 * c.d, (const float*)c.dm_x, c.dm.w1, c.r,
-             c.have_pred ? c.pred.w1 : nullptr, rp, kps, c.dm_u, (const int32_t*)c.status);
+    launch_k(route_gemm_kernel, g1, 256, kRtSmem, s, c.pdl, B, c.d, c.hd, c.nq / c.nkv, c.nkv, h1, pool, len, len_bias,
+             c.dm.w1, c.r, c.have_pred ? c.pred.w1 : nullptr, rp, kps, c.dm_u, (const int32_t*)c.status);
   }
   const int sel_threads = 32 * std::min(32, (c.have_pred ? 2 : 1) * c.Lm);
   launch_k(route_select_kernel, B, sel_threads, (2 * c.Lm + cols) * sizeof(float), s, c.pdl, c.Lm, c.cl + 1, c.r,
