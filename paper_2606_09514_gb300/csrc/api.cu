@@ -282,7 +282,7 @@ extern "C" int buddy_get_paths(buddy_ctx* ctx, int32_t* paths, int32_t n) {
   const Ctx& c = ctx->c;
   if (!c.have_weights) return BUDDY_ERR_STATE;
   const int32_t v[4] = {c.use_tc ? 1 : 0, attention_cl(c) ? 2 : (attention_tc(c) ? 1 : 0),
-                        (c.use_tc && c.tc_panel) ? 1 : 0,
+                        (c.use_tc ? c.tc_panel : c.maxB <= kSimtFuseRows) ? 1 : 0,
                         (c.use_tc && c.tc_defer) ? 1 : 0};
   for (int i = 0; i < n; ++i) paths[i] = v[i];
   return BUDDY_OK;
@@ -368,7 +368,7 @@ static GemmArgs qkv_args(const Ctx& c, const buddy_kv_state& kv, int l, RowSel s
   // the value-state feature is pooled with the QKV finalisation of the
   // context layer, the other features by launch_pool_update
   g.pool = (l == c.cl && c.feature == BUDDY_FEATURE_V) ? kv.pool_sum : nullptr;
-  if (c.use_tc) {
+  if (c.use_tc || panel) {
     // bias, RoPE, q, cache append and pool update in the GEMM epilogue
     g.qkv_bias = W.b_qkv; g.kv_len = kv.len; g.kv_seq_off = kv.seq_off; g.kv_cap = kv.cap;
     g.cache_len = cache_len(c, kv, l);
@@ -419,7 +419,7 @@ static void enqueue_layer(Ctx& c, const buddy_kv_state& kv, int l, RowSel sel, c
                           float* H, cudaStream_t s, bool prof) {
   const buddy_layer_weights& W = c.layers[l];
   const bool split = c.split0 && l <= c.cl;
-  const bool panel = c.use_tc && c.tc_panel;
+  const bool panel = c.use_tc ? c.tc_panel : sel.n <= kSimtFuseRows;   // the GEMMs normalise their own input
   if (!panel) {
     ProfScope p(c, s, BUDDY_PROF_RMSNORM, 1, prof);
     launch_rmsnorm(c, src, sel, W.attn_norm, c.xn, split ? c.xn_lo : nullptr, s);
@@ -428,7 +428,7 @@ static void enqueue_layer(Ctx& c, const buddy_kv_state& kv, int l, RowSel sel, c
   // no RMSNorm kernel in between: the first middle layer's QKV GEMM follows
   // the compaction kernel that writes its row count
   g.count_late = panel && l == c.cl + 1;
-  if (c.use_tc) {
+  if (c.use_tc || panel) {
     run_gemm(c, EPI_QKV, g, l, 0, s, BUDDY_PROF_GEMM_QKV, prof);
   } else {
     run_gemm(c, EPI_STORE_F32, g, l, 0, s, BUDDY_PROF_GEMM_QKV, prof);

@@ -16,6 +16,7 @@ namespace buddy {
 constexpr int kMaxLayers = 128;
 constexpr int kRouteZSlots = 32;  // K-split slots of the router's hidden-unit partial sums
 constexpr int kMaxBatch = 1024;
+constexpr int kSimtFuseRows = 24;  // fp32: rows up to which the GEMMs take in the norms and the QKV finalisation
 
 // Per-layer K/V base pointers passed by value to kernels that touch many layers.
 struct LayerPtrs {
@@ -48,7 +49,7 @@ struct GemmArgs {
   bool split;
   const float* resid_src; // EPI_RESID: dst[i] = src[i] + acc  (may equal dst)
   float* resid_dst;
-  // EPI_QKV (tensor-core path): QKV finalisation fused into the epilogue
+  // EPI_QKV: QKV finalisation fused into the epilogue
   const float* qkv_bias;
   const int32_t* kv_len;       // RoPE positions (tokens of each sequence)
   const int32_t* cache_len;    // where the layer's cache stores the new entry
@@ -61,8 +62,8 @@ struct GemmArgs {
   const int32_t* status;
   int layer;              // tensor-core path: which layer's weight map
   int which;              // 0 qkv, 1 o, 2 gate_up, 3 down
-  // tensor-core path, small batches: X = RMSNorm(in_norm_src[rows]) computed
-  // inside the GEMM (panel mode; X and X_lo unused)
+  // small batches: X = RMSNorm(in_norm_src[rows]) computed inside the GEMM (X
+  // and X_lo unused)
   const float* in_norm_src;
   const float* in_norm_gamma;
   bool count_late;        // the kernel enqueued just before wrote *sel.count

@@ -205,16 +205,16 @@ void launch_rmsnorm(const Ctx& c, const float* H, RowSel sel, const float* gamma
 }
 
 // ---------------------------------------------------------------------------
-// QKV finalisation for one layer: bias, rotate-half RoPE at position len[i],
+// QKV finalisation for one layer of an fp32 model (more than kSimtFuseRows rows;
+// elsewhere the QKV GEMM's epilogue does it): bias, rotate-half RoPE at position len[i],
 // q kept in fp32, K/V stored (config dtype) at position len[i] of the cache,
 // and for the first layer the pooled-context running sum += stored V.
 // ---------------------------------------------------------------------------
-template <typename T>
 __global__ void __launch_bounds__(256) qkv_finalize_kernel(
     const float* __restrict__ qkv, const float* __restrict__ bias, const int32_t* rows,
     const int32_t* count, int n, int nq, int nkv, int hd, const float* __restrict__ rc,
     const float* __restrict__ rs, const int32_t* len, const int32_t* cache_len, const int64_t* seq_off,
-    const int32_t* cap, T* Kc, T* Vc, float* __restrict__ q_out, float* pool, const int32_t* status) {
+    const int32_t* cap, float* Kc, float* Vc, float* __restrict__ q_out, float* pool, const int32_t* status) {
   pdl_wait();
   pdl_trigger();
   if (call_aborted(status)) return;
@@ -245,9 +245,9 @@ __global__ void __launch_bounds__(256) qkv_finalize_kernel(
       q_out[(size_t)j * nq * hd + c0 + half] = y2;
     } else {
       const int g = head - nq;
-      T* kp = Kc + kv_offset(seq_off, cap, i, nkv, hd, g, cpos);
-      kp[e] = from_f<T>(y1);
-      kp[e + half] = from_f<T>(y2);
+      float* kp = Kc + kv_offset(seq_off, cap, i, nkv, hd, g, cpos);
+      kp[e] = y1;
+      kp[e + half] = y2;
     }
   }
   const int vbase = (nq + nkv) * hd;
@@ -255,9 +255,8 @@ __global__ void __launch_bounds__(256) qkv_finalize_kernel(
     const int g = t / hd, e = t - g * hd;
     float v = x[vbase + t];
     if (bias) v += bias[vbase + t];
-    const T vs = from_f<T>(v);
-    Vc[kv_offset(seq_off, cap, i, nkv, hd, g, cpos) + e] = vs;
-    if (pool) pool[(size_t)i * nkv * hd + t] += to_f(vs);
+    Vc[kv_offset(seq_off, cap, i, nkv, hd, g, cpos) + e] = v;
+    if (pool) pool[(size_t)i * nkv * hd + t] += v;
   }
 }
 
@@ -265,16 +264,9 @@ void launch_qkv_finalize(const Ctx& c, const float* qkv, const float* bias, RowS
                          const buddy_kv_state& kv, int layer, float* q_out, float* pool,
                          cudaStream_t s) {
   const int32_t* cl = cache_len(c, kv, layer);
-  if (c.dtype == BUDDY_DTYPE_BF16)
-    launch_k(qkv_finalize_kernel<bf16>, sel.n, 256, 0, s, c.pdl,
-             qkv, bias, sel.rows, sel.count, sel.n, c.nq, c.nkv, c.hd, (const float*)c.rope_cos,
-             (const float*)c.rope_sin, (const int32_t*)kv.len, cl, kv.seq_off, kv.cap, (bf16*)kv.k_cache[layer],
-             (bf16*)kv.v_cache[layer], q_out, pool, (const int32_t*)c.status);
-  else
-    launch_k(qkv_finalize_kernel<float>, sel.n, 256, 0, s, c.pdl,
-             qkv, bias, sel.rows, sel.count, sel.n, c.nq, c.nkv, c.hd, (const float*)c.rope_cos,
-             (const float*)c.rope_sin, (const int32_t*)kv.len, cl, kv.seq_off, kv.cap, (float*)kv.k_cache[layer],
-             (float*)kv.v_cache[layer], q_out, pool, (const int32_t*)c.status);
+  launch_k(qkv_finalize_kernel, sel.n, 256, 0, s, c.pdl, qkv, bias, sel.rows, sel.count, sel.n, c.nq, c.nkv, c.hd,
+           (const float*)c.rope_cos, (const float*)c.rope_sin, (const int32_t*)kv.len, cl, kv.seq_off, kv.cap,
+           (float*)kv.k_cache[layer], (float*)kv.v_cache[layer], q_out, pool, (const int32_t*)c.status);
 }
 
 // ---------------------------------------------------------------------------
