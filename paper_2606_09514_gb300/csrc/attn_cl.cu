@@ -4,8 +4,8 @@
 // At a few rows the streams are few (batch 1 of an 8-KV-head model: 8
 // streams of ~2k positions) and short: cutting them across the whole GPU
 // leaves tens of partial results per stream whose merge costs as much as the
-// streaming.  Here a cluster of C CTAs (C = 16 where the device allows it,
-// else 8) takes one stream: CTA r streams positions [r np / C, (r+1) np / C)
+// streaming.  Here a cluster of C CTAs (cl_size: the largest of 16, 8, 4 and 2
+// of which all streams' clusters fit on the GPU at once) takes one stream: CTA r streams positions [r np / C, (r+1) np / C)
 // with its 4 warps (contiguous quarters, 32-position chunks through a
 // 2-buffer cp.async ring per warp; the contractions are those of the
 // tensor-core loop in attn_tc.cuh: S^T = K Q^T and O^T += V^T P^T on
@@ -44,11 +44,11 @@ __host__ __device__ constexpr size_t attn_cl_bufs() {
   // per warp: kClStages buffers of K and V rows (padded by 8 bf16)
   return (size_t)kClWarps * kClStages * 2 * kClChunk * (HD + 8) * 2;
 }
-// One partial in an owner's gather area: m[8], l[8], then the owner's slice
-// of outputs (at most 8 heads x HD channels / 8 CTAs).
+// The gather area of a CTA: for each of the C CTAs of the cluster a partial of
+// m[8], l[8] and the owner's slice of outputs (at most 8 heads x HD channels / C).
 template <int HD>
-__host__ __device__ constexpr int attn_cl_gstride() {
-  return 16 + HD;
+__host__ __device__ constexpr size_t attn_cl_gather() {
+  return (size_t)(kClMaxCtas * 16 + 8 * HD) * 4;
 }
 template <int HD>
 __host__ __device__ constexpr size_t attn_cl_smem() {
@@ -56,8 +56,7 @@ __host__ __device__ constexpr size_t attn_cl_smem() {
   // buffers once the streaming is done; then the gather area, one partial
   // per CTA of the cluster
   const size_t parts = (size_t)kClWarps * 8 * (HD + 2) * 4;
-  return (attn_cl_bufs<HD>() > parts ? attn_cl_bufs<HD>() : parts) +
-         (size_t)kClMaxCtas * attn_cl_gstride<HD>() * 4;
+  return (attn_cl_bufs<HD>() > parts ? attn_cl_bufs<HD>() : parts) + attn_cl_gather<HD>();
 }
 
 __device__ __forceinline__ void st_dsmem(uint32_t addr, float v) {
@@ -99,8 +98,9 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
   bf16* wbuf = reinterpret_cast<bf16*>(smraw) + (size_t)warp * NST * 2 * CH * KROW;
   float* parts = reinterpret_cast<float*>(smraw);   // overlays the buffers after the streaming
   float* mine = parts + (size_t)warp * PSTRIDE;
-  constexpr int GS = attn_cl_gstride<HD>();
-  constexpr size_t kBufBytes = attn_cl_smem<HD>() - (size_t)kClMaxCtas * GS * 4;
+  const int SL = (G * HD + (int)C - 1) / (int)C;   // outputs per owner
+  const int GS = 16 + SL;                          // floats of one partial in the gather area
+  constexpr size_t kBufBytes = attn_cl_smem<HD>() - attn_cl_gather<HD>();
   float* gather = reinterpret_cast<float*>(smraw + kBufBytes);   // one partial per CTA of the cluster
 
   auto issue = [&](int p, int cnt, int buf) {
@@ -314,8 +314,7 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
   // the CTA's partial, the warps' partials merged per (head, channel), stored
   // into the gather area of the output's owner (slot `rank`), four channels
   // per thread and per 16-byte store (a slice is a multiple of 4 outputs:
-  // G * HD is a multiple of 64 and C is 8 or 16)
-  const int SL = (G * HD + (int)C - 1) / (int)C;   // outputs per owner (<= HD for C >= 8)
+  // G * HD is a multiple of 64 and C at most 16)
   for (int x = tid * 4; x < G * HD; x += kClThreads * 4) {
     const int hh = x / HD, ch = x - hh * HD;
     float M = -INFINITY;
@@ -368,20 +367,22 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
   }
 }
 
-// Clusters of C CTAs the device can hold at once (C = 16 and 8), queried
-// once per instantiation; 0 where the size cannot be scheduled.
+// Clusters of 16, 8, 4 and 2 CTAs the device can hold at once, queried once per
+// instantiation; 0 where the size cannot be scheduled.
+constexpr int kClSizes = 4;
 template <int HD, bool SPLIT>
 static const int* cl_capacity() {
-  static int cap[2] = {-1, -1};   // [0]: C = 16, [1]: C = 8
-  if (cap[0] >= 0) return cap;
+  static int cap[kClSizes] = {-1, -1, -1, -1};   // [v]: C = 16 >> v
+  if (cap[kClSizes - 1] >= 0) return cap;
   const size_t smem = attn_cl_smem<HD>();
   cudaFuncSetAttribute(attn_cl_kernel<HD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  for (int v = 0; v < 2; ++v) {
-    const int C = v == 0 ? kClMaxCtas : 8;
-    cap[v] = 0;
+  for (int v = 0; v < kClSizes; ++v) {
+    const int C = kClMaxCtas >> v;
+    int n = 0;
     if (C > 8 && cudaFuncSetAttribute(attn_cl_kernel<HD, SPLIT>, cudaFuncAttributeNonPortableClusterSizeAllowed,
                                       1) != cudaSuccess) {
       cudaGetLastError();
+      cap[v] = 0;
       continue;
     }
     cudaLaunchConfig_t cfg = {};
@@ -395,21 +396,27 @@ static const int* cl_capacity() {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_cl_kernel<HD, SPLIT>, &cfg) == cudaSuccess) cap[v] = n;
+    if (cudaOccupancyMaxActiveClusters(&n, attn_cl_kernel<HD, SPLIT>, &cfg) != cudaSuccess) n = 0;
     cudaGetLastError();
+    cap[v] = n;
   }
   return cap;
 }
 
-// Cluster size for `streams` streams: 16 CTAs when every cluster fits at
-// once (a cluster that waits for another to finish doubles the latency),
-// else 8; 0 if neither size can be scheduled.
+// Cluster size for `streams` streams: the largest of which every stream's cluster
+// fits at once (a cluster that waits for others to finish starts its stream when
+// they have ended theirs: 56 streams of 970 positions take 21 us a block in three
+// waves of 8-CTA clusters, 12 us in one of 2-CTA clusters); else the smallest
+// that can be scheduled, 0 if none can.
 template <int HD, bool SPLIT>
 static int cl_size(int streams) {
   const int* cap = cl_capacity<HD, SPLIT>();
-  if (cap[0] > 0 && (streams <= cap[0] || cap[1] <= 0)) return kClMaxCtas;
-  return cap[1] > 0 ? 8 : 0;
+  int last = 0;
+  for (int v = 0; v < kClSizes; ++v) {
+    if (cap[v] > 0) last = kClMaxCtas >> v;
+    if (cap[v] >= streams) return last;
+  }
+  return last;
 }
 
 bool attention_cl(const Ctx& c) {

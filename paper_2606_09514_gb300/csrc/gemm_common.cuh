@@ -185,27 +185,45 @@ __device__ __forceinline__ void tc_mma_stage(const uint8_t* st, uint32_t d, cons
 // following 15 KiB (later blocks, the next panel, or the tail slack): those
 // rows only feed accumulator rows that are discarded.
 // ---------------------------------------------------------------------------
-// 1 / rms of each row (m <= 8), by the 128 epilogue threads (et = 0..127).
-__device__ __forceinline__ void tc_panel_inv(const TcParams& p, int m, int et, float* red, float* inv) {
+// 1 / rms of each row (m <= 8), by the 128 epilogue threads (et = 0..127): four
+// rows at a time, eight float4 of each per thread in flight together (a row at a
+// time took 7 us for 7 rows of 4096).  A function of its own, so that the kernel
+// of one or two rows, which does not call it, stays short.
+static __device__ __noinline__ void tc_panel_inv(const float* nsrc, int K, float neps, int m, int et,
+                                                 const int* row_of, float* red, float* inv) {
+  constexpr int RG = 4, KQ = 8;
   const int lane = et & 31, w = et >> 5;
-  for (int j = 0; j < m; ++j) {
-    const float* h = p.nsrc + (size_t)(p.rows ? p.rows[j] : j) * p.K;
-    float ss = 0.f;
-    for (int e0 = 0; e0 < p.K; e0 += 16 * 512) {
-      float4 x[16];
+#pragma unroll 1
+  for (int j0 = 0; j0 < m; j0 += RG) {
+    float ss[RG];
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const int e = e0 + (et + k * 128) * 4;
-        x[k] = e < p.K ? *reinterpret_cast<const float4*>(h + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r = 0; r < RG; ++r) ss[r] = 0.f;
+#pragma unroll 1
+    for (int e0 = 0; e0 < K; e0 += KQ * 512) {
+      float4 x[RG][KQ];
+#pragma unroll
+      for (int r = 0; r < RG; ++r) {
+        const float* h = nsrc + (size_t)row_of[min(j0 + r, m - 1)] * K;
+#pragma unroll
+        for (int k = 0; k < KQ; ++k) {
+          const int e = e0 + (et + k * 128) * 4;
+          x[r][k] = e < K ? *reinterpret_cast<const float4*>(h + e) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       }
 #pragma unroll
-      for (int k = 0; k < 16; ++k) ss += x[k].x * x[k].x + x[k].y * x[k].y + x[k].z * x[k].z + x[k].w * x[k].w;
+      for (int r = 0; r < RG; ++r)
+#pragma unroll
+        for (int k = 0; k < KQ; ++k)
+          ss[r] += x[r][k].x * x[r][k].x + x[r][k].y * x[r][k].y + x[r][k].z * x[r][k].z + x[r][k].w * x[r][k].w;
     }
-    ss = warp_sum(ss);
-    if (lane == 0) red[j * 4 + w] = ss;
+#pragma unroll
+    for (int r = 0; r < RG; ++r) {
+      const float s = warp_sum(ss[r]);
+      if (lane == 0 && j0 + r < m) red[(j0 + r) * 4 + w] = s;
+    }
   }
   epi_bar();
-  if (et < m) inv[et] = rsqrtf(((red[et * 4] + red[et * 4 + 1]) + (red[et * 4 + 2] + red[et * 4 + 3])) / (float)p.K + p.neps);
+  if (et < m) inv[et] = rsqrtf(((red[et * 4] + red[et * 4 + 1]) + (red[et * 4 + 2] + red[et * 4 + 3])) / (float)K + neps);
   epi_bar();
 }
 
@@ -261,8 +279,8 @@ __device__ __forceinline__ void tc_panel_write(const TcParams& p, uint8_t* panel
 // 512 columns, 16 per thread).
 constexpr int kPanelFirstMaxK = 16 * 512;
 
-// The first unit's panel in one pass over each row: every thread loads its
-// 16 float4 of row j (the loads of the sum of squares), the sum is reduced
+// The first unit's panel of one or two rows in one pass over each: every thread loads
+// its 16 float4 of a row (the loads of the sum of squares), the sum is reduced
 // across the 4 epilogue warps, and the thread then writes the panel entries
 // of the unit's K range [kb0, kb1) that it already holds, scaled by 1 / rms
 // and by the gains staged in shared memory (gst, from column kb0 * 64).  The

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
       }
     }
   }
-  const bool panel = !DEFER && p.nsrc != nullptr;
+  const bool panel = !DEFER && EPI != EPI_RESID && p.nsrc != nullptr;
   const bool first_pass = panel && p.K <= kPanelFirstMaxK;
   if (first_pass && warp >= 2 && blockIdx.x < p.units) {
     // Before the wait: the RMSNorm gains of the first unit's K range (weights,
@@ -255,12 +255,13 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
       // the first unit's panel (and the norm of every row)
       const int split = blockIdx.x / p.n_tiles;
       const int kb0 = split * p.kb_per_split, kb1 = min(p.kb_total, kb0 + p.kb_per_split);
-      if (first_pass) {
-        epi_bar();   // staged gains and rows visible to all epilogue warps
+      if (!first_pass && et < m) prow[et] = p.rows ? p.rows[et] : et;
+      epi_bar();   // staged gains and rows visible to all epilogue warps
+      if (first_pass && m <= 2) {
         tc_panel_first<SPLIT>(p, smem + p.panel_off, m, kb0, kb1, et, prow,
                               reinterpret_cast<const float*>(smem + p.gstage_off), pred, pinv);
       } else {
-        tc_panel_inv(p, m, et, pred, pinv);
+        tc_panel_inv(p.nsrc, p.K, p.neps, m, et, prow, pred, pinv);
         tc_panel_write<SPLIT>(p, smem + p.panel_off, m, kb0, kb1, et, pinv);
       }
       epi_bar();
