@@ -32,8 +32,8 @@ namespace buddy {
 // accumulator, so the product carries ~16 mantissa bits of the activations.
 // DEFER (more than kTcDeferRows rows): the units only stage their partials, a
 // second kernel (gemm_fix_kernel) sums the splits and applies the epilogue on
-// every SM; without it (up to that many rows) the kernel can run in panel mode
-// and the last split of a tile applies the epilogue.
+// every SM; without it (up to that many rows) the QKV and gate/up GEMMs run in
+// panel mode and the last split of a tile applies the epilogue.
 template <int EPI, bool SPLIT, bool DEFER>
 __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ XMaps tx,
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
     consumed = 0;
     ptx::fence_mbar_init();
     ptx::tma_prefetch_desc(&tw);
-    if (DEFER || !p.nsrc)
+    if (DEFER || EPI == EPI_RESID)
       for (int b = 0; b < 4; ++b) {
         ptx::tma_prefetch_desc(&tx.box[b]);
         if (SPLIT) ptx::tma_prefetch_desc(&txlo.box[b]);
@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
       }
     }
   }
-  const bool panel = !DEFER && EPI != EPI_RESID && p.nsrc != nullptr;
+  constexpr bool panel = !DEFER && EPI != EPI_RESID;
   const bool first_pass = panel && p.K <= kPanelFirstMaxK;
   if (first_pass && warp >= 2 && blockIdx.x < p.units) {
     // Before the wait: the RMSNorm gains of the first unit's K range (weights,
@@ -493,10 +493,10 @@ int gemm_tc_prepare(Ctx& c) {
       if (c.tc_pstages[v] < 3) c.tc_panel = false;
     }
   }
-  // Above kTcDeferRows rows a tile's partials are too many for the one CTA
-  // that would finish it (m x 256 fp32 per split): a fixup kernel spreads
-  // them over all SMs.
-  c.tc_defer = c.maxB > kTcDeferRows;
+  // Above kTcDeferRows rows a tile's partials are too many for the one CTA that
+  // would finish it (m x 256 fp32 per split): a fixup kernel spreads them over
+  // all SMs.  So does it where the panels do not fit.
+  c.tc_defer = c.maxB > kTcDeferRows || !c.tc_panel;
   if (c.pf_max > 0) {
     // prefill weights and activations: 128-row boxes (one CTA's part of a tile)
     c.pf_wmaps.assign((size_t)c.L * 4, CUtensorMap{});
