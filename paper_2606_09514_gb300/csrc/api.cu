@@ -621,10 +621,7 @@ extern "C" int buddy_route(buddy_ctx* ctx, const buddy_kv_state* kv, int32_t bat
   if (!kv || !kv->len || !kv->pool_sum || !kv->cap || kv->batch < batch) return BUDDY_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   // positions: the cache already holds the newest token (len >= 1)
-  buddy_kv_state kvc = *kv;
-  kvc.layer_len = nullptr;   // only the context layer's pool and len are read
-  launch_step_check(c, batch, k, kvc, 0, c.status, s);
-  launch_route(c, batch, h1, kv->pool_sum, kv->len, 0, k, mask_out, sel_out, scores_out, s);
+  launch_route(c, batch, h1, kv->pool_sum, kv->len, 0, k, mask_out, sel_out, scores_out, s, kv);
   CK(cudaGetLastError());
   return BUDDY_OK;
 }
@@ -642,8 +639,7 @@ extern "C" int buddy_kv_append(buddy_ctx* ctx, const buddy_kv_state* kv, int32_t
   if (rc) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   int32_t* base = const_cast<int32_t*>(cache_len(c, *kv, layer));
-  launch_kv_check(c, n_seq, seq_ids, n_new, kv->batch, base, kv->cap, c.status, s);
-  if (n_new > 0) launch_kv_append(c, *kv, layer, n_seq, seq_ids, n_new, k_new, v_new, s);
+  launch_kv_append(c, *kv, layer, n_seq, seq_ids, n_new, k_new, v_new, s);
   if (layer == c.cl) launch_pool_refresh(c, *kv, n_seq, seq_ids, n_new, s);
   // the masked variant's per-layer length grows with its own appends
   if (c.masked && n_new > 0) launch_advance(c, n_seq, base, n_new, seq_ids, s);

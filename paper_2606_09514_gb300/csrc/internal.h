@@ -95,6 +95,18 @@ struct PfEpi {
   void* vc;
 };
 
+// Device checks a kernel can make by itself, in every CTA, instead of a check
+// kernel before it (few sequences: a few loads against a launch).  `out` != null:
+// make them, and CTA 0 publishes the call's abort word in out[1] and the error
+// bits in out[0].
+struct RouteCheck {
+  const int32_t* k;      // budgets
+  const int32_t* len;
+  const int32_t* cap;
+  int B, Lm, k_min, max_pos;
+  int32_t* out;
+};
+
 // Launch with programmatic stream serialisation when `pdl` is set (the kernel
 // then overlaps its prologue with the predecessor and synchronises with
 // pdl_wait()).
@@ -135,12 +147,13 @@ void launch_attention_cl(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int
 cudaError_t route_prepare();
 void launch_route(const Ctx& c, int B, const float* h1, const float* pool, const int32_t* len,
                   int len_bias, const int32_t* k, uint8_t* mask, int32_t* sel, float* scores,
-                  cudaStream_t s);
+                  cudaStream_t s, const buddy_kv_state* check_kv = nullptr);   // check_kv: make the call's checks too
 void launch_compact(const Ctx& c, int B, const uint8_t* mask, const buddy_kv_state& kv,
                     int32_t* rows, int32_t* count, cudaStream_t s);
 void launch_advance(const Ctx& c, int B, int32_t* len, int by, const int32_t* seq_ids, cudaStream_t s,
                     const uint8_t* mask = nullptr, int32_t* layer_len = nullptr, int kv_batch = 0);
 void launch_pool_update(const Ctx& c, int B, const buddy_kv_state& kv, cudaStream_t s);
+// Makes the call's device checks and copies the given entries.
 void launch_kv_append(const Ctx& c, const buddy_kv_state& kv, int layer, int n_seq,
                       const int32_t* seq_ids, int n_new, const void* k_new, const void* v_new,
                       cudaStream_t s);

@@ -57,10 +57,7 @@ __global__ void step_check_kernel(int B, const int32_t* k, int Lm, int k_min, co
   }
   if (b) atomicOr(&bad, b);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    status[1] = bad ? 1 : 0;
-    if (bad) atomicOr(status, bad);
-  }
+  if (threadIdx.x == 0) publish_checks(status, bad);
 }
 
 void launch_step_check(const Ctx& c, int B, const int32_t* k, const buddy_kv_state& kv, int extra,
@@ -90,10 +87,7 @@ __global__ void kv_check_kernel(int n_seq, const int32_t* ids, int n_new, int ba
   }
   if (b) atomicOr(&bad, b);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    status[1] = bad ? 1 : 0;
-    if (bad) atomicOr(status, bad);
-  }
+  if (threadIdx.x == 0) publish_checks(status, bad);
 }
 
 void launch_kv_check(const Ctx& c, int n_seq, const int32_t* ids, int n_new, int batch,
@@ -318,6 +312,20 @@ void launch_pool_update(const Ctx& c, int B, const buddy_kv_state& kv, cudaStrea
 // (route_gemm_kernel): a tiled fp32 GEMM whose K splits leave
 // partial sums that part 2 adds in split order.
 // ---------------------------------------------------------------------------
+// The checks of a routing call, by every CTA: whether any failed.
+__device__ __forceinline__ bool route_check(const RouteCheck& c) {
+  int b = 0;
+  for (int i = threadIdx.x; i < c.B; i += blockDim.x) {
+    const int ki = c.k[i], n = c.len[i];
+    if (ki < c.k_min || ki > c.Lm) b |= BUDDY_DEV_BAD_BUDGET;
+    if (n < 0 || n > c.cap[i] || n > c.max_pos) b |= BUDDY_DEV_BAD_POSITION;
+  }
+  const int bad = (__syncthreads_or(b & BUDDY_DEV_BAD_BUDGET) ? BUDDY_DEV_BAD_BUDGET : 0) |
+                  (__syncthreads_or(b & BUDDY_DEV_BAD_POSITION) ? BUDDY_DEV_BAD_POSITION : 0);
+  if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) publish_checks(c.out, bad);
+  return bad != 0;
+}
+
 constexpr int kRouteRows = 8;
 constexpr int kRouteTiledMin = 16;    // batches above this take the tiled router GEMM
 constexpr int kRtBM = 64, kRtBN = 64, kRtBK = 32;
@@ -328,10 +336,10 @@ __global__ void __launch_bounds__(256) route_hidden_kernel(
     int B, int d, int hd, int group, int nkv, const float* __restrict__ h1,
     const float* __restrict__ pool, const int32_t* len, int len_bias, const float* __restrict__ w1,
     const float* __restrict__ b1, int r, const float* __restrict__ pw1, const float* __restrict__ pb1, int rp,
-    float* __restrict__ u, const int32_t* status) {
+    float* __restrict__ u, const int32_t* status, const RouteCheck chk) {
   pdl_wait();
   pdl_trigger();
-  if (call_aborted(status)) return;
+  if (chk.out ? route_check(chk) : call_aborted(status)) return;
   __shared__ float red[8][kRouteRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = blockIdx.x;
@@ -599,7 +607,17 @@ cudaError_t route_prepare() {
 
 void launch_route(const Ctx& c, int B, const float* h1, const float* pool, const int32_t* len,
                   int len_bias, const int32_t* k, uint8_t* mask, int32_t* sel, float* scores,
-                  cudaStream_t s) {
+                  cudaStream_t s, const buddy_kv_state* check_kv) {
+  // the call's checks: by the small-batch kernel itself, else by a kernel before
+  // the GEMM (checking in its 288 CTAs made 250 rows 15 us slower)
+  RouteCheck chk{};
+  if (check_kv && B <= kRouteTiledMin) {
+    chk = RouteCheck{k, len, check_kv->cap, B, c.Lm, c.have_pred ? 0 : 1, c.max_pos, c.status};
+  } else if (check_kv) {
+    buddy_kv_state kvc = *check_kv;
+    kvc.layer_len = nullptr;   // only the context layer's pool and len are read
+    launch_step_check(c, B, k, kvc, 0, c.status, s);
+  }
   const int rp = c.have_pred ? c.pred.hidden : 0;
   const int cols = c.r + rp;
   const int splits = route_splits(c, B);
@@ -607,7 +625,7 @@ void launch_route(const Ctx& c, int B, const float* h1, const float* pool, const
     dim3 g1(cols, (B + kRouteRows - 1) / kRouteRows);
     launch_k(route_hidden_kernel, g1, 256, 0, s, c.pdl, B, c.d, c.hd, c.nq / c.nkv, c.nkv, h1, pool, len,
              len_bias, c.dm.w1, c.dm.b1, c.r, c.have_pred ? c.pred.w1 : nullptr, c.have_pred ? c.pred.b1 : nullptr,
-             rp, c.dm_u, (const int32_t*)c.status);
+             rp, c.dm_u, (const int32_t*)c.status, chk);
   } else {
     const int half = splits / 2;
     const int kps = ((c.d + half - 1) / half + kRtBK - 1) / kRtBK * kRtBK;
@@ -776,14 +794,31 @@ __global__ void __launch_bounds__(256) kv_append_kernel(int n_new, int nkv, int 
 // Used when the given arrays are 16-byte aligned (the caches always are).
 constexpr int kAppendPos = 8;
 template <typename T>
-__global__ void __launch_bounds__(256) kv_append_vec_kernel(int n_new, int nkv, int hd, const int32_t* ids,
+__global__ void __launch_bounds__(256) kv_append_vec_kernel(int n_new, int nkv, int hd, int n_seq, const int32_t* ids,
                                                             const int32_t* len, const int64_t* seq_off,
                                                             const int32_t* cap, const T* __restrict__ kn,
-                                                            const T* __restrict__ vn, T* Kc, T* Vc,
-                                                            const int32_t* status) {
+                                                            const T* __restrict__ vn, T* Kc, T* Vc, int batch,
+                                                            int max_pos, int32_t* status, bool check) {
   pdl_wait();
   pdl_trigger();
-  if (call_aborted(status)) return;
+  if (check) {   // the call's checks, by every CTA (kv_check_kernel's)
+    int b = 0;
+    if (threadIdx.x < n_seq) {
+      const int s = ids[threadIdx.x];
+      if (s < 0 || s >= batch) {
+        b = BUDDY_DEV_BAD_SEQ;
+      } else {
+        const int n = len[s];
+        if (n < 0 || n + n_new > cap[s] || n + n_new > max_pos) b = BUDDY_DEV_BAD_POSITION;
+      }
+    }
+    const int bad = (__syncthreads_or(b & BUDDY_DEV_BAD_SEQ) ? BUDDY_DEV_BAD_SEQ : 0) |
+                    (__syncthreads_or(b & BUDDY_DEV_BAD_POSITION) ? BUDDY_DEV_BAD_POSITION : 0);
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) publish_checks(status, bad);
+    if (bad) return;
+  } else if (call_aborted(status)) {
+    return;
+  }
   constexpr int E = 16 / sizeof(T), U = 4;
   const int t0 = blockIdx.x * kAppendPos, jj = blockIdx.y;
   const int s = ids[jj];
@@ -895,11 +930,15 @@ static void kv_append_impl(const Ctx& c, const buddy_kv_state& kv, int layer, in
   const int32_t* base = cache_len(c, kv, layer);
   T* kc = (T*)kv.k_cache[layer];
   T* vc = (T*)kv.v_cache[layer];
-  if (((reinterpret_cast<uintptr_t>(kn) | reinterpret_cast<uintptr_t>(vn)) & 15u) == 0) {
+  const bool vec = n_new > 0 && ((reinterpret_cast<uintptr_t>(kn) | reinterpret_cast<uintptr_t>(vn)) & 15u) == 0;
+  // up to 256 sequences a thread of every CTA checks one: no check kernel before
+  const bool inside = vec && n_seq <= 256;
+  if (!inside) launch_kv_check(c, n_seq, ids, n_new, kv.batch, base, kv.cap, c.status, s);
+  if (vec) {
     const dim3 g((n_new + kAppendPos - 1) / kAppendPos, n_seq);
-    launch_k(kv_append_vec_kernel<T>, g, 256, 0, s, c.pdl, n_new, c.nkv, c.hd, ids, base, kv.seq_off, kv.cap,
-             (const T*)kn, (const T*)vn, kc, vc, (const int32_t*)c.status);
-  } else {
+    launch_k(kv_append_vec_kernel<T>, g, 256, 0, s, c.pdl, n_new, c.nkv, c.hd, n_seq, ids, base, kv.seq_off, kv.cap,
+             (const T*)kn, (const T*)vn, kc, vc, kv.batch, c.max_pos, c.status, inside);
+  } else if (n_new > 0) {
     const dim3 g(n_new, n_seq);
     launch_k(kv_append_kernel<T>, g, 256, 0, s, c.pdl, n_new, c.nkv, c.hd, ids, base, kv.seq_off, kv.cap,
              (const T*)kn, (const T*)vn, kc, vc, (const int32_t*)c.status);
