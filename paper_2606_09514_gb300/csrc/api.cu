@@ -56,7 +56,7 @@ static void free_ctx(buddy_ctx* x) {
                   c.attn_m, c.attn_l, c.attn_acc, c.attn_ctr, c.dm_u, c.mask, c.sel, c.scores, c.rows,
                   c.count, c.h_in_stage, c.h_out_stage, c.k_stage, c.mask_stage, c.xn_lo, c.act_lo, c.attn_lo,
                   c.gemm_ws, c.gemm_ctr, c.pf_xn, c.pf_xn_lo, c.pf_q, c.pf_attn, c.pf_attn_lo,
-                  c.pf_act, c.pf_act_lo, c.pf_tok_seq, c.pf_tok_t, c.pf_tok_pos, c.pf_rows, c.pf_items,
+                  c.pf_act, c.pf_act_lo, c.pf_tok_seq, c.pf_tok_t, c.pf_tok_pos, c.pf_tok_off, c.pf_tok_cap, c.pf_rows, c.pf_items,
                   c.pf_n_tok, c.pf_tok_end, c.pf_cnt, c.pf_hlast, c.pf_ws, c.pf_ctr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -157,7 +157,8 @@ extern "C" int buddy_create(const buddy_config* cfg, buddy_ctx** out) {
         (e = dalloc(&c.pf_q, T * c.qd)) || (e = cudaMalloc(&c.pf_attn, T * c.qd * c.esz)) ||
         (e = cudaMalloc(&c.pf_attn_lo, T * c.qd * c.esz)) || (e = cudaMalloc(&c.pf_act, T * c.F * c.esz)) ||
         (e = cudaMalloc(&c.pf_act_lo, T * c.F * c.esz)) || (e = dalloc(&c.pf_tok_seq, T)) ||
-        (e = dalloc(&c.pf_tok_t, T)) || (e = dalloc(&c.pf_tok_pos, T)) ||
+        (e = dalloc(&c.pf_tok_t, T)) || (e = dalloc(&c.pf_tok_pos, T)) || (e = dalloc(&c.pf_tok_off, T)) ||
+        (e = dalloc(&c.pf_tok_cap, T)) ||
         (e = dalloc(&c.pf_rows, (size_t)c.L * T)) ||
         (e = dalloc(&c.pf_items, (size_t)(c.L + 1) * c.pf_items_max)) || (e = dalloc(&c.pf_n_tok, B)) ||
         (e = dalloc(&c.pf_tok_end, B)) || (e = dalloc(&c.pf_cnt, B)) || (e = dalloc(&c.pf_hlast, B * c.d)))

@@ -715,6 +715,13 @@ int gemm_pf_prepare(Ctx& c) {
 // 1 attention output, 2 SwiGLU output); m rows.
 void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
                     cudaStream_t s) {
+  // Few tokens are bound by the weight stream: the decode GEMM (one CTA per weight
+  // tile and K split, a fixup over the whole GPU) beats pairs that each hold an
+  // M-tile mostly empty and sum their parts alone: 4 blocks of Llama-3-8B, 61 tokens
+  // 594 -> 461 us, 256 tokens 862 -> 802 us; Llama-2-13B, 240 tokens 1097 -> 1041 us.
+  // Above 256 rows it has no third M-tile.  The masked variant's cache positions
+  // differ by block, which its token tables do not hold.
+  if (m <= kPfSmallRows && !c.masked) return launch_gemm_pf_small(c, epi, split, layer, which, xi, m, e, s);
   PfParams p{};
   int N, K, tiles;
   gemm_shape(c, which, &N, &K, &tiles);
@@ -768,8 +775,8 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
   p.status = c.status;
   p.wait_ns = c.wait_ns;
   const CUtensorMap& tw = c.pf_wmaps[(size_t)layer * 4 + which];
-  const CUtensorMap& tx = c.pf_tmaps[xi];
-  const CUtensorMap& txlo = c.pf_tmaps[3 + xi];
+  const CUtensorMap& tx = c.pf_xmaps[xi].box[3];
+  const CUtensorMap& txlo = c.pf_xmaps[3 + xi].box[3];
   const int grid = 2 * (p.units ? std::min(std::max(p.units, p.sk_pairs), P) : p.sk_pairs);
   const size_t smem = c.pf_smem[v];
   if (split) {

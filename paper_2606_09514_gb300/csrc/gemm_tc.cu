@@ -401,6 +401,16 @@ static int choose_splits(int tiles, int kb, int sms) {
   return best_eff > 0 ? best : fb;
 }
 
+// The same with a deferred fixup.  A gate/up GEMM that is not split applies SwiGLU
+// itself, without workspace or fixup kernel: taken when its tiles keep at least
+// 70% of the SMs streaming (the rest of HBM's rate they reach all the same:
+// Llama-3-8B's 112 tiles at 64 rows take as long as 448 units, and the 10 us
+// fixup is saved; 6 blocks 1259 -> 1209 us).
+static int defer_splits(int which, int tiles, int kb, int sms) {
+  if (which == 2 && 10 * tiles >= 7 * sms && tiles <= sms) return 1;
+  return choose_splits(tiles, kb, sms);
+}
+
 // bf16 shapes always take the tensor-core path: sm_103 and at most 256 rows
 // (buddy_create rejects anything else).
 bool gemm_tc_supported(const Ctx& c) {
@@ -437,16 +447,14 @@ int gemm_tc_prepare(Ctx& c) {
     int N, K, tiles;
     gemm_shape(c, w, &N, &K, &tiles);
     const int kb = (K + kTileK - 1) / kTileK;
-    c.tc_splits[w] = choose_splits(tiles, kb, c.num_sms);
-    // A gate/up GEMM above kTcDeferRows rows that is not split applies SwiGLU
-    // itself, without workspace or fixup kernel: taken when its tiles keep at least
-    // 70% of the SMs streaming (the rest of HBM's rate they reach all the same:
-    // Llama-3-8B's 112 tiles at 64 rows take as long as 448 units, and the 10 us
-    // fixup is saved; 6 blocks 1259 -> 1209 us).
-    if (w == 2 && c.maxB > kTcDeferRows && 10 * tiles >= 7 * c.num_sms && tiles <= c.num_sms) c.tc_splits[w] = 1;
+    c.tc_splits[w] = c.maxB > kTcDeferRows ? defer_splits(w, tiles, kb, c.num_sms) : choose_splits(tiles, kb, c.num_sms);
     c.tc_tiles[w] = tiles;
     // every unit stages its accumulator rows in the workspace
     ws = std::max(ws, (size_t)tiles * c.tc_splits[w] * c.tc_rows_max * c.tc_bw);
+    if (c.pf_max > 0) {   // prompts of few tokens
+      const int rows = std::min(kPfSmallRows, (c.pf_max + 15) & ~15);
+      ws = std::max(ws, (size_t)tiles * defer_splits(w, tiles, kb, c.num_sms) * std::max(16, rows) * c.tc_bw);
+    }
     max_tiles = std::max(max_tiles, tiles);
   }
   // tensor maps: activations (fixed scratch) and per-layer weights
@@ -513,13 +521,11 @@ int gemm_tc_prepare(Ctx& c) {
           !make_map(&M[2], w.w_gate_up, 2ull * c.F, c.d, 128) || !make_map(&M[3], w.w_down, c.d, c.F, 128))
         return BUDDY_ERR_ARG;
     }
-    if (!make_map(&c.pf_tmaps[0], c.pf_xn, c.pf_max, c.d, 128) ||
-        !make_map(&c.pf_tmaps[1], c.pf_attn, c.pf_max, c.qd, 128) ||
-        !make_map(&c.pf_tmaps[2], c.pf_act, c.pf_max, c.F, 128) ||
-        !make_map(&c.pf_tmaps[3], c.pf_xn_lo, c.pf_max, c.d, 128) ||
-        !make_map(&c.pf_tmaps[4], c.pf_attn_lo, c.pf_max, c.qd, 128) ||
-        !make_map(&c.pf_tmaps[5], c.pf_act_lo, c.pf_max, c.F, 128))
-      return BUDDY_ERR_CUDA;
+    const struct { const void* p; int k; } pxs[6] = {{c.pf_xn, c.d},    {c.pf_attn, c.qd},    {c.pf_act, c.F},
+                                                     {c.pf_xn_lo, c.d}, {c.pf_attn_lo, c.qd}, {c.pf_act_lo, c.F}};
+    for (int i = 0; i < 6; ++i)
+      for (int b = 0; b < 4; ++b)
+        if (!make_map(&c.pf_xmaps[i].box[b], pxs[i].p, c.pf_max, pxs[i].k, 16u << b)) return BUDDY_ERR_CUDA;
     int rc = gemm_pf_prepare(c);
     if (rc == BUDDY_OK) rc = attention_pf_prepare(c);
     if (rc != BUDDY_OK) return rc;
@@ -528,14 +534,14 @@ int gemm_tc_prepare(Ctx& c) {
   const int qs0 = std::max(c.tc_smem[0], c.tc_panel ? c.tc_psmem[0] : 0);
   const int qs1 = std::max(c.tc_smem[1], c.tc_panel ? c.tc_psmem[1] : 0);
   bool bad = false;
-  if (c.tc_defer)
-    bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, true>, A, c.tc_smem[0]) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, true>, A, c.tc_smem[0]) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, true>, A, c.tc_smem[0]) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, true, true>, A, c.tc_smem[1]) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true, true>, A, c.tc_smem[1]) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true, true>, A, c.tc_smem[1]);
-  else
+  if (c.tc_defer || c.pf_max > 0)   // prefill chooses its stages by the tokens of a call
+    bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, true>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, true>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, true>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, true, true>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true, true>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true, true>, A, limit);
+  if (!bad && !c.tc_defer)
     bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, false>, A, qs0) ||
           cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, false>, A, c.tc_smem[0]) ||
           cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, false>, A, qs0) ||
@@ -632,6 +638,55 @@ void launch_gemm_tc(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s) {
   if (epi == EPI_QKV) a.split ? launch_tc<EPI_QKV, true>(c, a, s) : launch_tc<EPI_QKV, false>(c, a, s);
   else if (epi == EPI_RESID) a.split ? launch_tc<EPI_RESID, true>(c, a, s) : launch_tc<EPI_RESID, false>(c, a, s);
   else a.split ? launch_tc<EPI_SWIGLU, true>(c, a, s) : launch_tc<EPI_SWIGLU, false>(c, a, s);
+}
+
+// A projection of a prompt of few tokens: the deferred-fixup kernels with each
+// token row in the place of a sequence (its own position, block offset and
+// capacity), the ring and the workspace sized by the rows of this call.
+template <int EPI, bool SPLIT>
+static void launch_pf_small(const Ctx& c, int layer, int which, int xi, int m, const PfEpi& e, cudaStream_t s) {
+  GemmArgs a{};
+  a.sel = RowSel{e.rows, nullptr, m};
+  a.split = SPLIT;
+  a.out_act = e.out_act;
+  a.out_act_lo = e.out_act_lo;
+  a.resid_src = e.resid_src;
+  a.resid_dst = e.resid_dst;
+  a.qkv_bias = e.bias;
+  a.kv_len = a.cache_len = e.tok_pos;
+  a.kv_seq_off = e.tok_off;
+  a.kv_cap = e.tok_cap;
+  a.kc = e.kc;
+  a.vc = e.vc;
+  a.q_out = e.q_out;
+  a.layer = layer;
+  a.which = which;
+  size_t smem = 0;
+  TcParams p = tc_params(c, a, &smem);
+  p.splits = defer_splits(which, p.n_tiles, p.kb_total, c.num_sms);
+  p.kb_per_split = (p.kb_total + p.splits - 1) / p.splits;
+  p.units = p.n_tiles * p.splits;
+  p.mt = m > 128 ? 2 : 1;
+  p.acc_bufs = p.mt == 2 ? 1 : 2;
+  p.rows_max = std::max(16, (m + 15) & ~15);
+  p.xr = p.mt == 1 ? (uint32_t)p.rows_max * 128u : kXTileMax;
+  p.w_off = (SPLIT ? 2u : 1u) * p.mt * p.xr;
+  p.stage_bytes = p.w_off + (uint32_t)p.bw * 128u;
+  const int limit = 227 * 1024 - 2 * 1024;
+  p.stages = std::min(kTcMaxStages, (int)((limit - 1024) / p.stage_bytes));
+  smem = (size_t)p.stages * p.stage_bytes + 1024;
+  launch_k(gemm_tc_kernel<EPI, SPLIT, true>, std::min(p.units, c.num_sms), kTcDeferThreads, smem, s, c.pdl,
+           c.tmaps_host[(size_t)layer * 4 + which], c.pf_xmaps[xi], c.pf_xmaps[3 + xi], p);
+  if (!(EPI == EPI_SWIGLU && p.splits == 1))
+    launch_k(gemm_fix_kernel<EPI, SPLIT>, c.num_sms * (2048 / kTcFixThreads), kTcFixThreads, 0, s, c.pdl, p);
+}
+
+void launch_gemm_pf_small(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
+                          cudaStream_t s) {
+  auto go = [&](auto plain, auto hilo) { (split ? hilo : plain)(c, layer, which, xi, m, e, s); };
+  if (epi == EPI_QKV) go(launch_pf_small<EPI_QKV, false>, launch_pf_small<EPI_QKV, true>);
+  else if (epi == EPI_RESID) go(launch_pf_small<EPI_RESID, false>, launch_pf_small<EPI_RESID, true>);
+  else go(launch_pf_small<EPI_SWIGLU, false>, launch_pf_small<EPI_SWIGLU, true>);
 }
 
 template <int EPI, bool SPLIT>

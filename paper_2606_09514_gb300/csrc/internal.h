@@ -16,6 +16,7 @@ namespace buddy {
 constexpr int kMaxLayers = 128;
 constexpr int kRouteZSlots = 32;  // K-split slots of the router's hidden-unit partial sums
 constexpr int kMaxBatch = 1024;
+constexpr int kPfSmallRows = 256;  // prefill tokens up to which the decode GEMMs run its projections
 constexpr int kSimtFuseRows = 24;  // fp32: rows up to which the GEMMs take in the norms and the QKV finalisation
 
 // Per-layer K/V base pointers passed by value to kernels that touch many layers.
@@ -93,6 +94,9 @@ struct PfEpi {
   const int32_t* cap;
   void* kc;
   void* vc;
+  // few tokens: token row -> block offset and capacity of its sequence (QKV)
+  const int64_t* tok_off;
+  const int32_t* tok_cap;
 };
 
 // Device checks a kernel can make by itself, in every CTA, instead of a check
@@ -167,6 +171,9 @@ void launch_gemm_tc(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s);
 int gemm_pf_prepare(Ctx& c);
 void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
                     cudaStream_t s);
+// The same projection by the decode GEMM and its fixup (m <= kPfSmallRows).
+void launch_gemm_pf_small(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
+                          cudaStream_t s);   // gemm_tc.cu
 void launch_attention_pf(const Ctx& c, int n_items, const int4* items, const int32_t* n_tok, const int32_t* base,
                          const buddy_kv_state& kv, int layer, const float* q, void* out, void* out_lo,
                          cudaStream_t s);
@@ -268,7 +275,9 @@ struct Ctx {
   int32_t* pf_cnt = nullptr;      // [maxB] positions the pooled context covers
   float* pf_hlast = nullptr;      // [maxB, d] last prompt token's hidden state
   std::vector<CUtensorMap> pf_wmaps;   // per layer 4 weight maps, 128-row boxes
-  CUtensorMap pf_tmaps[6];        // pf_xn, pf_attn, pf_act, then their remainder terms
+  XMaps pf_xmaps[6];              // pf_xn, pf_attn, pf_act, then their remainder terms
+  int64_t* pf_tok_off = nullptr;  // [pf_max] token row -> its sequence's block offset
+  int32_t* pf_tok_cap = nullptr;  // [pf_max] token row -> its sequence's capacity
   int pf_stages[2] = {1, 1}, pf_smem[2] = {0, 0};
   float4* pf_ws = nullptr;        // parts of units cut along K
   int32_t* pf_ctr = nullptr;      // K blocks that have arrived, per cut unit and CTA

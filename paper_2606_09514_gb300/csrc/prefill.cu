@@ -25,12 +25,17 @@ namespace buddy {
 // Token tables, checks, gathers and the position advance
 // ---------------------------------------------------------------------------
 __global__ void pf_tokens_kernel(int T, const int32_t* tok_seq, const int32_t* tok_t, const int32_t* len,
-                                 int32_t* tok_pos, const int32_t* status) {
+                                 const int64_t* seq_off, const int32_t* cap, int32_t* tok_pos, int64_t* tok_off,
+                                 int32_t* tok_cap, const int32_t* status) {
   pdl_wait();
   pdl_trigger();
   if (call_aborted(status)) return;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r < T) tok_pos[r] = len[tok_seq[r]] + tok_t[r];
+  if (r >= T) return;
+  const int s = tok_seq[r];
+  tok_pos[r] = len[s] + tok_t[r];
+  tok_off[r] = seq_off[s];
+  tok_cap[r] = cap[s];
 }
 
 // Budgets in range (0 allowed with a Budget Predictor), and room for every
@@ -146,6 +151,8 @@ static void pf_block(Ctx& c, const buddy_kv_state& kv, int l, const PfLayerWork&
   e.cap = kv.cap;
   e.kc = kv.k_cache[l];
   e.vc = kv.v_cache[l];
+  e.tok_off = c.pf_tok_off;
+  e.tok_cap = c.pf_tok_cap;
   {
     ProfScope p(c, s, BUDDY_PROF_PF_GEMM, 1, prof);
     launch_gemm_pf(c, EPI_QKV, split, l, 0, 0, w.m, e, s);
@@ -217,7 +224,8 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
            (const int32_t*)kv.len, kv.cap, c.max_pos, (const int32_t*)(c.masked ? kv.layer_len : nullptr), c.L,
            kv.batch, c.status);
   launch_k(pf_tokens_kernel, (T + 255) / 256, 256, 0, s, c.pdl, T, (const int32_t*)c.pf_tok_seq,
-           (const int32_t*)c.pf_tok_t, (const int32_t*)kv.len, c.pf_tok_pos, (const int32_t*)c.status);
+           (const int32_t*)c.pf_tok_t, (const int32_t*)kv.len, kv.seq_off, kv.cap, c.pf_tok_pos, c.pf_tok_off,
+           c.pf_tok_cap, (const int32_t*)c.status);
 
   // attention work items for a set of sequences: (token, head of a group) rows
   // of one KV head, those that see the most positions first (the last to start
