@@ -56,10 +56,12 @@ static void free_ctx(buddy_ctx* x) {
                   c.attn_m, c.attn_l, c.attn_acc, c.attn_ctr, c.dm_u, c.mask, c.sel, c.scores, c.rows,
                   c.count, c.h_in_stage, c.h_out_stage, c.k_stage, c.mask_stage, c.xn_lo, c.act_lo, c.attn_lo,
                   c.gemm_ws, c.gemm_ctr, c.pf_xn, c.pf_xn_lo, c.pf_q, c.pf_attn, c.pf_attn_lo,
-                  c.pf_act, c.pf_act_lo, c.pf_tok_seq, c.pf_tok_t, c.pf_tok_pos, c.pf_tok_off, c.pf_tok_cap, c.pf_rows, c.pf_items,
-                  c.pf_n_tok, c.pf_tok_end, c.pf_cnt, c.pf_hlast, c.pf_ws, c.pf_ctr};
+                  c.pf_act, c.pf_act_lo, c.pf_tok_pos, c.pf_tok_off, c.pf_tok_cap, c.pf_up,
+                  c.pf_cnt, c.pf_hlast, c.pf_ws, c.pf_ctr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  if (c.pf_up_host) cudaFreeHost(c.pf_up_host);
+  if (c.pf_down) cudaFreeHost(c.pf_down);
   if (x->cap_stream) cudaStreamDestroy(x->cap_stream);
   delete x;
 }
@@ -153,15 +155,18 @@ extern "C" int buddy_create(const buddy_config* cfg, buddy_ctx** out) {
   if (c.pf_max > 0) {
     const size_t T = c.pf_max;
     c.pf_items_max = (int64_t)(T / 64 + B) * c.nq;
+    // token -> sequence and index, lengths and ends per prompt, the items of two
+    // lists; then row lists and items of the routed blocks (pieces of 16 bytes)
+    c.pf_up_second = (2 * T + 2 * B) * sizeof(int32_t) + 2 * c.pf_items_max * sizeof(int4) + 16 * 5;
+    c.pf_up_bytes = c.pf_up_second + (size_t)c.L * T * sizeof(int32_t) +
+                    (size_t)(c.L - 1) * c.pf_items_max * sizeof(int4) + 16 * 2;
     if ((e = cudaMalloc(&c.pf_xn, T * c.d * c.esz)) || (e = cudaMalloc(&c.pf_xn_lo, T * c.d * c.esz)) ||
         (e = dalloc(&c.pf_q, T * c.qd)) || (e = cudaMalloc(&c.pf_attn, T * c.qd * c.esz)) ||
         (e = cudaMalloc(&c.pf_attn_lo, T * c.qd * c.esz)) || (e = cudaMalloc(&c.pf_act, T * c.F * c.esz)) ||
-        (e = cudaMalloc(&c.pf_act_lo, T * c.F * c.esz)) || (e = dalloc(&c.pf_tok_seq, T)) ||
-        (e = dalloc(&c.pf_tok_t, T)) || (e = dalloc(&c.pf_tok_pos, T)) || (e = dalloc(&c.pf_tok_off, T)) ||
+        (e = cudaMalloc(&c.pf_act_lo, T * c.F * c.esz)) || (e = dalloc(&c.pf_tok_pos, T)) || (e = dalloc(&c.pf_tok_off, T)) ||
         (e = dalloc(&c.pf_tok_cap, T)) ||
-        (e = dalloc(&c.pf_rows, (size_t)c.L * T)) ||
-        (e = dalloc(&c.pf_items, (size_t)(c.L + 1) * c.pf_items_max)) || (e = dalloc(&c.pf_n_tok, B)) ||
-        (e = dalloc(&c.pf_tok_end, B)) || (e = dalloc(&c.pf_cnt, B)) || (e = dalloc(&c.pf_hlast, B * c.d)))
+        (e = dalloc(&c.pf_up, c.pf_up_bytes)) || (e = cudaMallocHost((void**)&c.pf_up_host, c.pf_up_bytes)) ||
+        (e = cudaMallocHost((void**)&c.pf_down, B * c.L + 16)) || (e = dalloc(&c.pf_cnt, B)) || (e = dalloc(&c.pf_hlast, B * c.d)))
       return fail(e);
   }
   if ((e = cudaStreamCreateWithFlags(&x->cap_stream, cudaStreamNonBlocking)) != cudaSuccess) return fail(e);

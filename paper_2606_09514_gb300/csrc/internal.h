@@ -265,13 +265,17 @@ struct Ctx {
   void* pf_attn_lo = nullptr;
   void* pf_act = nullptr;         // [pf_max, F] bf16 (+ remainder)
   void* pf_act_lo = nullptr;
-  int32_t* pf_tok_seq = nullptr;  // [pf_max] token row -> sequence
-  int32_t* pf_tok_t = nullptr;    // [pf_max] token row -> index in its prompt
+  // a call's tables from the host: one pinned area and one device area, packed by
+  // each call; the part for the start of the call, then (at pf_up_second) the part
+  // for the routed blocks, so that the first can be refilled while a copy of the
+  // second is still under way.  pf_down: the routes and the status word, pinned.
+  uint8_t* pf_up_host = nullptr;
+  uint8_t* pf_up = nullptr;
+  size_t pf_up_second = 0, pf_up_bytes = 0;
+  uint8_t* pf_down = nullptr;
   int32_t* pf_tok_pos = nullptr;  // [pf_max] token row -> position
-  int32_t* pf_rows = nullptr;     // [L, pf_max] row lists of the routed blocks
-  int4* pf_items = nullptr;       // [(L + 1) * pf_items_max] attention work items
-  int32_t* pf_n_tok = nullptr;    // [maxB]
-  int32_t* pf_tok_end = nullptr;  // [maxB] one past the last token row of each prompt
+  const int32_t* pf_n_tok = nullptr;     // this call's prompt lengths (in pf_up)
+  const int32_t* pf_tok_seq = nullptr;   // this call's token row -> sequence (in pf_up)
   int32_t* pf_cnt = nullptr;      // [maxB] positions the pooled context covers
   float* pf_hlast = nullptr;      // [maxB, d] last prompt token's hidden state
   std::vector<CUtensorMap> pf_wmaps;   // per layer 4 weight maps, 128-row boxes
