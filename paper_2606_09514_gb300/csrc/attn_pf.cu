@@ -155,23 +155,36 @@ __global__ void __launch_bounds__(pfa_threads<SPLIT>(), 1) attn_pf_kernel(const 
     if (q < nq) {
       // ------------------------------------------------------------- softmax
       const int rt = (warp & 3) * 32 + lane;            // row of the tile
-      const bool live = row0 + q * kPfaRows + rt < R;
       const int row = min(R - 1, row0 + q * kPfaRows + rt);
       const int t = row / G, h = g * G + row - t * G;
       const size_t at = ((size_t)(it.z + t) * A.nq + h) * HD;
-      {   // the row's query, scaled, as bf16 (hi, lo) in the swizzled K-major layout
+      // The queries of this warp's 32 rows, scaled, as bf16 (hi, lo) in the swizzled
+      // K-major layout: the lanes share a row (HD / 4 lanes, 16 bytes each), eight
+      // loads in flight.  (A row per lane reads 32 sectors for 16 bytes each: 5 to
+      // 7 us of a work item.)
+      uint8_t* const qdst = sQ + (size_t)q * (SPLIT ? 2 : 1) * TILE;
+      {
+        constexpr int LPR = HD / 4, RPL = 32 / LPR;     // lanes per row, rows per load
         const float scale = 1.4426950408889634f * rsqrtf((float)HD);
-        const float4* src = reinterpret_cast<const float4*>(A.q + at);
-        uint8_t* dst = sQ + (size_t)q * (SPLIT ? 2 : 1) * TILE;
-#pragma unroll 8
-        for (int c = 0; c < V16; ++c) {
-          const float4 a = src[2 * c], b = src[2 * c + 1];
-          const float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-          uint32_t hi[4], lo[4];
+        const int l4 = lane % LPR;
+#pragma unroll 1
+        for (int r0 = 0; r0 < 32; r0 += 8 * RPL) {
+          float4 v[8];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) tca::split_pack(f[2 * i] * scale, f[2 * i + 1] * scale, hi[i], lo[i]);
-          *reinterpret_cast<uint4*>(dst + pfa_piece(rt, c)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          if (SPLIT) *reinterpret_cast<uint4*>(dst + TILE + pfa_piece(rt, c)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          for (int u = 0; u < 8; ++u) {
+            const size_t src = __shfl_sync(0xffffffffu, (unsigned long long)at, r0 + u * RPL + lane / LPR);
+            v[u] = *reinterpret_cast<const float4*>(A.q + src + l4 * 4);
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int r = (warp & 3) * 32 + r0 + u * RPL + lane / LPR;
+            uint32_t hi[2], lo[2];
+            tca::split_pack(v[u].x * scale, v[u].y * scale, hi[0], lo[0]);
+            tca::split_pack(v[u].z * scale, v[u].w * scale, hi[1], lo[1]);
+            uint8_t* d = qdst + pfa_piece(r, l4 >> 1) + (l4 & 1) * 8;
+            *reinterpret_cast<uint2*>(d) = make_uint2(hi[0], hi[1]);
+            if (SPLIT) *reinterpret_cast<uint2*>(d + TILE) = make_uint2(lo[0], lo[1]);
+          }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         ptx::mbar_arrive(&q_ready);
@@ -251,12 +264,13 @@ __global__ void __launch_bounds__(pfa_threads<SPLIT>(), 1) attn_pf_kernel(const 
       if (ok) {
         ptx::tc_fence_after();
         const float inv = 1.f / l;
+        // through this tile's query buffer (its MMAs are done), so that the lanes
+        // store whole rows
 #pragma unroll 1
         for (int c = 0; c < HD; c += 32) {
           uint32_t o[32];
           ptx::tmem_ld32(to + c, o);
           ptx::tmem_wait_ld();
-          if (!live) continue;
 #pragma unroll
           for (int i = 0; i < 32; i += 8) {
             uint32_t hi[4], lo[4];
@@ -264,8 +278,21 @@ __global__ void __launch_bounds__(pfa_threads<SPLIT>(), 1) attn_pf_kernel(const 
             for (int e = 0; e < 4; ++e)
               tca::split_pack(__uint_as_float(o[i + 2 * e]) * inv, __uint_as_float(o[i + 2 * e + 1]) * inv, hi[e],
                               lo[e]);
-            *reinterpret_cast<uint4*>(A.out + at + c + i) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            if (SPLIT) *reinterpret_cast<uint4*>(A.out_lo + at + c + i) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            uint8_t* d = qdst + pfa_piece(rt, (c + i) >> 3);
+            *reinterpret_cast<uint4*>(d) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            if (SPLIT) *reinterpret_cast<uint4*>(d + TILE) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          }
+        }
+        __syncwarp();
+        constexpr int RPS = 32 / V16;                   // rows per store
+#pragma unroll 4
+        for (int r0 = 0; r0 < 32; r0 += RPS) {
+          const int r = r0 + lane / V16, c = lane % V16;
+          const size_t dst = __shfl_sync(0xffffffffu, (unsigned long long)at, r) + c * 8;
+          const uint8_t* d = qdst + pfa_piece((warp & 3) * 32 + r, c);
+          if (row0 + q * kPfaRows + (warp & 3) * 32 + r < R) {
+            *reinterpret_cast<uint4*>(A.out + dst) = *reinterpret_cast<const uint4*>(d);
+            if (SPLIT) *reinterpret_cast<uint4*>(A.out_lo + dst) = *reinterpret_cast<const uint4*>(d + TILE);
           }
         }
       }
