@@ -31,7 +31,7 @@
 //
 // Bound by the MMA issue (about 100 cycles for the 64 cycles of an N = 128 MMA)
 // and the softmax chain.  Two prompts of 2,999 and 5,000 tokens, 28 heads of 128
-// over 4 KV heads: 0.30 ms (0.9 PFLOP/s of the visible positions), 0.57 ms with
+// over 4 KV heads: 0.28 ms (1.0 PFLOP/s of the visible positions), 0.54 ms with
 // SPLIT, against 1.16 and 1.55 ms on mma.sync with 64-row tiles of one head.
 #include <cuda_runtime.h>
 
