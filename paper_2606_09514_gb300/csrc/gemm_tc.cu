@@ -640,6 +640,15 @@ void launch_gemm_tc(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s) {
   else a.split ? launch_tc<EPI_SWIGLU, true>(c, a, s) : launch_tc<EPI_SWIGLU, false>(c, a, s);
 }
 
+// CTAs of a fixup over at most `rows` rows: one item per thread, up to what the
+// GPU holds at once (1,216 CTAs for 64 rows were mostly launched to find nothing).
+template <int EPI>
+static int fix_grid(const Ctx& c, const TcParams& p, int rows) {
+  const int groups = EPI == EPI_SWIGLU || EPI == EPI_QKV ? p.bw / 8 : p.bw / 4;
+  const int64_t items = (int64_t)p.n_tiles * groups * (p.rows_max <= 16 ? rows : (rows + 7) / 8 * 8);
+  return (int)std::min<int64_t>((items + kTcFixThreads - 1) / kTcFixThreads, c.num_sms * (2048 / kTcFixThreads));
+}
+
 // A projection of a prompt of few tokens: the deferred-fixup kernels with each
 // token row in the place of a sequence (its own position, block offset and
 // capacity), the ring and the workspace sized by the rows of this call.
@@ -678,7 +687,7 @@ static void launch_pf_small(const Ctx& c, int layer, int which, int xi, int m, c
   launch_k(gemm_tc_kernel<EPI, SPLIT, true>, std::min(p.units, c.num_sms), kTcDeferThreads, smem, s, c.pdl,
            c.tmaps_host[(size_t)layer * 4 + which], c.pf_xmaps[xi], c.pf_xmaps[3 + xi], p);
   if (!(EPI == EPI_SWIGLU && p.splits == 1))
-    launch_k(gemm_fix_kernel<EPI, SPLIT>, c.num_sms * (2048 / kTcFixThreads), kTcFixThreads, 0, s, c.pdl, p);
+    launch_k(gemm_fix_kernel<EPI, SPLIT>, fix_grid<EPI>(c, p, m), kTcFixThreads, 0, s, c.pdl, p);
 }
 
 void launch_gemm_pf_small(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
@@ -693,7 +702,7 @@ template <int EPI, bool SPLIT>
 static void launch_fix(const Ctx& c, const GemmArgs& a, cudaStream_t s) {
   size_t smem = 0;
   const TcParams p = tc_params(c, a, &smem);
-  launch_k(gemm_fix_kernel<EPI, SPLIT>, c.num_sms * (2048 / kTcFixThreads), kTcFixThreads, 0, s, c.pdl, p);
+  launch_k(gemm_fix_kernel<EPI, SPLIT>, fix_grid<EPI>(c, p, a.sel.n), kTcFixThreads, 0, s, c.pdl, p);
 }
 
 void launch_gemm_fix(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s) {
