@@ -379,9 +379,50 @@ __device__ __forceinline__ uint2 pack4_bf16(const float* y) {
                         ((uint32_t)__bfloat16_as_ushort(from_f<bf16>(y[3])) << 16));
 }
 
+// What an epilogue item reads besides the accumulator: nothing the GEMM before
+// it writes, so that a fixup kernel loads it before its dependency wait.
+struct TcPre {
+  int seq;
+  float rs[4];            // residual: the source row's columns
+  int64_t kv;             // QKV: element offset of the item's K or V entry
+  float co[4], si[4];     // q and K: the rotation's factors
+};
+template <int EPI>
+__device__ __forceinline__ TcPre tc_pre(const TcParams& p, int tile, int j, int c) {
+  TcPre r{};
+  const int n0 = tile * p.bw + c;
+  if (EPI == EPI_RESID) {
+    r.seq = p.rows ? p.rows[j] : j;
+    const float* src = p.resid_src + (size_t)r.seq * p.N + n0;
+    if (n0 + 4 <= p.N) {
+      const float4 r4 = *reinterpret_cast<const float4*>(src);
+      r.rs[0] = r4.x; r.rs[1] = r4.y; r.rs[2] = r4.z; r.rs[3] = r4.w;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (n0 + i < p.N) r.rs[i] = src[i];
+    }
+  } else if (EPI == EPI_QKV) {
+    if (n0 >= p.N) return r;
+    const int hd = p.hd, half = hd >> 1, head = n0 / hd, e0 = n0 - head * hd;
+    r.seq = p.rows ? p.rows[j] : j;
+    if (head < p.nq + p.nkv) {
+      const size_t at = (size_t)p.len[r.seq] * half + e0;   // a multiple of 4
+      const float4 c4 = *reinterpret_cast<const float4*>(p.rope_cos + at);
+      const float4 s4 = *reinterpret_cast<const float4*>(p.rope_sin + at);
+      r.co[0] = c4.x; r.co[1] = c4.y; r.co[2] = c4.z; r.co[3] = c4.w;
+      r.si[0] = s4.x; r.si[1] = s4.y; r.si[2] = s4.z; r.si[3] = s4.w;
+    }
+    if (head >= p.nq)
+      r.kv = kv_offset(p.seq_off, p.cap, r.seq, p.nkv, hd, head - p.nq - (head < p.nq + p.nkv ? 0 : p.nkv),
+                       p.cache_len[r.seq]) + e0;
+  }
+  return r;
+}
+
 template <int EPI, bool SPLIT>
 __device__ __forceinline__ void tc_apply4(const TcParams& p, int tile, int j, int c, const float* v, const float* vp,
-                                          const float* rs) {
+                                          const TcPre& pre) {
   if (EPI == EPI_SWIGLU) {
     const int f0 = tile * (p.bw >> 1) + c;
     if (f0 + 4 <= p.N) {   // one 8-byte store (N % 8 == 0, c % 4 == 0)
@@ -415,9 +456,7 @@ __device__ __forceinline__ void tc_apply4(const TcParams& p, int tile, int j, in
     const int n0 = tile * p.bw + c;
     if (n0 >= p.N) return;   // heads are whole: a group and its partner are in or out together
     const int head = n0 / hd, e0 = n0 - head * hd;
-    const int seq = p.rows ? p.rows[j] : j;
-    const int pos = p.len[seq];
-    const int cpos = p.cache_len[seq];
+    const int seq = pre.seq;
     float x[4], xp[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -425,26 +464,24 @@ __device__ __forceinline__ void tc_apply4(const TcParams& p, int tile, int j, in
       xp[i] = vp[i] + (p.bias ? p.bias[n0 + half + i] : 0.f);
     }
     if (head < p.nq + p.nkv) {
-      const float* co = p.rope_cos + (size_t)pos * half + e0;
-      const float* si = p.rope_sin + (size_t)pos * half + e0;
       float lo[4], hi[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        lo[i] = x[i] * co[i] - xp[i] * si[i];
-        hi[i] = xp[i] * co[i] + x[i] * si[i];
+        lo[i] = x[i] * pre.co[i] - xp[i] * pre.si[i];
+        hi[i] = xp[i] * pre.co[i] + x[i] * pre.si[i];
       }
       if (head < p.nq) {
         float* q = p.q_out + (size_t)j * p.nq * hd + n0;
         *reinterpret_cast<float4*>(q) = make_float4(lo[0], lo[1], lo[2], lo[3]);
         *reinterpret_cast<float4*>(q + half) = make_float4(hi[0], hi[1], hi[2], hi[3]);
       } else {
-        bf16* k = p.kc + kv_offset(p.seq_off, p.cap, seq, p.nkv, hd, head - p.nq, cpos) + e0;
+        bf16* k = p.kc + pre.kv;
         *reinterpret_cast<uint2*>(k) = pack4_bf16(lo);
         *reinterpret_cast<uint2*>(k + half) = pack4_bf16(hi);
       }
     } else {
       const int g = head - p.nq - p.nkv;
-      bf16* vv = p.vc + kv_offset(p.seq_off, p.cap, seq, p.nkv, hd, g, cpos) + e0;
+      bf16* vv = p.vc + pre.kv;
       float* pl = p.pool ? p.pool + (size_t)seq * p.nkv * hd + g * hd + e0 : nullptr;
       *reinterpret_cast<uint2*>(vv) = pack4_bf16(x);
       *reinterpret_cast<uint2*>(vv + half) = pack4_bf16(xp);
@@ -459,10 +496,9 @@ __device__ __forceinline__ void tc_apply4(const TcParams& p, int tile, int j, in
   } else {
     const int n0 = tile * p.bw + c;
     float w[4];
-    const int seq = p.rows ? p.rows[j] : j;
-    float* dst = p.resid_dst + (size_t)seq * p.N + n0;
+    float* dst = p.resid_dst + (size_t)pre.seq * p.N + n0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = rs[i] + v[i];
+    for (int i = 0; i < 4; ++i) w[i] = pre.rs[i] + v[i];
     if (n0 + 4 <= p.N) {   // one 16-byte store (N % 4 == 0, c % 4 == 0)
       *reinterpret_cast<float4*>(dst) = make_float4(w[0], w[1], w[2], w[3]);
     } else {
@@ -486,25 +522,12 @@ __device__ __forceinline__ size_t tc_ws_idx(const TcParams& p, int j, int c) {
 // all K splits (and of the partner columns) are summed in split order, eight
 // splits' loads in flight at a time, and the epilogue is applied.
 template <int EPI, bool SPLIT>
-__device__ __forceinline__ void tc_fix_item(const TcParams& p, int tile, int j, int c) {
+__device__ __forceinline__ void tc_fix_item(const TcParams& p, int tile, int j, int c, const TcPre& pre) {
   const int po = tc_partner_off<EPI>(p);
   const size_t sstride = (size_t)p.n_tiles * p.rows_max * p.bw / 4;   // one split's slots (float4)
   const size_t pstride = tc_ws_idx(p, j, c + po) - tc_ws_idx(p, j, c);
   const float4* sl = reinterpret_cast<const float4*>(p.ws + (size_t)tile * p.rows_max * p.bw) + tc_ws_idx(p, j, c);
-  float v[4] = {0.f, 0.f, 0.f, 0.f}, vp[4] = {0.f, 0.f, 0.f, 0.f}, rs[4] = {0.f, 0.f, 0.f, 0.f};
-  if (EPI == EPI_RESID) {
-    const int seq = p.rows ? p.rows[j] : j;
-    const int n0 = tile * p.bw + c;
-    const float* src = p.resid_src + (size_t)seq * p.N + n0;
-    if (n0 + 4 <= p.N) {
-      const float4 r4 = *reinterpret_cast<const float4*>(src);
-      rs[0] = r4.x; rs[1] = r4.y; rs[2] = r4.z; rs[3] = r4.w;
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (n0 + i < p.N) rs[i] = src[i];
-    }
-  }
+  float v[4] = {0.f, 0.f, 0.f, 0.f}, vp[4] = {0.f, 0.f, 0.f, 0.f};
   for (int s0 = 0; s0 < p.splits; s0 += 8) {
     float4 x[8], y[8];
 #pragma unroll
@@ -524,7 +547,7 @@ __device__ __forceinline__ void tc_fix_item(const TcParams& p, int tile, int j, 
       }
     }
   }
-  tc_apply4<EPI, SPLIT>(p, tile, j, c, v, vp, rs);
+  tc_apply4<EPI, SPLIT>(p, tile, j, c, v, vp, pre);
 }
 
 // ---------------------------------------------------------------------------
@@ -632,7 +655,8 @@ __device__ __forceinline__ void tc_epilogue_unit(const TcParams& p, int u, int m
     const int items = m * ng;
     for (int it = et; it < items; it += 128) {   // one item per thread per round
       const int j = it / ng;
-      tc_fix_item<EPI, SPLIT>(p, tile, j, tc_group_col<EPI>(p, it - j * ng));
+      const int c = tc_group_col<EPI>(p, it - j * ng);
+      tc_fix_item<EPI, SPLIT>(p, tile, j, c, tc_pre<EPI>(p, tile, j, c));
     }
   }
   epi_bar();

@@ -309,33 +309,51 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
 // 4 contiguous groups of each row's outputs).
 template <int EPI, bool SPLIT>
 __global__ void __launch_bounds__(kTcFixThreads) gemm_fix_kernel(const TcParams p) {
-  pdl_wait();
-  pdl_trigger();
-  if (call_aborted(p.status)) return;
+  // The abort word, the row count and list, the positions and the residual rows
+  // were written before the GEMM this kernel follows (by kernels complete
+  // when that GEMM let this one launch): a thread loads its first item's before
+  // the wait, and only the partial sums after it.
   const int m = p.count ? *p.count : p.n;
-  if (m <= 0) return;
   const int ng = tc_groups<EPI>(p);
   const long long stride = (long long)gridDim.x * kTcFixThreads;
-  if (p.rows_max <= 16) {
-    const long long items = (long long)p.n_tiles * m * ng;
-    for (long long it = (long long)blockIdx.x * kTcFixThreads + threadIdx.x; it < items; it += stride) {
-      const int g = (int)(it % ng);
+  const bool flat = p.rows_max <= 16;
+  // flat: items (tile, row, group); else warp blocks of 8 rows x 4 groups (ng is a
+  // multiple of 4)
+  const int rb = (m + 7) >> 3, gb = ng >> 2, lane = threadIdx.x & 31;
+  const long long items = flat ? (long long)p.n_tiles * m * ng : (long long)p.n_tiles * gb * rb * 32;
+  long long it = (long long)blockIdx.x * kTcFixThreads + threadIdx.x;
+  int tile = 0, j = 0, c = 0;
+  auto place = [&]() {   // the item's tile, row and column; false past the rows
+    if (it >= items) return false;
+    int g;
+    if (flat) {
+      g = (int)(it % ng);
       const long long r = it / ng;
-      const int j = (int)(r % m), tile = (int)(r / m);
-      tc_fix_item<EPI, SPLIT>(p, tile, j, tc_group_col<EPI>(p, g));
-    }
-  } else {
-    // warp blocks of 8 rows x 4 groups (ng is a multiple of 4)
-    const int rb = (m + 7) >> 3, gb = ng >> 2;
-    const long long items = (long long)p.n_tiles * gb * rb * 32;
-    const int lane = threadIdx.x & 31;
-    for (long long it = (long long)blockIdx.x * kTcFixThreads + threadIdx.x; it < items; it += stride) {
+      j = (int)(r % m);
+      tile = (int)(r / m);
+    } else {
       const long long wb = it >> 5;
-      const int j = (int)(wb % rb) * 8 + (lane & 7);
+      j = (int)(wb % rb) * 8 + (lane & 7);
       const long long r = wb / rb;
-      const int g = (int)(r % gb) * 4 + (lane >> 3), tile = (int)(r / gb);
-      if (j < m) tc_fix_item<EPI, SPLIT>(p, tile, j, tc_group_col<EPI>(p, g));
+      g = (int)(r % gb) * 4 + (lane >> 3);
+      tile = (int)(r / gb);
     }
+    c = tc_group_col<EPI>(p, g);
+    return j < m;
+  };
+  // (not for a call whose checks failed: its positions may lie outside the tables)
+  const bool aborted = call_aborted(p.status);
+  bool live = place();
+  TcPre pre{};
+  if (live && !aborted) pre = tc_pre<EPI>(p, tile, j, c);
+  pdl_wait();
+  pdl_trigger();
+  if (aborted) return;
+  while (it < items) {
+    if (live) tc_fix_item<EPI, SPLIT>(p, tile, j, c, pre);
+    it += stride;
+    live = place();
+    if (live) pre = tc_pre<EPI>(p, tile, j, c);
   }
 }
 
