@@ -129,6 +129,15 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ 
                                                       const float* __restrict__ gamma, float eps,
                                                       T* __restrict__ xn, T* __restrict__ xn_lo,
                                                       const int32_t* status) {
+  constexpr int R = 8;   // float4 of the row per thread: rows up to 8192 stay in registers
+  float4 g[R];           // the gains, which no kernel writes, before the dependency wait
+  if (d <= 256 * 4 * R) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int e = (threadIdx.x + r * 256) * 4;
+      if (e < d) g[r] = *reinterpret_cast<const float4*>(gamma + e);
+    }
+  }
   pdl_wait();
   pdl_trigger();
   if (call_aborted(status)) return;
@@ -140,7 +149,6 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ 
   const float* h = H + (size_t)i * d;
   T* o = xn + (size_t)j * d;
   T* olo = xn_lo ? xn_lo + (size_t)j * d : nullptr;
-  constexpr int R = 8;   // float4 of the row per thread: rows up to 8192 stay in registers
   if (d <= 256 * 4 * R) {
     float4 x[R];
     float ss = 0.f;
@@ -157,8 +165,7 @@ __global__ void __launch_bounds__(256) rmsnorm_kernel(const float* __restrict__ 
     for (int r = 0; r < R; ++r) {
       const int e = (threadIdx.x + r * 256) * 4;
       if (e >= d) break;
-      const float4 g = *reinterpret_cast<const float4*>(gamma + e);
-      const float y[4] = {x[r].x * inv * g.x, x[r].y * inv * g.y, x[r].z * inv * g.z, x[r].w * inv * g.w};
+      const float y[4] = {x[r].x * inv * g[r].x, x[r].y * inv * g[r].y, x[r].z * inv * g[r].z, x[r].w * inv * g[r].w};
       store4(o + e, y);
       if (olo) {   // remainder term (split activations)
         const float z[4] = {y[0] - to_f(from_f<T>(y[0])), y[1] - to_f(from_f<T>(y[1])),
