@@ -22,14 +22,14 @@
 // The ring fills shared memory and, with one M-tile, two accumulators let the
 // MMAs of the next unit overlap the epilogue.
 //
-// Panel mode (up to 8 rows): the ring holds weight tiles only and the
+// Panel mode (up to kTcDeferRows rows): the ring holds weight tiles only and the
 // activations of the QKV and gate/up GEMMs are the RMSNorm of the fp32
 // residual rows, computed by the epilogue warps into a shared-memory panel.
 //
 // Split-K: every unit stages its accumulator rows in a workspace slot; up to
-// 8 rows the last split of a tile to arrive sums the slots in split order
-// and applies the epilogue, above 8 rows gemm_fix_kernel does so over all
-// SMs (tc_ws_idx gives the slot layout).
+// kTcDeferRows rows the last split of a tile to arrive sums the slots in split
+// order and applies the epilogue, above them gemm_fix_kernel does so over all SMs
+// (tc_ws_idx gives the slot layout).
 #pragma once
 
 #include <cuda.h>
@@ -52,7 +52,11 @@ constexpr uint32_t kXTileMax = 128 * 128;        // bytes one M-tile operand spa
 constexpr int kTileN = 256;                      // weight rows per tile (MMA N)
 constexpr uint64_t kWaitLimitNs = 4000000000ull; // 4 s
 constexpr int kTcFixThreads = 256;                // deferred-fixup kernel
-constexpr int kTcDeferRows = 8;                   // larger batches defer the split-K fixup
+// Larger batches defer the split-K fixup.  The line lies where the panels and the
+// last split's own fixup stop paying for the launches they save: 4 blocks of
+// Llama-3-8B take 422 us at 2 rows with them and 429 us without, 465 and 440 us at
+// 3 rows, 523 and 456 us at 8 (one row: 406 and 414 us).
+constexpr int kTcDeferRows = 2;
 
 struct TcParams {
   int N, K;

@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
       const int kb0 = split * p.kb_per_split, kb1 = min(p.kb_total, kb0 + p.kb_per_split);
       if (!first_pass && et < m) prow[et] = p.rows ? p.rows[et] : et;
       epi_bar();   // staged gains and rows visible to all epilogue warps
-      if (first_pass && m <= 2) {
+      if (first_pass) {
         tc_panel_first<SPLIT>(p, smem + p.panel_off, m, kb0, kb1, et, prow,
                               reinterpret_cast<const float*>(smem + p.gstage_off), pred, pinv);
       } else {
@@ -503,12 +503,12 @@ int gemm_tc_prepare(Ctx& c) {
     c.gemm_ctr_n = max_tiles;
   }
   if (cudaMemset(c.gemm_ctr, 0, c.gemm_ctr_n * sizeof(int32_t)) != cudaSuccess) return BUDDY_ERR_CUDA;
-  // Panel mode for up to eight rows: the QKV and gate/up GEMMs normalise their
+  // Panel mode for up to kTcDeferRows rows: the QKV and gate/up GEMMs normalise their
   // own activations (no RMSNorm kernels, no activation copies).  Stages hold
   // weight tiles only; two panels of the largest K range follow the ring, then
   // 15 KiB for the tail of an M = 128 operand read, then the first unit's
   // RMSNorm gains (staged before the dependency wait).
-  c.tc_panel = c.maxB <= 8 && c.d % kTileK == 0;
+  c.tc_panel = c.maxB <= kTcDeferRows && c.d % kTileK == 0;
   if (c.tc_panel) {
     int N, K, tiles;
     gemm_shape(c, 0, &N, &K, &tiles);
