@@ -1,0 +1,190 @@
+"""GPU tests at the sizes where a kernel's tile, split or dispatch rule changes:
+prefill projections (one or two 128-row M-tiles of the decode GEMM up to 256
+tokens, CTA pairs above) and its attention (tiles of 128 (token, head) rows),
+small-batch decode modes and attention cluster sizes, the fp32 GEMMs, the router's
+and the bulk append's own argument checks, and the wait limits of these paths.
+Values are compared with the float64 oracle at the bounds of parity.py.
+"""
+import numpy as np
+import pytest
+import torch
+
+import paper_2606_09514_gb300 as pkg
+from paper_2606_09514_gb300 import binding as Bd
+from test_gpu_decode import run_parity
+from test_gpu_prefill import run_prefill_parity
+from workloads import configs as C
+from workloads import device as D
+from workloads import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def rows_of(base, batch):
+    """The workload's own contexts and budgets, repeated to `batch` rows."""
+    if base.ctx_kind != "list":
+        return C.scaled(base, batch=batch, name=f"{base.name}-b{batch}")
+    n = len(base.ctx_args)
+    return C.scaled(base, ctx=[base.ctx_args[i % n] for i in range(batch)],
+                    k=[base.k_args[i % n] for i in range(batch)], name=f"{base.name}-b{batch}")
+
+
+# tokens in all: 1; 16 and 17 (workspace layouts); 128 and 129 (M-tiles); 256 and
+# 257 (decode GEMMs and CTA pairs); 126 and 129 rows of a 3-head group (attention
+# tiles); the masked variant takes the CTA pairs at any size
+@pytest.mark.parametrize("base,lengths,ctx", [
+    (C.T_GQA, [1], [0]), (C.T_GQA, [16], [40]), (C.T_GQA, [17], [0]), (C.T_QWEN, [128], [1]),
+    (C.T_QWEN, [100, 29], [0, 127]), (C.T_QWEN, [256], [0]), (C.T_QWEN, [1, 256], [128, 3]),
+    (C.T_GQA, [42, 43], [0, 86]), (C.T_VARIANTS[2], [5, 40], [0, 65])],
+    ids=lambda v: v.shape.name if hasattr(v, "shape") else "-".join(map(str, v)))
+def test_prefill_parity_at_tile_edges(base, lengths, ctx):
+    w = C.scaled(base, ctx=ctx, k=[1 + i for i in range(len(ctx))], name="pf-edge")
+    assert run_prefill_parity(w, lengths, decode_steps=1) < 2e-2
+
+
+# 2 and 3 rows: panels and deferred fixup; 5, 10 and 21 rows of 3 KV heads: 15, 30
+# and 63 streams, in clusters of 8, 4 and 2 CTAs
+@pytest.mark.parametrize("base,batch", [(C.T_QWEN, 2), (C.T_QWEN, 3), (C.T_GQA, 2), (C.T_GQA, 5), (C.T_GQA, 10),
+                                        (C.T_GQA, 21)], ids=lambda v: v.shape.name if hasattr(v, "shape") else str(v))
+def test_decode_parity_small_batch_modes(base, batch):
+    assert run_parity(rows_of(base, batch), steps=2)[0] < 2e-2
+
+
+# fp32: four or eight rows per pass (4, 5), norms and QKV finalisation inside the
+# GEMMs up to 24 rows, tiles of 32 rows above (25, 32, 33)
+@pytest.mark.parametrize("batch", [4, 5, 24, 25, 32, 33])
+def test_decode_parity_f32_batch_modes(batch):
+    assert run_parity(rows_of(C.T_F32, batch), steps=2)[0] < 1e-4
+
+
+def route_scores64(dm, pool, length, h1, group, hd):
+    x = (pool.double() / length.double()[:, None]).view(pool.shape[0], -1, 1, hd)
+    x = torch.cat([x.expand(-1, -1, group, -1).reshape(pool.shape[0], -1), h1.double()], 1)
+    w = {k: v.double() for k, v in dm.items()}
+    return torch.nn.functional.silu(x @ w["w1"].T + w["b1"]) @ w["w2"].T + w["b2"]
+
+
+@pytest.mark.parametrize("batch", [1, 16, 17, 64, 65])
+def test_route_scores_at_batch_modes(batch):
+    s = C.SMALL_QWEN_BF16
+    w = rows_of(C.T_QWEN, batch)
+    dw = D.build(w)
+    h1 = synth.h_in(s, 5, 0, range(batch), "cuda")
+    dw.kv.len.clamp_(min=1)
+    sc = torch.empty(batch, s.n_cand, device="cuda")
+    dw.ctx.buddy_route(dw.kv, h1, dw.k, scores_out=sc)
+    assert dw.ctx.buddy_device_status() == 0
+    ref = route_scores64(dw.dm, dw.kv.pool_sum, dw.kv.len, h1, s.group, s.head_dim)
+    # sums of 2 d = 1536 and r = 96 fp32 products: 1e-6 of the scores' size
+    assert float((sc.double() - ref).abs().max()) < 2e-6 * max(1.0, float(ref.abs().max()))
+
+
+def test_route_checks_write_nothing():
+    w = rows_of(C.T_GQA, 3)
+    dw = D.build(w)
+    s = w.shape
+    h1 = synth.h_in(s, 5, 0, range(3), "cuda")
+    dw.kv.len.clamp_(min=1)
+    sc = torch.full((3, s.n_cand), 7.0, device="cuda")
+    bad = dw.k.clone()
+    bad[2] = 0   # no Budget Predictor
+    dw.ctx.buddy_route(dw.kv, h1, bad, scores_out=sc)
+    assert dw.ctx.buddy_device_status() == Bd.BUDDY_DEV_BAD_BUDGET and bool((sc == 7.0).all())
+    good_len = dw.kv.len.clone()
+    dw.kv.len[1] = dw.kv.cap[1] + 1
+    dw.ctx.buddy_route(dw.kv, h1, dw.k, scores_out=sc)
+    assert dw.ctx.buddy_device_status() == Bd.BUDDY_DEV_BAD_POSITION and bool((sc == 7.0).all())
+    dw.kv.len.copy_(good_len)
+    dw.ctx.buddy_route(dw.kv, h1, dw.k, scores_out=sc)
+    assert dw.ctx.buddy_device_status() == 0 and not bool((sc == 7.0).any())
+
+
+def append_state(shape, caps, max_batch):
+    ctx = pkg.Context.for_shape(shape, max_batch=max_batch, max_pos=max(caps))
+    layer = pkg.pack_layer(synth.layer_weights(shape, 0, 0, "cuda"))
+    ctx.buddy_set_weights([layer] * shape.n_layers, synth.dm_weights(shape, 0, "cuda"))
+    return ctx, pkg.KVCache(shape.n_layers, shape.n_kv_heads, shape.head_dim, caps, synth.storage_dtype(shape), "cuda")
+
+
+# 16-byte copies (8 positions per CTA) and, from a misaligned source, element
+# copies; up to 256 sequences the copy kernel checks the arguments itself
+@pytest.mark.parametrize("shape", [C.SMALL_GQA_BF16, C.SMALL_F32], ids=lambda s: s.name)
+@pytest.mark.parametrize("n_new,n_seq", [(1, 3), (8, 1), (9, 256), (33, 257)])
+def test_append_aligned_and_misaligned(shape, n_new, n_seq):
+    dt = synth.storage_dtype(shape)
+    n = n_seq * n_new * shape.kv_dim
+    g = torch.Generator(device="cuda").manual_seed(n)
+    flat = [torch.empty(n + 1, dtype=dt, device="cuda").normal_(generator=g) for _ in range(2)]
+    view = lambda t, o: t[o:o + n].view(n_seq, n_new, shape.n_kv_heads, shape.head_dim)
+    off = [view(t, 1) for t in flat]                 # not 16-byte aligned
+    same = [t.clone() for t in off]                  # aligned
+    ids = torch.arange(n_seq, dtype=torch.int32, device="cuda").flip(0).contiguous()
+    states = []
+    for kn, vn in (same, off):
+        ctx, kv = append_state(shape, [2 * n_new + 3] * n_seq, 4)
+        for _ in range(2):
+            ctx.buddy_kv_append(kv, 0, ids, kn, vn, advance=True)
+        assert ctx.buddy_device_status() == 0
+        states.append((kv, ctx))
+    a, b = states[0][0], states[1][0]
+    assert torch.equal(a.k[0], b.k[0]) and torch.equal(a.v[0], b.v[0]) and torch.equal(a.pool_sum, b.pool_sum)
+    for j in (0, n_seq - 1):
+        s = int(ids[j])
+        assert torch.equal(a.view("k", 0, s)[:, n_new:2 * n_new].transpose(0, 1), same[0][j])
+        ref = a.view("v", 0, s)[:, :2 * n_new].double().sum(1).reshape(-1)
+        np.testing.assert_allclose(a.pool_sum[s].double().cpu(), ref.cpu(), rtol=1e-5, atol=1e-5)
+    # a third append does not fit: flagged, nothing written
+    k0, len0 = a.k[0].clone(), a.len.clone()
+    a.len.add_(4)
+    states[0][1].buddy_kv_append(a, 0, ids, same[0], same[1], advance=True)
+    assert states[0][1].buddy_device_status() & Bd.BUDDY_DEV_BAD_POSITION
+    assert torch.equal(a.k[0], k0) and torch.equal(a.len, len0 + 4)
+    a.len.copy_(len0 - n_new)
+    ids[0] = n_seq
+    states[0][1].buddy_kv_append(a, 0, ids, same[0], same[1], advance=True)
+    assert states[0][1].buddy_device_status() & Bd.BUDDY_DEV_BAD_SEQ and torch.equal(a.k[0], k0)
+
+
+def test_panel_wait_limit_runs_out_and_context_recovers():
+    """As the other batches' test: 1 ns runs out, the restored limit gives a fresh context's result."""
+    w = C.scaled(C.T_GQA, ctx=[5, 200], k=[1, 3], name="t-gqa-b2-timeout")
+    h_in = synth.workload_h_in(w, 0, "cuda")
+    outs = []
+    for limited in (False, True):
+        dw = D.build(w)
+        h = torch.empty(2, w.shape.d_model, device="cuda")
+        len0, pool0 = dw.kv.len.clone(), dw.kv.pool_sum.clone()
+        if limited:
+            dw.ctx.buddy_set_wait_limit(1)
+            dw.ctx.buddy_decode_step(dw.kv, h_in, dw.k, h)
+            assert dw.ctx.buddy_device_status() & Bd.BUDDY_DEV_TIMEOUT
+            dw.ctx.buddy_set_wait_limit(0)
+            dw.kv.len.copy_(len0)
+            dw.kv.pool_sum.copy_(pool0)
+        dw.ctx.buddy_decode_step(dw.kv, h_in, dw.k, h)
+        assert dw.ctx.buddy_device_status() == 0
+        outs.append(h)
+    assert torch.equal(*outs)
+
+
+# the decode GEMMs (40 tokens), the CTA pairs and units cut along K (300 tokens)
+@pytest.mark.parametrize("lengths", [[33, 7], [290, 10]], ids=lambda v: str(sum(v)))
+def test_prefill_wait_limit_runs_out_and_context_recovers(lengths):
+    w = C.scaled(C.T_QWEN, ctx=[3, 60], k=[2, 4], name="pf-timeout")
+    T = sum(lengths)
+    x = synth.prompt_inputs(w.shape, w.seed, lengths, "cuda")
+    outs = []
+    for limited in (False, True):
+        dw = D.build(w, extra_steps=max(lengths) + 2, max_prefill_tokens=T)
+        h = torch.empty(T, w.shape.d_model, device="cuda")
+        len0 = dw.kv.len.clone()
+        if limited:
+            dw.ctx.buddy_set_wait_limit(1)
+            dw.ctx.buddy_prefill(dw.kv, lengths, x, dw.k, h)
+            assert dw.ctx.buddy_device_status() & Bd.BUDDY_DEV_TIMEOUT
+            dw.ctx.buddy_set_wait_limit(0)
+            dw.kv.len.copy_(len0)
+        dw.ctx.buddy_prefill(dw.kv, lengths, x, dw.k, h)
+        assert dw.ctx.buddy_device_status() == 0
+        outs.append(h)
+    assert torch.equal(*outs)
