@@ -2,14 +2,15 @@
 //
 //   C[j][n] = sum_k X[j][k] * W[n][k]      (j < m active rows, n < N features)
 //
-// Orientation.  A tcgen05.mma instruction (K = 16) takes about 150 cycles
-// whatever its M and N, so a decode GEMM, bound by streaming W, must move as
-// many weight bytes per instruction as it can.  The active rows are therefore
-// the MMA's M side (one or two 128-row M-tiles; rows past m are never read
-// back) and a tile of bw = 256 weight rows is its N side: 8 KiB of weights per
-// instruction.  (With the weights as M and the rows as N, an instruction moves
-// 4 KiB and the instruction rate caps an SM's weight stream near 5 TB/s for
-// the whole GPU.)
+// Orientation.  A tcgen05.mma instruction (K = 16) takes 128 cycles at N = 256
+// and about 97, its issue rate, at N <= 128 (M = 64 or 128), so a decode GEMM,
+// bound by streaming W, must move as many weight bytes per instruction as it
+// can.  The active rows are therefore the MMA's M side (one or two 128-row
+// M-tiles; rows past m are never read back) and a tile of bw = 256 weight rows
+// is its N side: 8 KiB of weights per instruction, 20 TB/s over the GPU at one
+// M-tile.  (With the weights as M = 128 and the rows as N, an instruction moves
+// 4 KiB: 13 TB/s, and half that with the first layer's remainder terms, which
+// is less than HBM's rate.)
 //
 // A stage of the shared-memory ring holds, for one 64-column K block, the
 // activation region of each M-tile (then, for the first layer, the regions of
@@ -90,7 +91,7 @@ struct TcParams {
   float* q_out;
   float* pool;
   int nq, nkv, hd;
-  // Panel mode (at most 8 rows, K a multiple of 64): the activations are the
+  // Panel mode (at most kTcDeferRows rows, K a multiple of 64): the activations are the
   // RMSNorm of the fp32 rows nsrc[rows[j]] (width K), x = bf16(h * rsqrt(
   // mean(h^2) + neps) * ngamma) (+ remainder), computed by the epilogue warps
   // into a shared-memory panel holding the unit's K range (two panels, for the
@@ -189,7 +190,7 @@ __device__ __forceinline__ void tc_mma_stage(const uint8_t* st, uint32_t d, cons
 // following 15 KiB (later blocks, the next panel, or the tail slack): those
 // rows only feed accumulator rows that are discarded.
 // ---------------------------------------------------------------------------
-// 1 / rms of each row (m <= 8), by the 128 epilogue threads (et = 0..127): four
+// 1 / rms of each row, by the 128 epilogue threads (et = 0..127): four
 // rows at a time, eight float4 of each per thread in flight together (a row at a
 // time took 7 us for 7 rows of 4096).  A function of its own, so that the kernel
 // of one or two rows, which does not call it, stays short.

@@ -24,8 +24,9 @@
 // stages the accumulator of a part in a workspace slot, and the pair that
 // completes a unit sums the parts in K order and applies the epilogue.  With one
 // short prompt every unit is such a unit: Llama-3-8B's O projection has 16, which
-// kept 16 of the 76 pairs busy for 64 K blocks (61 tokens on a 4-block
-// Llama-3-8B: 0.85 -> 0.73 ms; 5 prompts, 2,878 tokens: 4.06 -> 3.93 ms).
+// kept 16 of the 76 pairs busy for 64 K blocks (4 blocks of Llama-3-8B, 5 prompts,
+// 2,878 tokens: 4.06 -> 3.93 ms; 61 tokens, which launch_gemm_pf now sends
+// elsewhere: 0.85 -> 0.73 ms).
 //
 // Warp 0 of each CTA issues the TMA loads of its part of a stage ([X 128 x 64]
 // [X remainder 128 x 64 with SPLIT][W 128 x 64], 128-byte swizzle; the bytes of
