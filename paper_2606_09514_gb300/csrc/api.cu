@@ -135,7 +135,7 @@ extern "C" int buddy_create(const buddy_config* cfg, buddy_ctx** out) {
       (e = dalloc(&c.attn_m, B * c.nq * c.attn_max_chunks)) ||
       (e = dalloc(&c.attn_l, B * c.nq * c.attn_max_chunks)) ||
       (e = dalloc(&c.attn_acc, B * c.nq * c.attn_max_chunks * c.hd)) ||
-      (e = dalloc(&c.attn_ctr, B * c.nkv)) ||
+      (e = dalloc(&c.attn_ctr, B * c.nkv + 2)) ||
       (e = dalloc(&c.dm_u, (size_t)kRouteZSlots * B * c.r)) || (e = route_prepare()) ||
       (e = dalloc(&c.mask, B * c.L)) ||
       (e = dalloc(&c.sel, B * c.Lm)) || (e = dalloc(&c.scores, B * c.Lm)) ||
@@ -148,7 +148,7 @@ extern "C" int buddy_create(const buddy_config* cfg, buddy_ctx** out) {
                    (e = cudaMalloc(&c.attn_lo, B * c.qd * c.esz))))
     return fail(e);
   if ((e = cudaMemset(c.status, 0, 4 * sizeof(int32_t))) != cudaSuccess ||
-      (e = cudaMemset(c.attn_ctr, 0, B * c.nkv * sizeof(int32_t))) != cudaSuccess)
+      (e = cudaMemset(c.attn_ctr, 0, (B * c.nkv + 2) * sizeof(int32_t))) != cudaSuccess)
     return fail(e);
   c.dm_u_cols = c.r;
   c.pf_max = g.max_prefill_tokens;
@@ -276,7 +276,7 @@ extern "C" int buddy_device_status(buddy_ctx* ctx, void* stream, int32_t* flags)
     // a GEMM that gave up left split-K arrival counters mid-count: re-arm them
     if (c.gemm_ctr) CK(cudaMemsetAsync(c.gemm_ctr, 0, c.gemm_ctr_n * sizeof(int32_t), s));
     if (c.pf_ctr) CK(cudaMemsetAsync(c.pf_ctr, 0, c.pf_ctr_n * sizeof(int32_t), s));
-    CK(cudaMemsetAsync(c.attn_ctr, 0, (size_t)c.maxB * c.nkv * sizeof(int32_t), s));
+    CK(cudaMemsetAsync(c.attn_ctr, 0, ((size_t)c.maxB * c.nkv + 2) * sizeof(int32_t), s));
   }
   CK(cudaStreamSynchronize(s));
   *flags = h[0];

@@ -55,7 +55,8 @@ static void attn_tc_impl(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int
   const int grid = c.num_sms * std::max(1, std::min(occ, 4));
   AttnArgs<bf16> A{q, sel.rows, sel.count, sel.n, c.nq, c.nkv, cache_len(c, kv, layer), kv.seq_off, kv.cap,
                    (const bf16*)kv.k_cache[layer], (const bf16*)kv.v_cache[layer], c.attn_max_chunks, c.attn_m,
-                   c.attn_l, c.attn_acc, c.attn_ctr, (bf16*)out, (bf16*)out_lo, c.status};
+                   c.attn_l, c.attn_acc, c.attn_ctr, (bf16*)out, (bf16*)out_lo, c.status,
+                   c.attn_ctr + (size_t)c.maxB * c.nkv};
   launch_k(attn_tc_kernel<HD, SPLIT>, grid, kTcaThreads, smem, s, c.pdl, A);
 }
 

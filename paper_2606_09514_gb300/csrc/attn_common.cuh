@@ -82,6 +82,7 @@ struct AttnArgs {
   T* out;
   T* out_lo;
   const int32_t* status;
+  int32_t* claim;   // attn_tc.cuh: units claimed, warps done (self-resetting)
 };
 
 // Dynamic shared memory used by attn_run (bytes): double-buffered K (rows

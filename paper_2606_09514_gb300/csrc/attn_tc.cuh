@@ -4,12 +4,24 @@
 // Work decomposition: the (row j, KV head g) streams of positions 0..len[i]
 // are laid end to end (row-major, heads inside a row) and every warp of the
 // grid takes an equal contiguous share of that sequence (a multiple of the
-// chunk, at least two chunks).  A share may end in the middle of a stream and
-// cover several short ones; the piece of a stream that one warp holds is a
-// span.  A stream held by one warp is written out directly; otherwise every
-// warp writes its span's partial (running max, sum of exponentials,
-// unnormalised output), and the warp that completes the stream last (an
-// arrival counter per stream) merges the partials in span order
+// chunk, at least two chunks).  SMs do not get equal shares of HBM's rate: with
+// all positions in equal shares, the warps of the slowest SM ended 16-20% after
+// the mean (Qwen2.5-7B, 256 rows: 150 us on the fastest, 191 us on average, 227
+// us on the slowest).  So where a warp's equal part is at least kTcaDynMin
+// positions, the shares hold three quarters of the sequence, and the rest is
+// cut into units of 1/12 of an equal part that warps claim one by one.  The
+// pieces are the same whoever takes them, and so are the results.  A unit's
+// partial, its arrival and its share of the merge cost a warp about 4 us: with
+// parts of 1,900 positions (Llama-3-8B, 64 rows) units made a step 3% slower, at
+// 3,800 (Qwen2.5-7B, 256 rows) no faster; 3 blocks of Llama-2-13B, 24 rows of
+// 4,090 positions (6,500 a part) 1393 -> 1349 us, 64 rows 2917 -> 2766 us; of
+// Llama-3-8B, 128 rows of 8,100 positions 2398 -> 2305 us.
+//
+// A share may end in the middle of a stream and cover several short ones; the
+// piece of a stream that one share or unit holds is a span.  A stream held by
+// one warp is written out directly; otherwise every warp writes its span's
+// partial (running max, sum of exponentials, unnormalised output), and the warp
+// that completes the stream last (an arrival counter per stream) merges the partials in span order
 // (deterministic), kTcaWarpMerge spans' loads at a time.  Because warps never
 // wait for each other, each streams its share without a break: the copies of
 // the next span are in flight while the current one finishes (or merges), and
@@ -49,7 +61,10 @@ constexpr int kTcaWarps = 4;
 constexpr int kTcaThreads = 32 * kTcaWarps;
 constexpr int kTcaStages = 3;     // chunk buffers per warp (kTcaStages - 1 in flight)
 constexpr int kTcaMinShare = 2 * kTcaChunk;   // positions of a warp's share, at least
-constexpr int kTcaWarpMerge = 4;              // span partials loaded at a time by the merging warp
+constexpr int kTcaDynMin = 6144;   // positions of an equal part from which a quarter is claimed in units
+constexpr int kTcaUnits = 12;      // units of an equal part
+constexpr int kTcaWarpMerge = 4;              // span partials loaded at a time by the merging warp,
+constexpr int kTcaMergeRounds = 4;            // of this many rounds of 32 lanes
 
 template <int HD>
 __host__ __device__ constexpr size_t attn_tc_smem_fixed() {
@@ -111,7 +126,7 @@ __device__ __forceinline__ float exp2a(float x) {
 }  // namespace tca
 
 // Merge of a (row j, KV head g)'s nsp span partials by one warp: lane ->
-// (head, four channels) per round of 32 lanes.  For two rounds at a time the
+// (head, four channels) per round of 32 lanes.  For kTcaMergeRounds rounds at a time the
 // partials (output, max and sum) of kTcaWarpMerge spans are loaded at once and
 // folded into a running max M, sum L and output O in span order (a group
 // raising M rescales what came before by 2^(M_old - M_new)); the result is
@@ -121,18 +136,24 @@ __device__ __forceinline__ void attn_tc_warp_merge(const AttnArgs<bf16>& A, int 
                                                    int lane) {
   constexpr int Q = HD / 4;      // float4 outputs per head
   constexpr int HPR = 32 / Q;    // heads per round (1 or 2)
-  constexpr int NS = kTcaWarpMerge;
+  constexpr int NS = kTcaWarpMerge, NU = kTcaMergeRounds;
   const int G = A.nq / A.nkv, ms = A.max_spans;
   const size_t hb0 = ((size_t)j * A.nq + (size_t)g * G) * ms;
   const int hsub = lane / Q, e0 = (lane % Q) * 4;
-  for (int r0 = 0; r0 * HPR < G; r0 += 2) {
-    float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f};
-    float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-    for (int s0 = 0; s0 < nsp; s0 += NS) {
-      float4 v[2][NS];
-      float mv[2][NS], lv[2][NS];
+  for (int r0 = 0; r0 * HPR < G; r0 += NU) {
+    float M[NU], L[NU];
+    float4 acc[NU];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+    for (int u = 0; u < NU; ++u) {
+      M[u] = -INFINITY;
+      L[u] = 0.f;
+      acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int s0 = 0; s0 < nsp; s0 += NS) {
+      float4 v[NU][NS];
+      float mv[NU][NS], lv[NU][NS];
+#pragma unroll
+      for (int u = 0; u < NU; ++u) {
         const int h = (r0 + u) * HPR + hsub;
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
@@ -145,7 +166,7 @@ __device__ __forceinline__ void attn_tc_warp_merge(const AttnArgs<bf16>& A, int 
         }
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < NU; ++u) {
         const int h = (r0 + u) * HPR + hsub;
         if (h >= G) continue;
         float mn = M[u];
@@ -174,7 +195,7 @@ __device__ __forceinline__ void attn_tc_warp_merge(const AttnArgs<bf16>& A, int 
       }
     }
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
+    for (int u = 0; u < NU; ++u) {
       const int h = (r0 + u) * HPR + hsub;
       if (h >= G) continue;
       const float inv = 1.f / L[u];
@@ -248,13 +269,23 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
       pref[0] = 0;
       const int nw = ncta * kTcaWarps;
       const int even = (carry + nw - 1) / nw;
-      sc[0] = max(kTcaMinShare, (even + CH - 1) / CH * CH);
+      if (even >= kTcaDynMin) {
+        sc[0] = (even / 4 * 3 + CH - 1) / CH * CH;
+        sc[1] = nw * sc[0];   // below carry
+        sc[2] = max(kTcaMinShare, (even / kTcaUnits + CH - 1) / CH * CH);
+      } else {
+        sc[0] = max(kTcaMinShare, (even + CH - 1) / CH * CH);
+        sc[1] = carry;
+        sc[2] = kTcaMinShare;
+      }
     }
   }
   __syncthreads();
   const int share = sc[0];
   const int total = pref[m];
-  const int gw = cta * kTcaWarps + warp;
+  const int gw = cta * kTcaWarps + warp, nw = ncta * kTcaWarps;
+  const int dyn0 = sc[1], unit = sc[2];   // units: from position dyn0 on
+  const int n_units = (total - dyn0 + unit - 1) / unit;
   const long long a0 = (long long)gw * share;
   if (a0 >= total) {   // nothing for this warp
     if (pdl) {
@@ -263,7 +294,7 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
     }
     return;
   }
-  const int a = (int)a0, b = min(total, a + share);
+  const int a = (int)a0, b = min(total, a + share);   // (total: without units only)
 
   // cursor at flattened position x (binary search of the row prefix)
   auto seek = [&](int x) {
@@ -282,7 +313,9 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
     return c;
   };
   // positions of the chunk at cursor c (flattened position x)
-  auto chunk_len = [&](const TcaCursor& c, int x) { return min(CH, min(c.np - c.p, b - x)); };
+  auto chunk_len = [&](const TcaCursor& c, int x, int end) { return min(CH, min(c.np - c.p, end - x)); };
+  // the share or unit of flattened position x
+  auto piece = [&](int x) { return x < dyn0 ? x / share : nw + (x - dyn0) / unit; };
   // advance past a chunk of n positions (never beyond the stream end)
   auto advance = [&](TcaCursor& c, int n) {
     c.p += n;
@@ -325,7 +358,7 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
   int k0 = 0;
   if (pdl) {
     for (; k0 < NST - 1 && xi < b; ++k0) {
-      const int cnt = chunk_len(ci, xi);
+      const int cnt = chunk_len(ci, xi, b);
       if (ci.p + cnt == ci.np) break;
       issue(ci, cnt, k0);
       cp_async_commit();
@@ -335,33 +368,55 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
     pdl_wait();
     pdl_trigger();
   }
-  for (int k = k0; k < NST - 1; ++k) {
-    if (xi < b) {
-      const int cnt = chunk_len(ci, xi);
-      issue(ci, cnt, k);
+  // The next chunk's copies; past the end of its share or unit the warp goes on
+  // to the unit it claimed when a last chunk was left to copy (the claim's
+  // latency passes while the chunks in flight are used).  Units have at least
+  // two chunks (but for the last of all), so copies are never more than one
+  // unit ahead of the chunk in use.
+  bool more = n_units > 0, claimed = false;
+  int claim = 0, bi = b;            // claim: lane 0's
+  TcaCursor cn = ci;                // the unit the copies went on to: its cursor,
+  int xn = 0, bn = 0, un = gw;      // range and number
+  auto issue_next = [&](int buf) {
+    if (xi == bi && more) {
+      const int id = __shfl_sync(0xffffffffu, claim, 0);
+      claimed = false;
+      if (id < n_units) {
+        xi = xn = dyn0 + id * unit;
+        bi = bn = min(total, xi + unit);
+        ci = cn = seek(xi);
+        un = nw + id;
+      } else {
+        more = false;
+      }
+    }
+    if (xi < bi) {
+      const int cnt = chunk_len(ci, xi, bi);
+      issue(ci, cnt, buf);
       advance(ci, cnt);
       xi += cnt;
+      if (more && !claimed && bi - xi <= CH) {
+        if (lane == 0) claim = atomicAdd(A.claim, 1);
+        claimed = true;
+      }
     }
     cp_async_commit();
-  }
+  };
+  for (int k = k0; k < NST - 1; ++k) issue_next(k);
 
   const float scale = 1.4426950408889634f * rsqrtf((float)HD);   // log2(e) / sqrt(d_h)
   const int h0 = lane >> 2, c2 = (lane & 3) * 2;   // fragment row (head) and column pair
   TcaCursor cc = seek(a);
-  int xc = a;
+  int xc = a, bc = b, uc = gw;
+  bool fresh = true;        // the chunk begins a share or unit
   uint32_t qh[KSTEPS][2], ql[KSTEPS][2];
   float mrun[2], lrun[2];   // heads c2, c2 + 1
   float o[DT / 2][4];       // O^T: channels 16 * t + lane / 4 (+8) x heads c2, c2 + 1
-  for (int k = 0; xc < b; ++k) {
-    if (xi < b) {
-      const int cnt = chunk_len(ci, xi);
-      issue(ci, cnt, (k + NST - 1) % NST);
-      advance(ci, cnt);
-      xi += cnt;
-    }
-    cp_async_commit();
-    const int cnt = chunk_len(cc, xc);
-    if (xc == a || cc.p == 0) {
+  for (int k = 0; xc < bc; ++k) {
+    issue_next((k + NST - 1) % NST);
+    const int cnt = chunk_len(cc, xc, bc);
+    if (fresh || cc.p == 0) {
+      fresh = false;
       // a new span: query fragments as the B operand (column = head h0 < G,
       // rows = dims), scaled by log2(e) / sqrt(d_h), and a fresh running state
       const float* qj = A.q + ((size_t)cc.j * nq + (size_t)cc.g * G + h0) * HD;
@@ -485,11 +540,11 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
     const TcaCursor cs = cc;   // the span this chunk belongs to
     advance(cc, cnt);
     xc += cnt;
-    if (cs.p + cnt == cs.np || xc == b) {
+    if (cs.p + cnt == cs.np || xc == bc) {
       // end of the span: its stream covers flattened [S0, S0 + np), cut by the
-      // shares into spans first .. last (this warp's is gw - first)
+      // shares and units into spans first .. last (this one is uc - first)
       const int S0 = pref[cs.j] + cs.g * cs.np;
-      const int first = S0 / share, nsp = (S0 + cs.np - 1) / share - first + 1;
+      const int first = piece(S0), nsp = piece(S0 + cs.np - 1) - first + 1;
       const size_t obase = ((size_t)cs.j * nq + (size_t)cs.g * G) * HD;
       // this lane: heads c2 + e (e = 0, 1), channels 16 t + h0 (+ 8)
       if (nsp == 1) {
@@ -506,7 +561,7 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
           }
         }
       } else {   // a partial, merged by the warp that completes the stream
-        const int sp = gw - first;
+        const int sp = uc - first;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           if (c2 + e < G) {
@@ -538,7 +593,17 @@ __device__ __forceinline__ void attn_tc_run(const AttnArgs<bf16>& A, int cta, in
         if (last) attn_tc_warp_merge<HD>(A, cs.j, cs.g, nsp, obase, lane);
       }
     }
+    if (xc == bc && un != uc) {   // on to the unit whose chunks are in flight
+      cc = cn;
+      xc = xn;
+      bc = bn;
+      uc = un;
+      fresh = true;
+    }
   }
+  // every warp has claimed past the last unit when the last one gets here: the
+  // counters are re-armed for a later launch
+  if (n_units > 0 && lane == 0 && atomicAdd(A.claim + 1, 1) == nw - 1) A.claim[0] = A.claim[1] = 0;
 }
 
 }  // namespace buddy

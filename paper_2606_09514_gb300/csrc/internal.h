@@ -222,7 +222,7 @@ struct Ctx {
   float* attn_m = nullptr;     // [maxB, nq, max_chunks]
   float* attn_l = nullptr;
   float* attn_acc = nullptr;   // [maxB, nq, max_chunks, hd]
-  int32_t* attn_ctr = nullptr; // [maxB, nkv] chunk arrivals (self-resetting)
+  int32_t* attn_ctr = nullptr; // [maxB, nkv] chunk arrivals, then 2 of the unit claims (self-resetting)
   float* dm_u = nullptr;       // [kRouteZSlots, maxB, r + predictor hidden] partial sums
   uint8_t* mask = nullptr;     // [maxB, L]
   int32_t* sel = nullptr;      // [maxB, Lm]

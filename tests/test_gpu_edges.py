@@ -5,11 +5,14 @@ small-batch decode modes and attention cluster sizes, the fp32 GEMMs, the router
 and the bulk append's own argument checks, and the wait limits of these paths.
 Values are compared with the float64 oracle at the bounds of parity.py.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
 
 import paper_2606_09514_gb300 as pkg
+import test_gpu_fullsize as FS
 from paper_2606_09514_gb300 import binding as Bd
 from test_gpu_decode import run_parity
 from test_gpu_prefill import run_prefill_parity
@@ -48,6 +51,17 @@ def test_prefill_parity_at_tile_edges(base, lengths, ctx):
                                         (C.T_GQA, 21)], ids=lambda v: v.shape.name if hasattr(v, "shape") else str(v))
 def test_decode_parity_small_batch_modes(base, batch):
     assert run_parity(rows_of(base, batch), steps=2)[0] < 2e-2
+
+
+# 6144 positions per warp or more: a quarter of them claimed in units; short and long
+# streams in turn, one row of every part of the sequence checked
+def test_decode_parity_claimed_units():
+    base = C.P_QWEN_3L_B256
+    ctx = [7600 - 3 * i if i % 2 else 5 + 11 * i // 2 for i in range(256)]
+    warps = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    assert base.shape.n_kv_heads * sum(ctx) >= 6144 * warps
+    w = dataclasses.replace(C.scaled(base, ctx=ctx, k=[1] * 256, name="qwen2.5-7b-3layer-units"), steps=2)
+    FS.test_fullsize_trajectory_parity(w, [0, 1, 100, 201, 254, 255])
 
 
 # fp32: four or eight rows per pass (4, 5), norms and QKV finalisation inside the
