@@ -860,18 +860,18 @@ __global__ void __launch_bounds__(256) kv_append_vec_kernel(int n_new, int nkv, 
 }
 
 // Pooled context of a sequence, recomputed: the sum of the planner feature over
-// the context layer's first len + n_new positions.  A cluster of kPoolCtas CTAs
-// per (KV head, sequence), each over a contiguous share of the positions: a
+// the context layer's first len + n_new positions.  A cluster of NC CTAs per (KV
+// head, sequence), each over a contiguous share of the positions: a
 // thread takes 16 bytes of a position (E channels) and every (threads per
 // position)-th position, four loads in flight; the CTA's sums meet in shared
 // memory and CTA 0 adds the CTAs' sums in rank order (the same order on every
 // run).  Bound by HBM and by latency: 6 sequences of 1,100 positions of 8 heads
 // from cold caches in 20 us, against 128 us with one thread per channel (5
 // prompts of 128..1023 tokens just written: 12 us against 121 us).
-constexpr int kPoolCtas = 8;
+constexpr int kPoolCtas = 8;   // NC with few (KV head, sequence) pairs; else 1
 constexpr int kPoolThreads = 512;
-template <typename T>
-__global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(kPoolThreads)
+template <typename T, int NC>
+__global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kPoolThreads)
     pool_refresh_kernel(int n_new, const int32_t* n_new_of, int nkv, int hd, int feature, const int32_t* ids,
                         const int32_t* len, const int64_t* seq_off, const int32_t* cap, const T* K0, const T* V0,
                         float* pool, const int32_t* status) {
@@ -880,11 +880,11 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(kPoolThreads
   if (call_aborted(status)) return;   // the same in every CTA of the cluster
   constexpr int E = 16 / sizeof(T), U = 4;
   __shared__ __align__(16) float part[kPoolThreads * E];   // [threads per piece][hd]
-  __shared__ float sums[kPoolCtas * 128];                  // CTA 0: the CTAs' sums
+  __shared__ float sums[NC * 128];                         // CTA 0: the CTAs' sums
   const int g = blockIdx.y, s = ids ? ids[blockIdx.z] : blockIdx.z;
   const int rank = (int)ptx::cluster_rank();
   const int n = len[s] + (n_new_of ? n_new_of[s] : n_new);
-  const int p0 = (int)((int64_t)n * rank / kPoolCtas), p1 = (int)((int64_t)n * (rank + 1) / kPoolCtas);
+  const int p0 = (int)((int64_t)n * rank / NC), p1 = (int)((int64_t)n * (rank + 1) / NC);
   const int ph = hd / E, lanes = kPoolThreads / ph;   // pieces of a position, positions at a time
   const int c = threadIdx.x % ph, w = threadIdx.x / ph;
   const int64_t off = kv_offset(seq_off, cap, s, nkv, hd, g, 0) + c * E;
@@ -926,7 +926,7 @@ __global__ void __cluster_dims__(kPoolCtas, 1, 1) __launch_bounds__(kPoolThreads
   ptx::cluster_sync();
   if (rank == 0 && threadIdx.x < hd) {
     float v = 0.f;
-    for (int i = 0; i < kPoolCtas; ++i) v += sums[i * hd + threadIdx.x];
+    for (int i = 0; i < NC; ++i) v += sums[i * hd + threadIdx.x];
     pool[(size_t)s * nkv * hd + g * hd + threadIdx.x] = v;
   }
 }
@@ -964,8 +964,12 @@ template <typename T>
 static void pool_refresh_impl(const Ctx& c, const buddy_kv_state& kv, int n_seq, const int32_t* ids, int n_new,
                               const int32_t* n_new_of, cudaStream_t s) {
   const int l = c.cl;
-  const dim3 g(kPoolCtas, c.nkv, n_seq);
-  launch_k(pool_refresh_kernel<T>, g, kPoolThreads, 0, s, c.pdl, n_new, n_new_of, c.nkv, c.hd, c.feature, ids,
+  // Clusters while they fit the GPU at once (four CTAs per SM); with more pairs a
+  // CTA each: whole calls over three layers with 40 heads, 32 sequences of 2
+  // positions 210 -> 44 us, 8 heads, 19 sequences of 750 positions 83 -> 67 us.
+  const bool few = (int64_t)n_seq * c.nkv * kPoolCtas <= 4 * c.num_sms;
+  launch_k(few ? pool_refresh_kernel<T, kPoolCtas> : pool_refresh_kernel<T, 1>, dim3(few ? kPoolCtas : 1, c.nkv, n_seq),
+           kPoolThreads, 0, s, c.pdl, n_new, n_new_of, c.nkv, c.hd, c.feature, ids,
            cache_len(c, kv, l), kv.seq_off, kv.cap, (const T*)kv.k_cache[l], (const T*)kv.v_cache[l], kv.pool_sum,
            (const int32_t*)c.status);
 }
