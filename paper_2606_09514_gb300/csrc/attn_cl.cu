@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
     pdl_trigger();
     return;
   }
+  ptx::cluster_arrive_started();
   const uint32_t rank = ptx::cluster_rank(), C = ptx::cluster_size();
   const int i = A.rows ? A.rows[j] : j;
   const int np = A.len[i] + 1;   // cached positions and the new token
@@ -311,6 +312,7 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
     }
   }
   __syncthreads();
+  ptx::cluster_wait_started();
   // the CTA's partial, the warps' partials merged per (head, channel), stored
   // into the gather area of the output's owner (slot `rank`), four channels
   // per thread and per 16-byte store (a slice is a multiple of 4 outputs:

@@ -878,6 +878,7 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kPoolThreads)
   pdl_wait();
   pdl_trigger();
   if (call_aborted(status)) return;   // the same in every CTA of the cluster
+  if constexpr (NC > 1) ptx::cluster_arrive_started();
   constexpr int E = 16 / sizeof(T), U = 4;
   __shared__ __align__(16) float part[kPoolThreads * E];   // [threads per piece][hd]
   __shared__ float sums[NC * 128];                         // CTA 0: the CTAs' sums
@@ -916,6 +917,7 @@ __global__ void __cluster_dims__(NC, 1, 1) __launch_bounds__(kPoolThreads)
 #pragma unroll
   for (int e = 0; e < E; ++e) part[w * hd + c * E + e] = acc[e];
   __syncthreads();
+  if constexpr (NC > 1) ptx::cluster_wait_started();
   if (threadIdx.x < hd) {
     float v = 0.f;
     for (int i = 0; i < lanes; ++i) v += part[i * hd + threadIdx.x];

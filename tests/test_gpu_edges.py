@@ -159,6 +159,32 @@ def test_append_aligned_and_misaligned(shape, n_new, n_seq):
     assert states[0][1].buddy_device_status() & Bd.BUDDY_DEV_BAD_SEQ and torch.equal(a.k[0], k0)
 
 
+# clusters of 8 CTAs over 1 to 9 positions: CTAs with an empty share reach their
+# stores to CTA 0 at once
+@pytest.mark.parametrize("shape", [C.SMALL_GQA_BF16, C.SMALL_QWEN_BF16, C.SMALL_F32], ids=lambda s: s.name)
+@pytest.mark.parametrize("n_new", [1, 2, 7, 9])
+def test_pooled_context_of_shares_shorter_than_the_cluster(shape, n_new):
+    g = torch.Generator(device="cuda").manual_seed(n_new)
+    ids = torch.tensor([0, 1], dtype=torch.int32, device="cuda")
+    kn, vn = (torch.empty(2, n_new, shape.n_kv_heads, shape.head_dim, dtype=synth.storage_dtype(shape),
+                          device="cuda").normal_(generator=g) for _ in range(2))
+    ctx, kv = append_state(shape, [n_new, n_new], 2)
+    pools = []
+    for _ in range(20):
+        ctx.buddy_kv_append(kv, 0, ids, kn, vn, advance=False)
+        pools.append(kv.pool_sum.clone())
+    assert ctx.buddy_device_status() == 0
+    np.testing.assert_allclose(pools[0].double().cpu(), vn.double().sum(1).reshape(2, -1).cpu(), rtol=1e-5, atol=1e-5)
+    assert all(torch.equal(p, pools[0]) for p in pools)
+
+
+# attention clusters of 16 to 2 CTAs over 1 to 4 positions
+@pytest.mark.parametrize("batch", [1, 2, 5, 10, 21])
+def test_decode_parity_shares_shorter_than_the_cluster(batch):
+    w = C.scaled(C.T_GQA, ctx=[i % 4 for i in range(batch)], k=[1 + i % 4 for i in range(batch)], name="short-ctx")
+    assert run_parity(w, steps=2)[0] < 2e-2
+
+
 def test_panel_wait_limit_runs_out_and_context_recovers():
     """As the other batches' test: 1 ns runs out, the restored limit gives a fresh context's result."""
     w = C.scaled(C.T_GQA, ctx=[5, 200], k=[1, 3], name="t-gqa-b2-timeout")
