@@ -319,18 +319,15 @@ void launch_pool_update(const Ctx& c, int B, const buddy_kv_state& kv, cudaStrea
 // (route_gemm_kernel): a tiled fp32 GEMM whose K splits leave
 // partial sums that part 2 adds in split order.
 // ---------------------------------------------------------------------------
-// The checks of a routing call, by every CTA: whether any failed.
-__device__ __forceinline__ bool route_check(const RouteCheck& c) {
+// The checks of a routing call (at most blockDim.x sequences): this thread's error bits.
+__device__ __forceinline__ int route_check(const RouteCheck& c) {
   int b = 0;
-  for (int i = threadIdx.x; i < c.B; i += blockDim.x) {
-    const int ki = c.k[i], n = c.len[i];
+  if (threadIdx.x < c.B) {
+    const int ki = c.k[threadIdx.x], n = c.len[threadIdx.x];
     if (ki < c.k_min || ki > c.Lm) b |= BUDDY_DEV_BAD_BUDGET;
-    if (n < 0 || n > c.cap[i] || n > c.max_pos) b |= BUDDY_DEV_BAD_POSITION;
+    if (n < 0 || n > c.cap[threadIdx.x] || n > c.max_pos) b |= BUDDY_DEV_BAD_POSITION;
   }
-  const int bad = (__syncthreads_or(b & BUDDY_DEV_BAD_BUDGET) ? BUDDY_DEV_BAD_BUDGET : 0) |
-                  (__syncthreads_or(b & BUDDY_DEV_BAD_POSITION) ? BUDDY_DEV_BAD_POSITION : 0);
-  if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) publish_checks(c.out, bad);
-  return bad != 0;
+  return b;
 }
 
 constexpr int kRouteRows = 8;
@@ -339,14 +336,22 @@ constexpr int kRtBM = 64, kRtBN = 64, kRtBK = 32;
 constexpr int kRtStages = 4, kRtRow = kRtBK + 4;   // buffers, floats from one row to the next
 constexpr int kRtSmem = kRtStages * (kRtBM + kRtBN) * kRtRow * 4;
 
-__global__ void __launch_bounds__(256) route_hidden_kernel(
+// CHECK: the first kernel of a routing call, which checks its arguments.  The
+// verdict falls after the products (they read nothing that a bad budget or length
+// could move out of bounds) and before the sums are written: checked first, the
+// arguments' loads and two barriers stood before all others, which at 16 rows of
+// 5120 channels cost more than the check kernel saved (30.6 us a call with a check
+// kernel, 33.5 us checked first, 29.0 us so; one row of 4096 12.8, 10.8, 10.8 us).
+template <bool CHECK>
+__device__ __forceinline__ void route_hidden(
     int B, int d, int hd, int group, int nkv, const float* __restrict__ h1,
     const float* __restrict__ pool, const int32_t* len, int len_bias, const float* __restrict__ w1,
     const float* __restrict__ b1, int r, const float* __restrict__ pw1, const float* __restrict__ pb1, int rp,
-    float* __restrict__ u, const int32_t* status, const RouteCheck chk) {
+    float* __restrict__ u, const int32_t* status, const RouteCheck& chk) {
   pdl_wait();
   pdl_trigger();
-  if (chk.out ? route_check(chk) : call_aborted(status)) return;
+  if (!CHECK && call_aborted(status)) return;
+  const int mine = CHECK ? route_check(chk) : 0;
   __shared__ float red[8][kRouteRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int unit = blockIdx.x;
@@ -391,7 +396,14 @@ __global__ void __launch_bounds__(256) route_hidden_kernel(
 #pragma unroll
     for (int t = 0; t < kRouteRows; ++t) red[warp][t] = acc[t];
   }
-  __syncthreads();
+  if (CHECK) {
+    const int bad = (__syncthreads_or(mine & BUDDY_DEV_BAD_BUDGET) ? BUDDY_DEV_BAD_BUDGET : 0) |
+                    (__syncthreads_or(mine & BUDDY_DEV_BAD_POSITION) ? BUDDY_DEV_BAD_POSITION : 0);
+    if (threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) publish_checks(chk.out, bad);
+    if (bad) return;
+  } else {
+    __syncthreads();
+  }
   if (threadIdx.x < nr) {
     const int t = threadIdx.x;
     float v = 0.f;
@@ -399,6 +411,22 @@ __global__ void __launch_bounds__(256) route_hidden_kernel(
     for (int w = 0; w < 8; ++w) v += red[w][t];
     u[(size_t)(i0 + t) * (r + rp) + unit] = v;
   }
+}
+
+__global__ void __launch_bounds__(256) route_hidden_kernel(
+    int B, int d, int hd, int group, int nkv, const float* __restrict__ h1,
+    const float* __restrict__ pool, const int32_t* len, int len_bias, const float* __restrict__ w1,
+    const float* __restrict__ b1, int r, const float* __restrict__ pw1, const float* __restrict__ pb1, int rp,
+    float* __restrict__ u, const int32_t* status) {
+  route_hidden<false>(B, d, hd, group, nkv, h1, pool, len, len_bias, w1, b1, r, pw1, pb1, rp, u, status, RouteCheck{});
+}
+
+__global__ void __launch_bounds__(256) route_hidden_check_kernel(
+    int B, int d, int hd, int group, int nkv, const float* __restrict__ h1,
+    const float* __restrict__ pool, const int32_t* len, int len_bias, const float* __restrict__ w1,
+    const float* __restrict__ b1, int r, const float* __restrict__ pw1, const float* __restrict__ pb1, int rp,
+    float* __restrict__ u, const RouteCheck chk) {
+  route_hidden<true>(B, d, hd, group, nkv, h1, pool, len, len_bias, w1, b1, r, pw1, pb1, rp, u, nullptr, chk);
 }
 
 // Router part 1 for larger batches: Z[i][unit] = X[i] . W[unit] over one K split,
@@ -630,9 +658,14 @@ void launch_route(const Ctx& c, int B, const float* h1, const float* pool, const
   const int splits = route_splits(c, B);
   if (B <= kRouteTiledMin) {
     dim3 g1(cols, (B + kRouteRows - 1) / kRouteRows);
-    launch_k(route_hidden_kernel, g1, 256, 0, s, c.pdl, B, c.d, c.hd, c.nq / c.nkv, c.nkv, h1, pool, len,
-             len_bias, c.dm.w1, c.dm.b1, c.r, c.have_pred ? c.pred.w1 : nullptr, c.have_pred ? c.pred.b1 : nullptr,
-             rp, c.dm_u, (const int32_t*)c.status, chk);
+    const float* pw1 = c.have_pred ? c.pred.w1 : nullptr;
+    const float* pb1 = c.have_pred ? c.pred.b1 : nullptr;
+    if (chk.out)
+      launch_k(route_hidden_check_kernel, g1, 256, 0, s, c.pdl, B, c.d, c.hd, c.nq / c.nkv, c.nkv, h1, pool, len,
+               len_bias, c.dm.w1, c.dm.b1, c.r, pw1, pb1, rp, c.dm_u, chk);
+    else
+      launch_k(route_hidden_kernel, g1, 256, 0, s, c.pdl, B, c.d, c.hd, c.nq / c.nkv, c.nkv, h1, pool, len,
+               len_bias, c.dm.w1, c.dm.b1, c.r, pw1, pb1, rp, c.dm_u, (const int32_t*)c.status);
   } else {
     const int half = splits / 2;
     const int kps = ((c.d + half - 1) / half + kRtBK - 1) / kRtBK * kRtBK;

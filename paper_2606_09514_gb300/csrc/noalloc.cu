@@ -15,7 +15,7 @@ namespace buddy {
 __global__ void route_hidden_kernel(int B, int d, int hd, int group, int nkv, const float* h1,
                                     const float* pool, const int32_t* len, int len_bias,
                                     const float* w1, const float* b1, int r, const float* pw1,
-                                    const float* pb1, int rp, float* u, const int32_t* status, const RouteCheck chk);
+                                    const float* pb1, int rp, float* u, const int32_t* status);
 __global__ void route_select_kernel(int Lm, int first, int r, int rp, const float* z, int splits, int B,
                                     const float* b1, const float* w2, const float* b2, const float* prior,
                                     float omega, const float* pb1, const float* pw2, const float* pb2,
@@ -98,7 +98,7 @@ extern "C" int buddy_route_noalloc(int32_t n_layers, int32_t d_model, int32_t n_
   dim3 g1(dm_hidden, (batch + 7) / 8);
   route_hidden_kernel<<<g1, 256, 0, s>>>(batch, d_model, head_dim, n_q_heads / n_kv_heads, n_kv_heads,
                                          h1, pool_sum, len, 0, dm->w1, dm->b1, dm_hidden, nullptr, nullptr, 0,
-                                         u, status, RouteCheck{});
+                                         u, status);
   const int sel_threads = 32 * (Lm < 32 ? Lm : 32);
   route_select_kernel<<<batch, sel_threads, (2 * Lm + dm_hidden) * sizeof(float), s>>>(
       Lm, 1, dm_hidden, 0, u, 1, batch, dm->b1, dm->w2, dm->b2, dm->prior, dm->omega, nullptr, nullptr, nullptr, k,

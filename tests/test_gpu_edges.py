@@ -113,6 +113,27 @@ def test_route_checks_write_nothing():
     assert dw.ctx.buddy_device_status() == 0 and not bool((sc == 7.0).any())
 
 
+# two groups of rows (the first kernel checks after its products), the bad row in the second
+def test_route_checks_write_nothing_two_row_groups():
+    w = rows_of(C.T_GQA, 16)
+    dw = D.build(w)
+    s = w.shape
+    h1 = synth.h_in(s, 5, 0, range(16), "cuda")
+    dw.kv.len.clamp_(min=1)
+    sc, sel = torch.full((16, s.n_cand), 7.0, device="cuda"), torch.full((16, s.n_cand), 7, dtype=torch.int32, device="cuda")
+    bad = dw.k.clone()
+    bad[15] = s.n_cand + 1
+    good_len = dw.kv.len.clone()
+    for k, length, flag in ((bad, good_len[15], Bd.BUDDY_DEV_BAD_BUDGET), (dw.k, dw.kv.cap[15] + 1, Bd.BUDDY_DEV_BAD_POSITION),
+                            (bad, -1, Bd.BUDDY_DEV_BAD_BUDGET | Bd.BUDDY_DEV_BAD_POSITION)):
+        dw.kv.len[15] = length
+        dw.ctx.buddy_route(dw.kv, h1, k, sel_out=sel, scores_out=sc)
+        assert dw.ctx.buddy_device_status() == flag and bool((sc == 7.0).all()) and bool((sel == 7).all())
+    dw.kv.len.copy_(good_len)
+    dw.ctx.buddy_route(dw.kv, h1, dw.k, sel_out=sel, scores_out=sc)
+    assert dw.ctx.buddy_device_status() == 0 and not bool((sc == 7.0).any())
+
+
 def append_state(shape, caps, max_batch):
     ctx = pkg.Context.for_shape(shape, max_batch=max_batch, max_pos=max(caps))
     layer = pkg.pack_layer(synth.layer_weights(shape, 0, 0, "cuda"))
