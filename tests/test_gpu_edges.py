@@ -113,6 +113,51 @@ def test_route_checks_write_nothing():
     assert dw.ctx.buddy_device_status() == 0 and not bool((sc == 7.0).any())
 
 
+def silu_context(r, n_layers):
+    """A router whose scores are silu(x + b1) of the first r channels x of h1."""
+    s = dataclasses.replace(C.SMALL_F32, n_layers=n_layers, dm_hidden=r)
+    ctx = pkg.Context.for_shape(s, max_batch=256, max_pos=4)
+    layer = pkg.pack_layer(synth.layer_weights(s, 0, 0, "cuda"))
+    dm = {"w1": torch.zeros(r, 2 * s.d_model, device="cuda"), "b1": torch.zeros(r, device="cuda"),
+          "w2": torch.eye(s.n_cand, r, device="cuda"), "b2": torch.zeros(s.n_cand, device="cuda")}
+    dm["w1"][:, s.d_model:s.d_model + r] = torch.eye(r, device="cuda")
+    kv = pkg.KVCache(s.n_layers, s.n_kv_heads, s.head_dim, [1] * 256, torch.float32, "cuda")
+    kv.len.fill_(1)
+    h1, k = torch.zeros(256, s.d_model, device="cuda"), torch.ones(256, dtype=torch.int32, device="cuda")
+    scores = torch.empty(256, s.n_cand, device="cuda")
+
+    def run(x=None, b1=None):
+        if x is not None:
+            h1[:, :r] = x
+        if b1 is not None:
+            dm["b1"].fill_(b1)
+        ctx.buddy_set_weights([layer] * s.n_layers, dm)
+        ctx.buddy_route(kv, h1, k, scores_out=scores)
+        assert ctx.buddy_device_status() == 0
+        return scores
+    return run
+
+
+def test_silu_is_the_division():
+    """silu(x) over the float range: at most an ulp from the device's own x / (1 + e^-x), where 1 + e^-x
+    passes 1e38 (x below -87.5) and overflows (below -88.7) included."""
+    run = silu_context(126, 128)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    n = 256 * 126
+    bits = torch.randint(-2**31, 2**31 - 1, (n,), generator=g, device="cuda").int().view(torch.float32)
+    for x in (bits.nan_to_num(0.5, 3e38, -3e38), torch.linspace(-89, -87, n, device="cuda"),
+              torch.linspace(-110, 30, n, device="cuda"), torch.linspace(-1, 1, n, device="cuda")):
+        x = x.view(256, 126)
+        got, ref = run(x), x / (1.0 + torch.exp(-x))
+        ulp = torch.maximum((torch.nextafter(ref.abs(), ref.new_tensor(float("inf"))) - ref.abs()), ref.new_tensor(2.0**-149))
+        assert bool(((got - ref).abs() <= ulp).all()), float(((got - ref).abs() / ulp).max())
+    one = silu_context(1, 3)
+    for b in (float("inf"), float("-inf"), float("nan"), 3.4e38, -3.4e38, -88.72, -88.73, -0.0):
+        x = torch.tensor(b, device="cuda")
+        ref = float(x / (1.0 + torch.exp(-x)))
+        np.testing.assert_allclose(one(b1=b)[:, 0].cpu().numpy(), np.float32(ref), rtol=1.2e-7, atol=0)
+
+
 # two groups of rows (the first kernel checks after its products), the bad row in the second
 def test_route_checks_write_nothing_two_row_groups():
     w = rows_of(C.T_GQA, 16)
