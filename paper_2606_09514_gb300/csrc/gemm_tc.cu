@@ -423,11 +423,17 @@ static int choose_splits(int tiles, int kb, int sms) {
 // itself, without workspace or fixup kernel: taken when its tiles keep at least
 // 70% of the SMs streaming (the rest of HBM's rate they reach all the same:
 // Llama-3-8B's 112 tiles at 64 rows take as long as 448 units, and the 10 us
-// fixup is saved; 6 blocks 1259 -> 1209 us).
+// fixup is saved; 6 blocks 1259 -> 1209 us).  Not in a decode block that feeds the
+// router (hi + lo activations): its sums would run over the whole K in one fp32
+// accumulator, four times as long as with the splits, and the scores' error against
+// 64 bits doubled (Llama-3-8B, 3 to 200 rows: 1.0e-5 -> 2.2e-5 of their size).
 static int defer_splits(int which, int tiles, int kb, int sms) {
   if (which == 2 && 10 * tiles >= 7 * sms && tiles <= sms) return 1;
   return choose_splits(tiles, kb, sms);
 }
+
+// K splits of projection `which` of a decode block.
+int gemm_tc_splits(const Ctx& c, int which, bool split) { return c.tc_splits[split ? 1 : 0][which]; }
 
 // bf16 shapes always take the tensor-core path: sm_103 and at most 256 rows
 // (buddy_create rejects anything else).
@@ -465,10 +471,11 @@ int gemm_tc_prepare(Ctx& c) {
     int N, K, tiles;
     gemm_shape(c, w, &N, &K, &tiles);
     const int kb = (K + kTileK - 1) / kTileK;
-    c.tc_splits[w] = c.maxB > kTcDeferRows ? defer_splits(w, tiles, kb, c.num_sms) : choose_splits(tiles, kb, c.num_sms);
+    c.tc_splits[1][w] = choose_splits(tiles, kb, c.num_sms);
+    c.tc_splits[0][w] = c.maxB > kTcDeferRows ? defer_splits(w, tiles, kb, c.num_sms) : c.tc_splits[1][w];
     c.tc_tiles[w] = tiles;
     // every unit stages its accumulator rows in the workspace
-    ws = std::max(ws, (size_t)tiles * c.tc_splits[w] * c.tc_rows_max * c.tc_bw);
+    ws = std::max(ws, (size_t)tiles * std::max(c.tc_splits[0][w], c.tc_splits[1][w]) * c.tc_rows_max * c.tc_bw);
     if (c.pf_max > 0) {   // prompts of few tokens
       const int rows = std::min(kPfSmallRows, (c.pf_max + 15) & ~15);
       ws = std::max(ws, (size_t)tiles * defer_splits(w, tiles, kb, c.num_sms) * std::max(16, rows) * c.tc_bw);
@@ -512,9 +519,9 @@ int gemm_tc_prepare(Ctx& c) {
   if (c.tc_panel) {
     int N, K, tiles;
     gemm_shape(c, 0, &N, &K, &tiles);
-    c.tc_panel_kb = (K / kTileK + c.tc_splits[0] - 1) / c.tc_splits[0];
+    c.tc_panel_kb = (K / kTileK + c.tc_splits[0][0] - 1) / c.tc_splits[0][0];   // (as with hi + lo)
     gemm_shape(c, 2, &N, &K, &tiles);
-    c.tc_panel_kb = std::max(c.tc_panel_kb, (K / kTileK + c.tc_splits[2] - 1) / c.tc_splits[2]);
+    c.tc_panel_kb = std::max(c.tc_panel_kb, (K / kTileK + c.tc_splits[0][2] - 1) / c.tc_splits[0][2]);
     const int limit = 227 * 1024 - 2 * 1024;
     for (int v = 0; v < 2; ++v) {
       c.tc_panel_bytes[v] = (uint32_t)(v + 1) * (uint32_t)c.tc_panel_kb * 1024u;
@@ -580,7 +587,7 @@ static TcParams tc_params(const Ctx& c, const GemmArgs& a, size_t* smem_out) {
   p.K = K;
   p.n_tiles = tiles;
   p.kb_total = (K + kTileK - 1) / kTileK;
-  p.splits = c.tc_splits[which];
+  p.splits = gemm_tc_splits(c, which, a.split);
   p.kb_per_split = (p.kb_total + p.splits - 1) / p.splits;
   p.units = tiles * p.splits;
   p.bw = c.tc_bw;

@@ -166,6 +166,7 @@ void launch_pool_refresh(const Ctx& c, const buddy_kv_state& kv, int n_seq, cons
 // GEMMs (gemm_simt.cu, gemm_tc.cu)
 void launch_gemm_simt(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s);
 bool gemm_tc_supported(const Ctx& c);
+int gemm_tc_splits(const Ctx& c, int which, bool split);
 void launch_gemm_tc(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s);
 // prefill (gemm_pf.cu, attn_pf.cu, prefill.cu)
 int gemm_pf_prepare(Ctx& c);
@@ -242,7 +243,8 @@ struct Ctx {
   int tc_bw = 256, tc_mt = 1, tc_rows_max = 16, tc_acc_bufs = 2;   // tile geometry (gemm_common.cuh)
   int tc_stages[2] = {1, 1}, tc_smem[2] = {0, 0};                   // [plain, split activations]
   uint32_t tc_stage_bytes[2] = {0, 0}, tc_w_off[2] = {0, 0}, tc_xr = 0, tc_tmem_cols = 512;
-  int tc_splits[4] = {1, 1, 1, 1}, tc_tiles[4] = {1, 1, 1, 1};
+  int tc_splits[2][4] = {{1, 1, 1, 1}, {1, 1, 1, 1}};               // [plain, split activations][projection]
+  int tc_tiles[4] = {1, 1, 1, 1};
   float* gemm_ws = nullptr;
   size_t gemm_ws_elems = 0;
   int32_t* gemm_ctr = nullptr;

@@ -113,6 +113,37 @@ def test_route_checks_write_nothing():
     assert dw.ctx.buddy_device_status() == 0 and not bool((sc == 7.0).any())
 
 
+@pytest.mark.parametrize("base", [C.LLAMA3_8B, C.LLAMA2_13B], ids=lambda s: s.name)
+def test_scores_keep_the_feeding_blocks_precision(base):
+    """Scores after one block over a single position, against 64 bits from the stored V on.  What is left is
+    the fp32 sums: a tensor-core accumulator truncates at each K = 16 step, about 2^-24 of the sum a time,
+    and a sum of n steps (hi and lo) ends n / 2^24 off.  Gate and up in four K splits take 128 to 160 steps,
+    down about 200: 2e-5 of the block's update, less than half of the scores; gate and up in one sum take
+    512 to 640 and twice that in all."""
+    s = dataclasses.replace(base, n_layers=34)
+    B, T = 16, torch.float64
+    w = synth.layer_weights(s, 5, 0, "cuda")
+    dm = synth.dm_weights(s, 5, "cuda")
+    ctx = pkg.Context.for_shape(s, max_batch=B, max_pos=4)
+    layer = pkg.pack_layer(w)
+    ctx.buddy_set_weights([layer] * s.n_layers, dm)
+    kv = pkg.KVCache(s.n_layers, s.n_kv_heads, s.head_dim, [1] * B, torch.bfloat16, "cuda")
+    h = synth.h_in(s, 5, 0, range(B), "cuda")
+    sc = torch.empty(B, s.n_cand, device="cuda")
+    ctx.buddy_decode_step(kv, h, torch.ones(B, dtype=torch.int32, device="cuda"), torch.empty_like(h), scores_out=sc)
+    assert ctx.buddy_device_status() == 0
+    v = torch.stack([kv.view("v", 0, i)[:, 0] for i in range(B)]).to(T)
+    v = v[:, :, None].expand(-1, -1, s.group, -1).reshape(B, s.q_dim)
+    x = h.to(T) + v @ layer["w_o"].to(T).T
+    y = x * torch.rsqrt(x.square().mean(1, keepdim=True) + s.rms_eps) * layer["ffn_norm"].to(T)
+    g, u = (y @ layer["w_gate_up"].to(T).T).chunk(2, 1)
+    x = torch.cat([v, x + (torch.nn.functional.silu(g) * u) @ layer["w_down"].to(T).T], 1)
+    d = {k: t.to(T) for k, t in dm.items()}
+    ref = torch.nn.functional.silu(x @ d["w1"].T + d["b1"]) @ d["w2"].T + d["b2"]
+    err = float((sc.to(T) - ref).norm() / ref.norm())
+    assert err < 1.0e-5
+
+
 def silu_context(r, n_layers):
     """A router whose scores are silu(x + b1) of the first r channels x of h1."""
     s = dataclasses.replace(C.SMALL_F32, n_layers=n_layers, dm_hidden=r)
