@@ -14,9 +14,9 @@
 //
 // Above that (gemm_simt_tiled_kernel) tiles of 32 rows x 32 weight rows, K in
 // steps of 32 through a four-stage cp.async ring: the weights are read once per 32
-// rows, not once per four.  5 blocks of width 256, 200 rows: 587 us a step against
-// 2152 us.  The line lies where the two meet: 17 rows take 211 us fused and 254 us
-// tiled, 32 rows 306 us and 294 us.
+// rows, not once per four.  5 blocks of width 256, 200 rows: 546 us a step against
+// 2094 us.  The line lies where the two meet: 25 rows take 286 us fused and 300 us
+// tiled, 28 rows 312 and 318 us, 32 rows 328 and 318 us.
 #include <cuda_runtime.h>
 
 #include "attn_common.cuh"
@@ -222,36 +222,69 @@ __global__ void __launch_bounds__(256) gemm_simt_tiled_kernel(const SimtArgs p) 
     if (s < steps) load(s);
     cp_async_commit();
   }
-  float4 acc4[2][2];   // four sums per output, over k mod 4: a shorter chain of roundings
+  // Each output is summed as a tree with short branches, so that its rounding errors
+  // are no larger than those of the warps' sums in the other kernel: over k mod 4, of
+  // those over the halves of a step (4 products each), then even and odd steps.  (Four
+  // chains of K / 4 left stored values 1.6, 1.9 and 2.5 times as far from 64 bits at K =
+  // 256, 512 and 2048.)
+  auto add4 = [](float4& s, const float4& v) {
+    s.x += v.x;
+    s.y += v.y;
+    s.z += v.z;
+    s.w += v.w;
+  };
+  float4 even[2][2], odd[2][2];
 #pragma unroll
-  for (int a = 0; a < 2; ++a) acc4[a][0] = acc4[a][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s = 0; s < steps; ++s) {
+  for (int a = 0; a < 2; ++a) even[a][0] = even[a][1] = odd[a][0] = odd[a][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto step = [&](int s, float4 (&sum)[2][2]) {
     cp_async_wait<kStStages - 2>();
     __syncthreads();   // step s has landed for every thread, step s - 1 is consumed
     if (s + kStStages - 1 < steps) load(s + kStStages - 1);
     cp_async_commit();
+    float4 t[2][2][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int a = 0; a < 2; ++a) t[h][a][0] = t[h][a][1] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < kStK; k += 4) {
+      const int h = k / (kStK / 2);
 #pragma unroll
       for (int a = 0; a < 2; ++a) {
         const float4 x = *reinterpret_cast<const float4*>(&sm[s % kStStages][ty + 16 * a][k]);
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
           const float4 w = *reinterpret_cast<const float4*>(&sm[s % kStStages][kStM + tx + 16 * b][k]);
-          acc4[a][b].x += x.x * w.x;
-          acc4[a][b].y += x.y * w.y;
-          acc4[a][b].z += x.z * w.z;
-          acc4[a][b].w += x.w * w.w;
+          t[h][a][b].x += x.x * w.x;
+          t[h][a][b].y += x.y * w.y;
+          t[h][a][b].z += x.z * w.z;
+          t[h][a][b].w += x.w * w.w;
         }
       }
     }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        add4(t[0][a][b], t[1][a][b]);
+        add4(sum[a][b], t[0][a][b]);
+      }
+  };
+  int s = 0;
+  for (; s + 1 < steps; s += 2) {
+    step(s, even);
+    step(s + 1, odd);
   }
+  if (s < steps) step(s, even);
   cp_async_wait<0>();
   float acc[2][2];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 2; ++b) acc[a][b] = (acc4[a][b].x + acc4[a][b].y) + (acc4[a][b].z + acc4[a][b].w);
+    for (int b = 0; b < 2; ++b) {
+      add4(even[a][b], odd[a][b]);
+      acc[a][b] = (even[a][b].x + even[a][b].y) + (even[a][b].z + even[a][b].w);
+    }
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
     const int j = i0 + ty + 16 * a;

@@ -17,7 +17,7 @@ constexpr int kMaxLayers = 128;
 constexpr int kRouteZSlots = 32;  // K-split slots of the router's hidden-unit partial sums
 constexpr int kMaxBatch = 1024;
 constexpr int kPfSmallRows = 256;  // prefill tokens up to which the decode GEMMs run its projections
-constexpr int kSimtFuseRows = 24;  // fp32: rows up to which the GEMMs take in the norms and the QKV finalisation
+constexpr int kSimtFuseRows = 28;  // fp32: rows up to which the GEMMs take in the norms and the QKV finalisation
 
 // Per-layer K/V base pointers passed by value to kernels that touch many layers.
 struct LayerPtrs {

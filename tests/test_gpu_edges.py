@@ -65,8 +65,8 @@ def test_decode_parity_claimed_units():
 
 
 # fp32: four or eight rows per pass (4, 5), norms and QKV finalisation inside the
-# GEMMs up to 24 rows, tiles of 32 rows above (25, 32, 33)
-@pytest.mark.parametrize("batch", [4, 5, 24, 25, 32, 33])
+# GEMMs up to 28 rows, tiles of 32 rows above (29, 32, 33)
+@pytest.mark.parametrize("batch", [4, 5, 24, 25, 28, 29, 32, 33])
 def test_decode_parity_f32_batch_modes(batch):
     assert run_parity(rows_of(C.T_F32, batch), steps=2)[0] < 1e-4
 
@@ -113,6 +113,30 @@ def test_route_checks_write_nothing():
     assert dw.ctx.buddy_device_status() == 0 and not bool((sc == 7.0).any())
 
 
+def value_error(d, batch):
+    """Stored V of an fp32 model's first block against 64 bits: relative error, 2-norm."""
+    s = dataclasses.replace(C.SMALL_F32, d_model=d, n_q_heads=d // 64, n_kv_heads=d // 64, n_layers=3)
+    w = synth.layer_weights(s, 5, 0, "cuda")
+    layer = pkg.pack_layer(w)
+    ctx = pkg.Context.for_shape(s, max_batch=batch, max_pos=4)
+    ctx.buddy_set_weights([layer] * 3, synth.dm_weights(s, 5, "cuda"))
+    kv = pkg.KVCache(3, s.n_kv_heads, 64, [1] * batch, torch.float32, "cuda")
+    h = synth.h_in(s, 5, 0, range(batch), "cuda")
+    ctx.buddy_decode_step(kv, h, torch.ones(batch, dtype=torch.int32, device="cuda"), torch.empty_like(h))
+    assert ctx.buddy_device_status() == 0
+    v = torch.stack([kv.view("v", 0, i)[:, 0].reshape(-1) for i in range(batch)]).double()
+    x = h.double()
+    x = x * torch.rsqrt(x.square().mean(1, keepdim=True) + s.rms_eps) * layer["attn_norm"].double()
+    ref = x @ w["w_v"].double().T + w["b_v"].double()
+    return float((v - ref).norm() / ref.norm())
+
+
+# above 28 rows tiles, up to 28 a warp per sum: a tree of 32 sums of K / 32 products; 2%: other rows, other errors
+@pytest.mark.parametrize("d", [256, 512, 2048])
+def test_f32_tiles_keep_the_warp_sums_precision(d):
+    assert value_error(d, 64) < 1.02 * value_error(d, 24)
+
+
 @pytest.mark.parametrize("base", [C.LLAMA3_8B, C.LLAMA2_13B], ids=lambda s: s.name)
 def test_scores_keep_the_feeding_blocks_precision(base):
     """Scores after one block over a single position, against 64 bits from the stored V on.  What is left is
@@ -141,6 +165,7 @@ def test_scores_keep_the_feeding_blocks_precision(base):
     d = {k: t.to(T) for k, t in dm.items()}
     ref = torch.nn.functional.silu(x @ d["w1"].T + d["b1"]) @ d["w2"].T + d["b2"]
     err = float((sc.to(T) - ref).norm() / ref.norm())
+    print("score error", err)
     assert err < 1.0e-5
 
 
