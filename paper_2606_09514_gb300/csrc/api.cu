@@ -136,7 +136,7 @@ extern "C" int buddy_create(const buddy_config* cfg, buddy_ctx** out) {
       (e = dalloc(&c.attn_l, B * c.nq * c.attn_max_chunks)) ||
       (e = dalloc(&c.attn_acc, B * c.nq * c.attn_max_chunks * c.hd)) ||
       (e = dalloc(&c.attn_ctr, B * c.nkv + 2)) ||
-      (e = dalloc(&c.dm_u, (size_t)kRouteZSlots * B * c.r)) || (e = route_prepare()) ||
+      (e = dalloc(&c.dm_u, (size_t)kRouteZSlots * B * c.r)) || (e = route_prepare()) || (e = attention_prepare(c)) ||
       (e = dalloc(&c.mask, B * c.L)) ||
       (e = dalloc(&c.sel, B * c.Lm)) || (e = dalloc(&c.scores, B * c.Lm)) ||
       (e = dalloc(&c.rows, (size_t)c.L * B)) || (e = dalloc(&c.count, (size_t)c.L)) ||

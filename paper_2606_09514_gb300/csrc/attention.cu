@@ -23,6 +23,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "attn_common.cuh"
 #include "attn_tc.cuh"
@@ -38,21 +39,28 @@ __global__ void __launch_bounds__(kTcaThreads) attn_tc_kernel(AttnArgs<bf16> A) 
   attn_tc_run<HD, SPLIT>(A, blockIdx.x, gridDim.x, smraw, sc, true);
 }
 
+// Grid of a persistent attention kernel: the CTAs resident at once, at most four per
+// SM.  The attribute is the largest any context uses: it belongs to the function on the
+// device, so a context's own size would take it from another one's launches.
+template <typename K>
+static cudaError_t attn_prepare(K kernel, int threads, size_t smem, int smem_limit, int num_sms, int* grid) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
+  if (e != cudaSuccess) return e;
+  int occ = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    occ = 1;
+  }
+  *grid = num_sms * std::max(1, std::min(occ, 4));
+  return cudaSuccess;
+}
+
 // bf16 caches with at most 8 query heads per KV head: the tensor-core loop
 template <int HD, bool SPLIT>
 static void attn_tc_impl(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int layer, const float* q, void* out,
                          void* out_lo, cudaStream_t s) {
   const size_t smem = attn_tc_smem_bytes(HD, c.maxB);
-  static int occ = 0;   // one per instantiation
-  static size_t occ_smem = 0;
-  if (occ == 0 || occ_smem != smem) {
-    cudaFuncSetAttribute(attn_tc_kernel<HD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, attn_tc_kernel<HD, SPLIT>, kTcaThreads, smem) !=
-        cudaSuccess)
-      occ = 1;
-    occ_smem = smem;
-  }
-  const int grid = c.num_sms * std::max(1, std::min(occ, 4));
+  const int grid = c.attn_grid[SPLIT ? 1 : 0];
   AttnArgs<bf16> A{q, sel.rows, sel.count, sel.n, c.nq, c.nkv, cache_len(c, kv, layer), kv.seq_off, kv.cap,
                    (const bf16*)kv.k_cache[layer], (const bf16*)kv.v_cache[layer], c.attn_max_chunks, c.attn_m,
                    c.attn_l, c.attn_acc, c.attn_ctr, (bf16*)out, (bf16*)out_lo, c.status,
@@ -72,35 +80,36 @@ static void attn_impl(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int la
                       void* out, void* out_lo, cudaStream_t s) {
   const int G = c.nq / c.nkv;
   const size_t smem = attn_smem_bytes(attn_smem_fixed<T, HD>(), G, HD, c.attn_max_chunks, c.maxB);
-  static bool attr_set = false;   // one per instantiation
-  static int occ = 0;
-  static size_t occ_smem = 0;
-  if (!attr_set) {
-    cudaFuncSetAttribute(attn_kernel<T, HD, GP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr_set = true;
-  }
-  if (occ == 0 || occ_smem != smem) {   // resident CTAs per SM at this shared-memory size
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, attn_kernel<T, HD, GP>, kAttnThreads, smem) !=
-        cudaSuccess)
-      occ = 1;
-    occ_smem = smem;
-  }
-  const int grid = c.num_sms * std::max(1, std::min(occ, 4));
+  const int grid = c.attn_grid[0];
   AttnArgs<T> A{q, sel.rows, sel.count, sel.n, c.nq, c.nkv, cache_len(c, kv, layer), kv.seq_off, kv.cap,
                 (const T*)kv.k_cache[layer], (const T*)kv.v_cache[layer], c.attn_max_chunks, c.attn_m, c.attn_l,
                 c.attn_acc, c.attn_ctr, (T*)out, (T*)out_lo, c.status};
   launch_k(attn_kernel<T, HD, GP>, grid, kAttnThreads, smem, s, c.pdl, A);
 }
 
+// f with the group size, padded to a power of two, as a compile-time constant
+template <typename F>
+static auto by_group(int G, F f) {
+  switch (attn_group_pad(G)) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    default: return f(std::integral_constant<int, 8>{});
+  }
+}
 template <typename T, int HD>
 static void attn_group(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int layer, const float* q, void* out,
                        void* out_lo, cudaStream_t s) {
-  switch (attn_group_pad(c.nq / c.nkv)) {
-    case 1: attn_impl<T, HD, 1>(c, sel, kv, layer, q, out, out_lo, s); break;
-    case 2: attn_impl<T, HD, 2>(c, sel, kv, layer, q, out, out_lo, s); break;
-    case 4: attn_impl<T, HD, 4>(c, sel, kv, layer, q, out, out_lo, s); break;
-    default: attn_impl<T, HD, 8>(c, sel, kv, layer, q, out, out_lo, s);
-  }
+  by_group(c.nq / c.nkv, [&](auto gp) { attn_impl<T, HD, decltype(gp)::value>(c, sel, kv, layer, q, out, out_lo, s); });
+}
+template <typename T, int HD>
+static cudaError_t attn_group_prepare(Ctx& c) {
+  const int G = c.nq / c.nkv;
+  const size_t smem = attn_smem_bytes(attn_smem_fixed<T, HD>(), G, HD, c.attn_max_chunks, c.maxB);
+  return by_group(G, [&](auto gp) {
+    return attn_prepare(attn_kernel<T, HD, decltype(gp)::value>, kAttnThreads, smem, 200 * 1024, c.num_sms,
+                        &c.attn_grid[0]);
+  });
 }
 
 // Partial slots per (row, query head): the CUDA-core loop's spans are at least
@@ -115,6 +124,23 @@ int attention_max_spans(int max_pos) {
 bool attention_tc(const Ctx& c) {
   return c.dtype == BUDDY_DTYPE_BF16 && c.nq / c.nkv <= 8 &&
          attn_tc_smem_bytes(c.hd, c.maxB) <= (size_t)kTcaSmemLimit;
+}
+
+template <int HD>
+static cudaError_t attn_tc_prepare(Ctx& c) {
+  const size_t smem = attn_tc_smem_bytes(HD, c.maxB);
+  const cudaError_t e = attn_prepare(attn_tc_kernel<HD, false>, kTcaThreads, smem, kTcaSmemLimit, c.num_sms, &c.attn_grid[0]);
+  return e != cudaSuccess ? e : attn_prepare(attn_tc_kernel<HD, true>, kTcaThreads, smem, kTcaSmemLimit, c.num_sms, &c.attn_grid[1]);
+}
+
+cudaError_t attention_prepare(Ctx& c) {
+  const cudaError_t e = attention_cl_prepare(c);
+  if (e != cudaSuccess) return e;
+  if (attention_cl(c)) return cudaSuccess;
+  const bool wide = c.hd == 128;
+  if (attention_tc(c)) return wide ? attn_tc_prepare<128>(c) : attn_tc_prepare<64>(c);
+  if (c.dtype == BUDDY_DTYPE_BF16) return wide ? attn_group_prepare<bf16, 128>(c) : attn_group_prepare<bf16, 64>(c);
+  return wide ? attn_group_prepare<float, 128>(c) : attn_group_prepare<float, 64>(c);
 }
 
 void launch_attention(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int layer, const float* q,

@@ -369,22 +369,19 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
   }
 }
 
-// Clusters of 16, 8, 4 and 2 CTAs the device can hold at once, queried once per
-// instantiation; 0 where the size cannot be scheduled.
-constexpr int kClSizes = 4;
+// Clusters of 16, 8, 4 and 2 CTAs the device can hold at once (cap[v]: C = 16 >> v);
+// 0 where the size cannot be scheduled.
 template <int HD, bool SPLIT>
-static const int* cl_capacity() {
-  static int cap[kClSizes] = {-1, -1, -1, -1};   // [v]: C = 16 >> v
-  if (cap[kClSizes - 1] >= 0) return cap;
+static cudaError_t cl_prepare(int* cap) {
   const size_t smem = attn_cl_smem<HD>();
-  cudaFuncSetAttribute(attn_cl_kernel<HD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(attn_cl_kernel<HD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   for (int v = 0; v < kClSizes; ++v) {
     const int C = kClMaxCtas >> v;
-    int n = 0;
+    cap[v] = 0;
     if (C > 8 && cudaFuncSetAttribute(attn_cl_kernel<HD, SPLIT>, cudaFuncAttributeNonPortableClusterSizeAllowed,
                                       1) != cudaSuccess) {
       cudaGetLastError();
-      cap[v] = 0;
       continue;
     }
     cudaLaunchConfig_t cfg = {};
@@ -398,21 +395,28 @@ static const int* cl_capacity() {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, attn_cl_kernel<HD, SPLIT>, &cfg) != cudaSuccess) n = 0;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, attn_cl_kernel<HD, SPLIT>, &cfg) == cudaSuccess) cap[v] = n;
     cudaGetLastError();
-    cap[v] = n;
   }
-  return cap;
+  return cudaSuccess;
+}
+cudaError_t attention_cl_prepare(Ctx& c) {
+  if (!(c.dtype == BUDDY_DTYPE_BF16 && c.nq / c.nkv <= 8 && c.maxB * c.nkv <= kClMaxStreams)) return cudaSuccess;
+  const cudaError_t e = c.hd == 128 ? cl_prepare<128, false>(c.cl_cap[0]) : cl_prepare<64, false>(c.cl_cap[0]);
+  if (e != cudaSuccess) return e;
+  return c.hd == 128 ? cl_prepare<128, true>(c.cl_cap[1]) : cl_prepare<64, true>(c.cl_cap[1]);
 }
 
 // Cluster size for `streams` streams: the largest of which every stream's cluster
 // fits at once (a cluster that waits for others to finish starts its stream when
-// they have ended theirs: 56 streams of 970 positions take 21 us a block in three
-// waves of 8-CTA clusters, 12 us in one of 2-CTA clusters); else the smallest
-// that can be scheduled, 0 if none can.
-template <int HD, bool SPLIT>
-static int cl_size(int streams) {
-  const int* cap = cl_capacity<HD, SPLIT>();
+// they have ended theirs); else the smallest that can be scheduled, 0 if none can.
+// Steps of 6 blocks of Llama-3-8B, against clusters of 8 in several waves: 32 streams
+// of 300, 1000 and 8000 positions 608, 631 and 738 us (655, 677, 821 us), 40 streams,
+// with clusters of 2, 610, 644 and 802 us (656, 678, 831 us), 64 streams 628, 656 and
+// 865 us (724, 749, 994 us).
+static int cl_size(const Ctx& c, bool split, int streams) {
+  const int* cap = c.cl_cap[split ? 1 : 0];
   int last = 0;
   for (int v = 0; v < kClSizes; ++v) {
     if (cap[v] > 0) last = kClMaxCtas >> v;
@@ -421,15 +425,13 @@ static int cl_size(int streams) {
   return last;
 }
 
-bool attention_cl(const Ctx& c) {
-  if (!(c.dtype == BUDDY_DTYPE_BF16 && c.nq / c.nkv <= 8 && c.maxB * c.nkv <= kClMaxStreams)) return false;
-  return (c.hd == 128 ? cl_size<128, false>(c.maxB * c.nkv) : cl_size<64, false>(c.maxB * c.nkv)) > 0;
-}
+// (no cluster fits where attention_cl_prepare found the shape too large)
+bool attention_cl(const Ctx& c) { return cl_size(c, false, c.maxB * c.nkv) > 0; }
 
 template <int HD, bool SPLIT>
 static void attn_cl_impl(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int layer, const float* q, void* out,
                          void* out_lo, cudaStream_t s) {
-  const int C = cl_size<HD, SPLIT>(sel.n * c.nkv);
+  const int C = cl_size(c, SPLIT, sel.n * c.nkv);
   AttnArgs<bf16> A{q, sel.rows, sel.count, sel.n, c.nq, c.nkv, cache_len(c, kv, layer), kv.seq_off, kv.cap,
                    (const bf16*)kv.k_cache[layer], (const bf16*)kv.v_cache[layer], 0, nullptr, nullptr, nullptr,
                    nullptr, (bf16*)out, (bf16*)out_lo, c.status};

@@ -365,15 +365,14 @@ typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 static PFN_encodeTiled get_encode() {
-  static PFN_encodeTiled fn = nullptr;
-  if (!fn) {
+  static const PFN_encodeTiled fn = [] {   // the driver's, the same for every device
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_encodeTiled>(p);
-  }
+    const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                        cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return reinterpret_cast<PFN_encodeTiled>(ok ? p : nullptr);
+  }();
   return fn;
 }
 
@@ -556,10 +555,10 @@ int gemm_tc_prepare(Ctx& c) {
     if (rc != BUDDY_OK) return rc;
   }
   const cudaFuncAttribute A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  const int qs0 = std::max(c.tc_smem[0], c.tc_panel ? c.tc_psmem[0] : 0);
-  const int qs1 = std::max(c.tc_smem[1], c.tc_panel ? c.tc_psmem[1] : 0);
+  // the largest size any context uses: the attribute belongs to the function on the
+  // device, and a context's own would take it from another one's launches
   bool bad = false;
-  if (c.tc_defer || c.pf_max > 0)   // prefill chooses its stages by the tokens of a call
+  if (c.tc_defer || c.pf_max > 0)
     bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, true>, A, limit) ||
           cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, true>, A, limit) ||
           cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, true>, A, limit) ||
@@ -567,12 +566,12 @@ int gemm_tc_prepare(Ctx& c) {
           cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true, true>, A, limit) ||
           cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true, true>, A, limit);
   if (!bad && !c.tc_defer)
-    bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, false>, A, qs0) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, false>, A, c.tc_smem[0]) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, false>, A, qs0) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, true, false>, A, qs1) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true, false>, A, c.tc_smem[1]) ||
-          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true, false>, A, qs1);
+    bad = cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, false, false>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, false, false>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, false, false>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, true, false>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, true, false>, A, limit) ||
+          cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, true, false>, A, limit);
   if (bad) return BUDDY_ERR_CUDA;
   return BUDDY_OK;
 }

@@ -17,6 +17,7 @@ constexpr int kMaxLayers = 128;
 constexpr int kRouteZSlots = 32;  // K-split slots of the router's hidden-unit partial sums
 constexpr int kMaxBatch = 1024;
 constexpr int kPfSmallRows = 256;  // prefill tokens up to which the decode GEMMs run its projections
+constexpr int kClSizes = 4;        // cluster sizes of the small batches' attention: 16, 8, 4 and 2 CTAs
 constexpr int kSimtFuseRows = 28;  // fp32: rows up to which the GEMMs take in the norms and the QKV finalisation
 
 // Per-layer K/V base pointers passed by value to kernels that touch many layers.
@@ -144,6 +145,8 @@ void launch_qkv_finalize(const Ctx& c, const float* qkv, const float* bias, RowS
 void launch_attention(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int layer, const float* q,
                       void* attn_out, void* attn_lo, cudaStream_t s);   // attention.cu
 int attention_max_spans(int max_pos);   // span partials per (row, query head)
+cudaError_t attention_prepare(Ctx& c);      // function attributes, grids and cluster capacities of this context's kernels
+cudaError_t attention_cl_prepare(Ctx& c);
 bool attention_tc(const Ctx& c);         // tensor-core loop over the whole GPU
 bool attention_cl(const Ctx& c);         // small batches: one cluster per stream (attn_cl.cu)
 void launch_attention_cl(const Ctx& c, RowSel sel, const buddy_kv_state& kv, int layer, const float* q, void* out,
@@ -220,6 +223,8 @@ struct Ctx {
   float* qkv = nullptr;        // [maxB, qkvN]
   float* q = nullptr;          // [maxB, qd]
   int attn_max_chunks = 1;   // span partial slots per (row, query head)
+  int attn_grid[2] = {1, 1};      // CTAs of the persistent attention kernels [plain, split activations]
+  int cl_cap[2][kClSizes] = {};   // clusters of 16 >> v CTAs the device holds at once [plain, split]; 0: not used
   float* attn_m = nullptr;     // [maxB, nq, max_chunks]
   float* attn_l = nullptr;
   float* attn_acc = nullptr;   // [maxB, nq, max_chunks, hd]

@@ -307,6 +307,33 @@ def test_decode_parity_shares_shorter_than_the_cluster(batch):
     assert run_parity(w, steps=2)[0] < 2e-2
 
 
+# kernel attributes belong to a function on the device, not to a context: contexts of other shapes and batches,
+# created in between and smaller or larger, must not take them from one another
+def test_contexts_of_other_shapes_side_by_side():
+    wide = dataclasses.replace(C.SMALL_QWEN_BF16, name="wide", d_model=4096, n_q_heads=32, n_kv_heads=8)
+    ws = [dataclasses.replace(C.scaled(C.T_QWEN, ctx=[40], k=[2], name="wide-b1"), shape=wide),
+          C.scaled(C.T_GQA, ctx=[70], k=[1], name="gqa-b1"),
+          rows_of(C.T_GQA, 200), rows_of(C.T_GQA, 37), rows_of(C.T_F32, 200), rows_of(C.T_F32, 30)]
+
+    def step(dw, w):
+        h = torch.empty(w.batch, w.shape.d_model, device="cuda")
+        dw.ctx.buddy_decode_step(dw.kv, synth.workload_h_in(w, 0, "cuda"), dw.k, h)
+        assert dw.ctx.buddy_device_status() == 0
+        return h
+    alone = []
+    for w in ws:
+        dw = D.build(w)
+        alone.append(step(dw, w))
+        dw.ctx.close()
+    live = [D.build(w) for w in ws]
+    for i in list(range(len(ws)))[::-1]:   # the smallest of each kind was prepared last
+        if ws[i].batch in (30, 37) or ws[i].name == "gqa-b1":
+            assert torch.equal(step(live[i], ws[i]), alone[i])
+    for i, w in enumerate(ws):
+        if not (w.batch in (30, 37) or w.name == "gqa-b1"):
+            assert torch.equal(step(live[i], w), alone[i])
+
+
 def test_panel_wait_limit_runs_out_and_context_recovers():
     """As the other batches' test: 1 ns runs out, the restored limit gives a fresh context's result."""
     w = C.scaled(C.T_GQA, ctx=[5, 200], k=[1, 3], name="t-gqa-b2-timeout")

@@ -41,3 +41,11 @@ def test_cluster_barrier_before_remote_shared_memory(body):
 
 def test_remote_kernels_are_found():
     assert {p.id for p in remote_kernels()} == {"attn_cl_kernel", "gemm_pf_kernel", "pool_refresh_kernel"}
+
+
+# What a function keeps between calls would be shared by contexts on other devices and
+# by host threads: only constants may be static in a function.
+def test_no_state_kept_in_functions():
+    found = [f"{f.name}: {line.strip()}" for f in sorted(CSRC.glob("*.cu*")) + sorted(CSRC.glob("*.h"))
+             for line in code(f).splitlines() if re.match(r"\s+static\s+(?!const\b|constexpr\b)", line)]
+    assert not found
