@@ -356,7 +356,8 @@ def test_panel_wait_limit_runs_out_and_context_recovers():
     assert torch.equal(*outs)
 
 
-# the decode GEMMs (40 tokens), the CTA pairs and units cut along K (300 tokens)
+# the decode GEMMs (40 tokens), the CTA pairs and, in the first block's down projection, units cut along K (300
+# tokens; test_gpu_prefill_units.py holds the other schedules)
 @pytest.mark.parametrize("lengths", [[33, 7], [290, 10]], ids=lambda v: str(sum(v)))
 def test_prefill_wait_limit_runs_out_and_context_recovers(lengths):
     w = C.scaled(C.T_QWEN, ctx=[3, 60], k=[2, 4], name="pf-timeout")
