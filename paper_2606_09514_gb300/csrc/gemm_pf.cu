@@ -714,8 +714,8 @@ int gemm_pf_prepare(Ctx& c) {
 // One prefill projection: `which` names the weight (0 qkv, 1 o, 2 gate_up,
 // 3 down) of `layer`; `xi` the prefill activation map (0 normalised input,
 // 1 attention output, 2 SwiGLU output); m rows.
-void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
-                    cudaStream_t s) {
+int launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
+                   cudaStream_t s) {
   // Few tokens are bound by the weight stream: the decode GEMM (one CTA per weight
   // tile and K split, a fixup over the whole GPU) beats pairs that each hold an
   // M-tile mostly empty and sum their parts alone: 4 blocks of Llama-3-8B, 61 tokens
@@ -793,6 +793,7 @@ void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int
       default: launch_k(gemm_pf_kernel<EPI_SWIGLU, false>, grid, kPfThreads, smem, s, c.pdl, tw, tx, txlo, p);
     }
   }
+  return 1;
 }
 
 }  // namespace buddy

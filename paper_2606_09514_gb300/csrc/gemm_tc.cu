@@ -677,7 +677,7 @@ static int fix_grid(const Ctx& c, const TcParams& p, int rows) {
 // token row in the place of a sequence (its own position, block offset and
 // capacity), the ring and the workspace sized by the rows of this call.
 template <int EPI, bool SPLIT>
-static void launch_pf_small(const Ctx& c, int layer, int which, int xi, int m, const PfEpi& e, cudaStream_t s) {
+static int launch_pf_small(const Ctx& c, int layer, int which, int xi, int m, const PfEpi& e, cudaStream_t s) {
   GemmArgs a{};
   a.sel = RowSel{e.rows, nullptr, m};
   a.split = SPLIT;
@@ -710,16 +710,17 @@ static void launch_pf_small(const Ctx& c, int layer, int which, int xi, int m, c
   smem = (size_t)p.stages * p.stage_bytes + 1024;
   launch_k(gemm_tc_kernel<EPI, SPLIT, true>, std::min(p.units, c.num_sms), kTcDeferThreads, smem, s, c.pdl,
            c.tmaps_host[(size_t)layer * 4 + which], c.pf_xmaps[xi], c.pf_xmaps[3 + xi], p);
-  if (!(EPI == EPI_SWIGLU && p.splits == 1))
-    launch_k(gemm_fix_kernel<EPI, SPLIT>, fix_grid<EPI>(c, p, m), kTcFixThreads, 0, s, c.pdl, p);
+  if (EPI == EPI_SWIGLU && p.splits == 1) return 1;
+  launch_k(gemm_fix_kernel<EPI, SPLIT>, fix_grid<EPI>(c, p, m), kTcFixThreads, 0, s, c.pdl, p);
+  return 2;
 }
 
-void launch_gemm_pf_small(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
-                          cudaStream_t s) {
-  auto go = [&](auto plain, auto hilo) { (split ? hilo : plain)(c, layer, which, xi, m, e, s); };
-  if (epi == EPI_QKV) go(launch_pf_small<EPI_QKV, false>, launch_pf_small<EPI_QKV, true>);
-  else if (epi == EPI_RESID) go(launch_pf_small<EPI_RESID, false>, launch_pf_small<EPI_RESID, true>);
-  else go(launch_pf_small<EPI_SWIGLU, false>, launch_pf_small<EPI_SWIGLU, true>);
+int launch_gemm_pf_small(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
+                         cudaStream_t s) {
+  auto go = [&](auto plain, auto hilo) { return (split ? hilo : plain)(c, layer, which, xi, m, e, s); };
+  if (epi == EPI_QKV) return go(launch_pf_small<EPI_QKV, false>, launch_pf_small<EPI_QKV, true>);
+  if (epi == EPI_RESID) return go(launch_pf_small<EPI_RESID, false>, launch_pf_small<EPI_RESID, true>);
+  return go(launch_pf_small<EPI_SWIGLU, false>, launch_pf_small<EPI_SWIGLU, true>);
 }
 
 template <int EPI, bool SPLIT>

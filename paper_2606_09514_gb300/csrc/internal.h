@@ -173,11 +173,12 @@ int gemm_tc_splits(const Ctx& c, int which, bool split);
 void launch_gemm_tc(const Ctx& c, int epi, const GemmArgs& a, cudaStream_t s);
 // prefill (gemm_pf.cu, attn_pf.cu, prefill.cu)
 int gemm_pf_prepare(Ctx& c);
-void launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
-                    cudaStream_t s);
+// Returns the kernels launched.
+int launch_gemm_pf(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
+                   cudaStream_t s);
 // The same projection by the decode GEMM and its fixup (m <= kPfSmallRows).
-void launch_gemm_pf_small(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
-                          cudaStream_t s);   // gemm_tc.cu
+int launch_gemm_pf_small(const Ctx& c, int epi, bool split, int layer, int which, int xi, int m, const PfEpi& e,
+                         cudaStream_t s);   // gemm_tc.cu
 void launch_attention_pf(const Ctx& c, int n_items, const int4* items, const int32_t* n_tok, const int32_t* base,
                          const buddy_kv_state& kv, int layer, const float* q, void* out, void* out_lo,
                          cudaStream_t s);

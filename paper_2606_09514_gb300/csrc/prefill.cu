@@ -159,7 +159,7 @@ static void pf_block(Ctx& c, const buddy_kv_state& kv, int l, const PfLayerWork&
   e.tok_cap = c.pf_tok_cap;
   {
     ProfScope p(c, s, BUDDY_PROF_PF_GEMM, 1, prof);
-    launch_gemm_pf(c, EPI_QKV, split, l, 0, 0, w.m, e, s);
+    p.rec.launches = launch_gemm_pf(c, EPI_QKV, split, l, 0, 0, w.m, e, s);
   }
   {
     ProfScope p(c, s, BUDDY_PROF_PF_ATTENTION, 1, prof);
@@ -172,7 +172,7 @@ static void pf_block(Ctx& c, const buddy_kv_state& kv, int l, const PfLayerWork&
   e.resid_dst = H;
   {
     ProfScope p(c, s, BUDDY_PROF_PF_GEMM, 1, prof);
-    launch_gemm_pf(c, EPI_RESID, split, l, 1, 1, w.m, e, s);
+    p.rec.launches = launch_gemm_pf(c, EPI_RESID, split, l, 1, 1, w.m, e, s);
   }
   {
     ProfScope p(c, s, BUDDY_PROF_PF_OTHER, 1, prof);
@@ -183,7 +183,7 @@ static void pf_block(Ctx& c, const buddy_kv_state& kv, int l, const PfLayerWork&
   e.out_act_lo = split ? c.pf_act_lo : nullptr;
   {
     ProfScope p(c, s, BUDDY_PROF_PF_GEMM, 1, prof);
-    launch_gemm_pf(c, EPI_SWIGLU, split, l, 2, 0, w.m, e, s);
+    p.rec.launches = launch_gemm_pf(c, EPI_SWIGLU, split, l, 2, 0, w.m, e, s);
   }
   e = PfEpi{};
   e.rows = w.rows;
@@ -191,7 +191,7 @@ static void pf_block(Ctx& c, const buddy_kv_state& kv, int l, const PfLayerWork&
   e.resid_dst = H;
   {
     ProfScope p(c, s, BUDDY_PROF_PF_GEMM, 1, prof);
-    launch_gemm_pf(c, EPI_RESID, split, l, 3, 2, w.m, e, s);
+    p.rec.launches = launch_gemm_pf(c, EPI_RESID, split, l, 3, 2, w.m, e, s);
   }
 }
 
@@ -285,7 +285,7 @@ int run_prefill(Ctx& c, const buddy_kv_state& kv, int B, const int32_t* n_tok_ho
   // blocks 0..c on every token, then the router per prompt
   for (int l = 0; l <= c.cl; ++l) pf_block(c, kv, l, feed, l == 0 ? x : h_out, h_out, s, prof);
   {
-    ProfScope p(c, s, BUDDY_PROF_ROUTE, 1, prof);
+    ProfScope p(c, s, BUDDY_PROF_ROUTE, 4, prof);
     launch_pool_refresh_n(c, kv, B, c.pf_n_tok, s);
     launch_k(pf_gather_kernel, B, 256, 0, s, c.pdl, B, c.d, d_ends, (const float*)h_out,
              (const int32_t*)kv.len, c.pf_n_tok, c.pf_hlast, c.pf_cnt, (const int32_t*)c.status);

@@ -110,3 +110,21 @@ def test_prefill_units(lengths):
             close(kv.view("v", l, i)[:, :n].transpose(0, 1).reshape(n, -1), vv[at:at + n].reshape(n, -1))
             at += n
     close(outs[0][0], h)
+
+
+# decode GEMMs and their fixups up to 256 tokens (gate/up in one K split where its tiles fill most SMs, then
+# without a fixup), one launch per projection above
+@pytest.mark.parametrize("shape,tokens,per_block", [(C.SMALL_QWEN_BF16, 20, 8), (C.LLAMA3_8B, 20, 7), (C.SMALL_QWEN_BF16, 257, 4)],
+                         ids=lambda v: getattr(v, "name", str(v)))
+def test_profiler_counts_prefill_launches(shape, tokens, per_block):
+    s = dataclasses.replace(shape, n_layers=3)
+    w = pkg.pack_layer(synth.layer_weights(s, 1, 0, "cuda"))
+    ctx = pkg.Context.for_shape(s, max_batch=1, max_pos=tokens, max_prefill_tokens=tokens)
+    ctx.buddy_set_weights([w] * 3, synth.dm_weights(s, 1, "cuda"))
+    kv = pkg.KVCache(3, s.n_kv_heads, s.head_dim, [tokens], torch.bfloat16, "cuda")
+    x = synth.prompt_inputs(s, 1, [tokens], "cuda")
+    ctx.buddy_set_profiling(True)
+    ctx.buddy_prefill(kv, [tokens], x, torch.ones(1, dtype=torch.int32, device="cuda"), torch.empty_like(x))
+    prof = ctx.buddy_profile_read()
+    assert {k: prof[k][1] for k in ("pf_gemm", "pf_attention", "route")} == {
+        "pf_gemm": 3 * per_block, "pf_attention": 3, "route": 4}
