@@ -184,48 +184,35 @@ __device__ __forceinline__ void tc_mma_stage(const uint8_t* st, uint32_t d, cons
 }
 
 // ---------------------------------------------------------------------------
-// Panel mode.  Panel layout: K block r of the unit at r * 1024 bytes, rows 0..7
-// of the 128-byte-swizzled K-major tile (rows past m unused); the remainder
+// Panel mode.  Panel layout: K block r of the unit at r * 1024 bytes, the first eight
+// rows of the 128-byte-swizzled K-major tile (those past m unused); the remainder
 // terms at panel_kb * 1024.  An M = 128 operand read from block r spans the
 // following 15 KiB (later blocks, the next panel, or the tail slack): those
 // rows only feed accumulator rows that are discarded.
 // ---------------------------------------------------------------------------
-// 1 / rms of each row, by the 128 epilogue threads (et = 0..127): four
-// rows at a time, eight float4 of each per thread in flight together (a row at a
-// time took 7 us for 7 rows of 4096).  A function of its own, so that the kernel
-// of one or two rows, which does not call it, stays short.
+// 1 / rms of each row wider than kPanelFirstMaxK, by the 128 epilogue threads (et =
+// 0..127), 16 float4 of a row per thread in flight.  A function of its own: the rows of
+// narrower models do not come here, and their kernel stays short.
 static __device__ __noinline__ void tc_panel_inv(const float* nsrc, int K, float neps, int m, int et,
                                                  const int* row_of, float* red, float* inv) {
-  constexpr int RG = 4, KQ = 8;
   const int lane = et & 31, w = et >> 5;
 #pragma unroll 1
-  for (int j0 = 0; j0 < m; j0 += RG) {
-    float ss[RG];
-#pragma unroll
-    for (int r = 0; r < RG; ++r) ss[r] = 0.f;
+  for (int j = 0; j < m; ++j) {
+    const float* h = nsrc + (size_t)row_of[j] * K;
+    float ss = 0.f;
 #pragma unroll 1
-    for (int e0 = 0; e0 < K; e0 += KQ * 512) {
-      float4 x[RG][KQ];
+    for (int e0 = 0; e0 < K; e0 += 16 * 512) {
+      float4 x[16];
 #pragma unroll
-      for (int r = 0; r < RG; ++r) {
-        const float* h = nsrc + (size_t)row_of[min(j0 + r, m - 1)] * K;
-#pragma unroll
-        for (int k = 0; k < KQ; ++k) {
-          const int e = e0 + (et + k * 128) * 4;
-          x[r][k] = e < K ? *reinterpret_cast<const float4*>(h + e) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+      for (int k = 0; k < 16; ++k) {
+        const int e = e0 + (et + k * 128) * 4;
+        x[k] = e < K ? *reinterpret_cast<const float4*>(h + e) : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
-      for (int r = 0; r < RG; ++r)
-#pragma unroll
-        for (int k = 0; k < KQ; ++k)
-          ss[r] += x[r][k].x * x[r][k].x + x[r][k].y * x[r][k].y + x[r][k].z * x[r][k].z + x[r][k].w * x[r][k].w;
+      for (int k = 0; k < 16; ++k) ss += x[k].x * x[k].x + x[k].y * x[k].y + x[k].z * x[k].z + x[k].w * x[k].w;
     }
-#pragma unroll
-    for (int r = 0; r < RG; ++r) {
-      const float s = warp_sum(ss[r]);
-      if (lane == 0 && j0 + r < m) red[(j0 + r) * 4 + w] = s;
-    }
+    ss = warp_sum(ss);
+    if (lane == 0) red[j * 4 + w] = ss;
   }
   epi_bar();
   if (et < m) inv[et] = rsqrtf(((red[et * 4] + red[et * 4 + 1]) + (red[et * 4 + 2] + red[et * 4 + 3])) / (float)K + neps);

@@ -45,8 +45,8 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
   __shared__ volatile int abort_flag;
   __shared__ volatile int consumed;
   __shared__ int last_flag;
-  __shared__ float pred[32], pinv[8];   // panel mode: sums of squares, 1 / rms per row
-  __shared__ int prow[8];               // panel mode: source row of each panel row
+  __shared__ float pred[4 * kTcDeferRows], pinv[kTcDeferRows];   // panel mode: sums of squares, 1 / rms per row
+  __shared__ int prow[kTcDeferRows];                             // panel mode: source row of each panel row
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(DEFER ? kTcDeferThreads : kTcThreads, 1)
     float* gst = reinterpret_cast<float*>(smem + p.gstage_off);
     for (int c = et * 4; c < (kb1 - kb0) * kTileK; c += 128 * 4)
       *reinterpret_cast<float4*>(gst + c) = *reinterpret_cast<const float4*>(p.ngamma + kb0 * kTileK + c);
-    if (et < 8 && et < p.n) prow[et] = p.rows ? p.rows[et] : et;
+    if (et < kTcDeferRows && et < p.n) prow[et] = p.rows ? p.rows[et] : et;
   }
   if (!waited) pdl_wait();
   pdl_trigger();

@@ -137,15 +137,9 @@ def test_f32_tiles_keep_the_warp_sums_precision(d):
     assert value_error(d, 64) < 1.02 * value_error(d, 24)
 
 
-@pytest.mark.parametrize("base", [C.LLAMA3_8B, C.LLAMA2_13B], ids=lambda s: s.name)
-def test_scores_keep_the_feeding_blocks_precision(base):
-    """Scores after one block over a single position, against 64 bits from the stored V on.  What is left is
-    the fp32 sums: a tensor-core accumulator truncates at each K = 16 step, about 2^-24 of the sum a time,
-    and a sum of n steps (hi and lo) ends n / 2^24 off.  Gate and up in four K splits take 128 to 160 steps,
-    down about 200: 2e-5 of the block's update, less than half of the scores; gate and up in one sum take
-    512 to 640 and twice that in all."""
-    s = dataclasses.replace(base, n_layers=34)
-    B, T = 16, torch.float64
+def score_error(s, B):
+    """Scores of a decode step after one block over a single position, against 64 bits from the stored V on."""
+    T = torch.float64
     w = synth.layer_weights(s, 5, 0, "cuda")
     dm = synth.dm_weights(s, 5, "cuda")
     ctx = pkg.Context.for_shape(s, max_batch=B, max_pos=4)
@@ -164,9 +158,24 @@ def test_scores_keep_the_feeding_blocks_precision(base):
     x = torch.cat([v, x + (torch.nn.functional.silu(g) * u) @ layer["w_down"].to(T).T], 1)
     d = {k: t.to(T) for k, t in dm.items()}
     ref = torch.nn.functional.silu(x @ d["w1"].T + d["b1"]) @ d["w2"].T + d["b2"]
-    err = float((sc.to(T) - ref).norm() / ref.norm())
-    print("score error", err)
-    assert err < 1.0e-5
+    return float((sc.to(T) - ref).norm() / ref.norm())
+
+
+@pytest.mark.parametrize("base", [C.LLAMA3_8B, C.LLAMA2_13B], ids=lambda s: s.name)
+def test_scores_keep_the_feeding_blocks_precision(base):
+    """What is left is the fp32 sums: a tensor-core accumulator truncates at each K = 16 step, about 2^-24 of
+    the sum a time, and a sum of n steps (hi and lo) ends n / 2^24 off.  Gate and up in four K splits take 128
+    to 160 steps, down about 200: 2e-5 of the block's update, less than half of the scores; gate and up in one
+    sum take 512 to 640 and twice that in all."""
+    assert score_error(dataclasses.replace(base, n_layers=34), 16) < 1.0e-5
+
+
+# rows wider than one pass of the epilogue warps holds (8192): 1056 steps if no projection is split
+@pytest.mark.parametrize("batch", [1, 2])
+def test_panels_of_a_wide_model(batch):
+    wide = dataclasses.replace(C.LLAMA3_8B, name="wide", n_layers=34, d_model=8448, n_q_heads=66, n_kv_heads=11,
+                               ffn_dim=2048, random_norm=True)
+    assert score_error(wide, batch) < 1056 / 2**24
 
 
 def silu_context(r, n_layers):
