@@ -418,16 +418,21 @@ static int choose_splits(int tiles, int kb, int sms) {
   return best_eff > 0 ? best : fb;
 }
 
-// The same with a deferred fixup.  A gate/up GEMM that is not split applies SwiGLU
-// itself, without workspace or fixup kernel: taken when its tiles keep at least
-// 70% of the SMs streaming (the rest of HBM's rate they reach all the same:
-// Llama-3-8B's 112 tiles at 64 rows take as long as 448 units, and the 10 us
-// fixup is saved; 6 blocks 1259 -> 1209 us).  Not in a decode block that feeds the
-// router (hi + lo activations): its sums would run over the whole K in one fp32
-// accumulator, four times as long as with the splits, and the scores' error against
-// 64 bits doubled (Llama-3-8B, 3 to 200 rows: 1.0e-5 -> 2.2e-5 of their size).
-static int defer_splits(int which, int tiles, int kb, int sms) {
-  if (which == 2 && 10 * tiles >= 7 * sms && tiles <= sms) return 1;
+// The same with a deferred fixup, for up to `rows` rows.  A gate/up GEMM that is not
+// split applies SwiGLU itself, without workspace or fixup kernel: taken above 16 rows
+// when its tiles keep at least 70% of the SMs streaming (the rest of HBM's rate they
+// reach nearly all the same).  Steps of 6 blocks of width 4096, split and not: 112
+// tiles (74% of the SMs), 8 rows 617 and 623 us, 16 rows 688 and 693, 24 rows 709 and
+// 698, 64 rows 817 and 779, 256 rows 1610 and 1425; 88 tiles (58%), 16 rows 620 and
+// 630, 24 rows 625 and 627, 64 rows 752 and 719; 72 tiles (47%), 64 rows 674 and 675,
+// 256 rows 1285 and 1303.  A prefill's projections are not split at any number of tokens
+// (4 blocks of Llama-3-8B, 9 tokens: 391 us split, 388 us not).
+// Not in a decode block that feeds the router (hi + lo activations): its sums would run
+// over the whole K in one fp32 accumulator, four times as long as with the splits, and
+// the scores' error against 64 bits doubled (Llama-3-8B, 3 to 200 rows: 1.0e-5 -> 2.2e-5
+// of their size).
+static int defer_splits(int which, int rows, int tiles, int kb, int sms) {
+  if (which == 2 && rows > 16 && 10 * tiles >= 7 * sms && tiles <= sms) return 1;
   return choose_splits(tiles, kb, sms);
 }
 
@@ -471,13 +476,13 @@ int gemm_tc_prepare(Ctx& c) {
     gemm_shape(c, w, &N, &K, &tiles);
     const int kb = (K + kTileK - 1) / kTileK;
     c.tc_splits[1][w] = choose_splits(tiles, kb, c.num_sms);
-    c.tc_splits[0][w] = c.maxB > kTcDeferRows ? defer_splits(w, tiles, kb, c.num_sms) : c.tc_splits[1][w];
+    c.tc_splits[0][w] = defer_splits(w, c.maxB, tiles, kb, c.num_sms);
     c.tc_tiles[w] = tiles;
     // every unit stages its accumulator rows in the workspace
     ws = std::max(ws, (size_t)tiles * std::max(c.tc_splits[0][w], c.tc_splits[1][w]) * c.tc_rows_max * c.tc_bw);
     if (c.pf_max > 0) {   // prompts of few tokens
       const int rows = std::min(kPfSmallRows, (c.pf_max + 15) & ~15);
-      ws = std::max(ws, (size_t)tiles * defer_splits(w, tiles, kb, c.num_sms) * std::max(16, rows) * c.tc_bw);
+      ws = std::max(ws, (size_t)tiles * defer_splits(w, kPfSmallRows, tiles, kb, c.num_sms) * std::max(16, rows) * c.tc_bw);
     }
     max_tiles = std::max(max_tiles, tiles);
   }
@@ -696,7 +701,7 @@ static int launch_pf_small(const Ctx& c, int layer, int which, int xi, int m, co
   a.which = which;
   size_t smem = 0;
   TcParams p = tc_params(c, a, &smem);
-  p.splits = defer_splits(which, p.n_tiles, p.kb_total, c.num_sms);
+  p.splits = defer_splits(which, kPfSmallRows, p.n_tiles, p.kb_total, c.num_sms);
   p.kb_per_split = (p.kb_total + p.splits - 1) / p.splits;
   p.units = p.n_tiles * p.splits;
   p.mt = m > 128 ? 2 : 1;

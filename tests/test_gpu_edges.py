@@ -178,6 +178,27 @@ def test_panels_of_a_wide_model(batch):
     assert score_error(wide, batch) < 1056 / 2**24
 
 
+# gate/up split up to 16 rows, whole above: the same step by its profile and by its values
+@pytest.mark.parametrize("batch,fixups", [(3, 4), (16, 4), (17, 3)])
+def test_gate_up_splits_by_rows(batch, fixups):
+    s = dataclasses.replace(C.LLAMA3_8B, n_layers=3)
+    layer = pkg.pack_layer(synth.layer_weights(s, 5, 0, "cuda"))
+    h, k = synth.h_in(s, 5, 0, range(batch), "cuda"), torch.ones(batch, dtype=torch.int32, device="cuda")
+    outs = []
+    for max_batch in (batch, 17 if batch < 17 else 200):   # both forms of the rows up to 16
+        ctx = pkg.Context.for_shape(s, max_batch=max_batch, max_pos=4)
+        ctx.buddy_set_weights([layer] * 3, synth.dm_weights(s, 5, "cuda"))
+        kv = pkg.KVCache(3, s.n_kv_heads, s.head_dim, [1] * batch, torch.bfloat16, "cuda")
+        out = torch.empty_like(h)
+        ctx.buddy_set_profiling(True)
+        ctx.buddy_decode_step(kv, h, k, out)
+        n = ctx.buddy_profile_read()["gemm_fixup"][1]
+        assert n == (2 * fixups + 4 if max_batch == batch else 10)   # the first block's gate/up is always split
+        outs.append(out)
+    # bf16 activations between the projections, as parity.py
+    assert float(((outs[0] - outs[1]).abs().amax(1) / outs[1].abs().amax(1)).max()) < 2e-2
+
+
 def silu_context(r, n_layers):
     """A router whose scores are silu(x + b1) of the first r channels x of h1."""
     s = dataclasses.replace(C.SMALL_F32, n_layers=n_layers, dm_hidden=r)

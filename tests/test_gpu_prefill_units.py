@@ -114,7 +114,7 @@ def test_prefill_units(lengths):
 
 # decode GEMMs and their fixups up to 256 tokens (gate/up in one K split where its tiles fill most SMs, then
 # without a fixup), one launch per projection above
-@pytest.mark.parametrize("shape,tokens,per_block", [(C.SMALL_QWEN_BF16, 20, 8), (C.LLAMA3_8B, 20, 7), (C.SMALL_QWEN_BF16, 257, 4)],
+@pytest.mark.parametrize("shape,tokens,per_block", [(C.SMALL_QWEN_BF16, 20, 8), (C.LLAMA3_8B, 16, 7), (C.SMALL_QWEN_BF16, 257, 4)],
                          ids=lambda v: getattr(v, "name", str(v)))
 def test_profiler_counts_prefill_launches(shape, tokens, per_block):
     s = dataclasses.replace(shape, n_layers=3)
