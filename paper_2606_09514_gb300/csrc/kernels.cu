@@ -999,10 +999,11 @@ template <typename T>
 static void pool_refresh_impl(const Ctx& c, const buddy_kv_state& kv, int n_seq, const int32_t* ids, int n_new,
                               const int32_t* n_new_of, cudaStream_t s) {
   const int l = c.cl;
-  // Clusters while they fit the GPU at once (four CTAs per SM); with more pairs a
-  // CTA each: whole calls over three layers with 40 heads, 32 sequences of 2
-  // positions 210 -> 44 us, 8 heads, 19 sequences of 750 positions 83 -> 67 us.
-  const bool few = (int64_t)n_seq * c.nkv * kPoolCtas <= 4 * c.num_sms;
+  // Clusters while there are at most three of their CTAs per SM, with more pairs a CTA
+  // each: whole calls over three layers, clusters and one CTA, 40 pairs of 4,100 positions
+  // 127 and 152 us, 48 pairs of 1,100 positions 51 and 49 us, 64 pairs of 2,100 98 and 94
+  // us, 80 pairs of 1,100 76 and 65 us, 1,280 pairs of 102 223 and 51 us.
+  const bool few = (int64_t)n_seq * c.nkv * kPoolCtas <= 3 * c.num_sms;
   launch_k(few ? pool_refresh_kernel<T, kPoolCtas> : pool_refresh_kernel<T, 1>, dim3(few ? kPoolCtas : 1, c.nkv, n_seq),
            kPoolThreads, 0, s, c.pdl, n_new, n_new_of, c.nkv, c.hd, c.feature, ids,
            cache_len(c, kv, l), kv.seq_off, kv.cap, (const T*)kv.k_cache[l], (const T*)kv.v_cache[l], kv.pool_sum,
