@@ -456,7 +456,9 @@ def measure_prefill(w, K, W, dev, ws, local):
                         "traffic": None, "flops_per_call": c["gemm_flops"], "peak_source": "measured bf16_tflops"},
            "call_roofline_frac": round(max(c["flops"] / (burst * 1e12), c["bytes"] / (hbm * 1e9)) * 1e3 / call_ms, 4),
            "kernel_ms_per_call": {k: round(v[0], 4) for k, v in prof.items() if v[1] > 0},
-           "paths": ctx.buddy_get_paths(), "clocks": clk.summary()}
+           "paths": {"gemm": "tcgen05 bf16 (TMA, TMEM), CTA pairs above 256 tokens in a block",
+                     "attention": "tcgen05 (TMEM), causal", "rmsnorm": "separate kernel"},
+           "clocks": clk.summary()}
     ctx.close()
     del dw, kv, ctx, x, h_out
     torch.cuda.empty_cache()

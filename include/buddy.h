@@ -40,8 +40,13 @@
  *     is reported by buddy_device_status().
  *   - The library allocates device memory only in buddy_create (scratch sized
  *     by max_batch, max_pos and max_prefill_tokens), in buddy_set_weights
- *     (tensor descriptors, split-K workspace) and in
- *     buddy_set_budget_predictor (its hidden units).
+ *     (tensor descriptors, split-K workspace; with max_prefill_tokens > 0 also
+ *     40 MB for the parts of cut prefill units) and in
+ *     buddy_set_budget_predictor (its hidden units).  With max_prefill_tokens
+ *     > 0 buddy_create also pins host memory, as much as the device holds of a
+ *     call's tables: about n_layers * (max_prefill_tokens * (4 + n_q_heads / 4)
+ *     + max_batch * n_q_heads * 16) bytes (30 MB for 32 layers, 32 heads, 256
+ *     sequences and 65,536 tokens).
  */
 #ifndef BUDDY_H_
 #define BUDDY_H_
@@ -316,7 +321,8 @@ BUDDY_API int buddy_set_options(buddy_ctx* ctx, int32_t use_graph);
  * bf16), paths[1] attention (0 CUDA-core, 1 mma.sync tensor-core loop over
  * the whole GPU, 2 the same contractions with one thread-block cluster per
  * (row, KV head) stream, for small batches),
- * paths[2] RMSNorm computed inside the QKV and gate/up GEMMs (0/1),
+ * paths[2] RMSNorm computed inside the QKV and gate/up GEMMs (0/1; fp32: by
+ * the rows of each call, here for max_batch rows),
  * paths[3] split-K sums in a separate fixup kernel (0/1).  n <= 4 entries. */
 BUDDY_API int buddy_get_paths(buddy_ctx* ctx, int32_t* paths, int32_t n);
 

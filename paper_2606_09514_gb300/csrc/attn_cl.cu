@@ -5,17 +5,18 @@
 // streams of ~2k positions) and short: cutting them across the whole GPU
 // leaves tens of partial results per stream whose merge costs as much as the
 // streaming.  Here a cluster of C CTAs (cl_size: the largest of 16, 8, 4 and 2
-// of which all streams' clusters fit on the GPU at once) takes one stream: CTA r streams positions [r np / C, (r+1) np / C)
-// with its 4 warps (contiguous quarters, 32-position chunks through a
+// of which all streams' clusters fit on the GPU at once) takes one stream: CTA r
+// streams positions [r np / C, (r+1) np / C) with its 4 warps (contiguous quarters, 32-position chunks through a
 // 2-buffer cp.async ring per warp; the contractions are those of the
 // tensor-core loop in attn_tc.cuh: S^T = K Q^T and O^T += V^T P^T on
 // mma.sync m16n8k16 with the G <= 8 query heads as the 8 columns, base-2
 // online softmax).  The 4 warps' partials are merged in shared memory and
-// every CTA stores its partial into CTA 0's gather area through distributed
-// shared memory (st.shared::cluster), cut by output: the G x HD outputs of
-// the stream are split into C contiguous slices and CTA s owns slice s.
-// Every CTA stores its (m, l) of each head and its unnormalised output of
-// each (head, channel) into the gather area of that output's owner; after
+// exchanged through distributed shared memory (st.shared::cluster), cut by
+// output: the G x HD outputs of the stream are split into C contiguous slices
+// and CTA s owns slice s.  Every CTA stores its (m, l) of each head and its
+// unnormalised output of each (head, channel) into the gather area of that
+// output's owner (once the owner has started: a cluster barrier whose first
+// half is passed at the kernel's start); after
 // one cluster barrier (release / acquire) every CTA merges the C partials of
 // its own slice from its own shared memory (log-sum-exp, in rank order:
 // deterministic) and writes those outputs.  No kernel-wide or cross-cluster

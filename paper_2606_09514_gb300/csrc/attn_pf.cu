@@ -18,7 +18,8 @@
 //               the row's maximum only when that rises by more than 8 (p stays
 //               below 2^8), so that the output is rescaled a few times per row
 //               instead of once per key tile; the final division makes the
-//               choice of m immaterial;
+//               choice of m immaterial (the online softmax of Milakov and
+//               Gimelshein 2018, rescaled late as FlashAttention-4 does);
 //   O += P V    M = 128, N = HD, K = 128: P from TMEM, V from shared memory
 //               (MN-major), O in TMEM.
 // With SPLIT every product is issued for both terms.

@@ -5,8 +5,8 @@
 // A prefill block runs its projections on every token of the prompts that
 // selected it, thousands of rows: the GEMM is bound by the tensor pipe, not
 // by the weight stream.  A work unit is a 256-row M-tile of X times one
-// 256-row weight tile over the whole K (no split), computed by a pair of CTAs
-// on two SMs (a cluster of 2, tcgen05 cta_group::2): each CTA holds 128 rows of
+// 256-row weight tile over the whole K (but for the last units, below), computed by
+// a pair of CTAs on two SMs (a cluster of 2, tcgen05 cta_group::2): each CTA holds 128 rows of
 // X and half of the weight tile, and 128 rows of the accumulator.  A K block
 // thus costs an SM 32 KiB of copies instead of the 48 KiB of a 128 x 256 tile
 // of its own, and the ring gets seven stages instead of four; a stage's four
@@ -19,7 +19,8 @@
 // weights: for a gate/up projection larger than L2 that is an HBM pass per
 // M-tile.)
 //
-// Units that do not fill a last wave of pairs are cut along K (pf_bound): each
+// Units that do not fill a last wave of pairs are cut along K (pf_bound; the cut of
+// Stream-K, Osama et al. 2023, for the remainder only): each
 // pair takes an equal, contiguous share of their K blocks, first of all its work,
 // stages the accumulator of a part in a workspace slot, and the pair that
 // completes a unit sums the parts in K order and applies the epilogue.  With one

@@ -105,10 +105,10 @@ def test_decode_parity_bf16(w):
     assert worst < 2e-2
 
 
-# Batch sizes at the mode boundaries of the bf16 path: up to 8 rows the QKV
+# Batch sizes at the mode boundaries of the bf16 path: up to 2 rows the QKV
 # and gate/up GEMMs normalise in-kernel panels and the last K split applies
-# the epilogue, above 8 a fixup kernel does; up to 16 rows the router's first
-# layer is one CTA per hidden unit, above it a packed tiled GEMM; above 128
+# the epilogue, above 2 a fixup kernel does; up to 16 rows the router's first
+# layer is one CTA per hidden unit, above it a tiled GEMM; above 128
 # rows the GEMMs take two M-tiles.
 @pytest.mark.parametrize("base,batch", [(C.T_QWEN, 8), (C.T_QWEN, 9), (C.T_QWEN, 16), (C.T_QWEN, 17),
                                         (C.T_QWEN, 128), (C.T_QWEN, 129), (C.T_GQA, 8), (C.T_GQA, 17)],
