@@ -183,9 +183,6 @@ extern "C" void buddy_destroy(buddy_ctx* ctx) {
   free_ctx(ctx);
 }
 
-// Device buffers the kernels read or write with 16-byte vector accesses.
-static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
-
 extern "C" int buddy_set_weights(buddy_ctx* ctx, const buddy_layer_weights* layers,
                                  const buddy_dm_weights* dm) {
   if (!ctx || !layers || !dm) return BUDDY_ERR_ARG;
@@ -199,7 +196,7 @@ extern "C" int buddy_set_weights(buddy_ctx* ctx, const buddy_layer_weights* laye
       if (!aligned16(p)) return BUDDY_ERR_ARG;
     if (c.cfg.qkv_bias && !w.b_qkv) return BUDDY_ERR_ARG;
   }
-  if (!dm->w1 || !dm->b1 || !dm->w2 || !dm->b2) return BUDDY_ERR_ARG;
+  if (!dm->w1 || !dm->b1 || !dm->w2 || !dm->b2 || !aligned16(dm->w1)) return BUDDY_ERR_ARG;
   c.layers.assign(layers, layers + c.L);
   if (!c.cfg.qkv_bias)
     for (auto& w : c.layers) w.b_qkv = nullptr;
@@ -218,7 +215,7 @@ extern "C" int buddy_set_weights(buddy_ctx* ctx, const buddy_layer_weights* laye
 extern "C" int buddy_set_budget_predictor(buddy_ctx* ctx, const buddy_predictor_weights* bp) {
   if (!ctx) return BUDDY_ERR_ARG;
   Ctx& c = ctx->c;
-  if (bp && (!bp->w1 || !bp->b1 || !bp->w2 || !bp->b2 || bp->hidden < 1 || bp->hidden > 65536))
+  if (bp && (!bp->w1 || !bp->b1 || !bp->w2 || !bp->b2 || bp->hidden < 1 || bp->hidden > 65536 || !aligned16(bp->w1)))
     return BUDDY_ERR_ARG;
   CK(cudaDeviceSynchronize());   // dm_u may be in use by queued work
   for (auto& kv : c.graphs) cudaGraphExecDestroy(kv.second);
@@ -624,7 +621,7 @@ extern "C" int buddy_route(buddy_ctx* ctx, const buddy_kv_state* kv, int32_t bat
   Ctx& c = ctx->c;
   if (!c.have_weights) return BUDDY_ERR_STATE;
   if (batch < 1 || batch > c.maxB || !h1 || !k || !aligned16(h1)) return BUDDY_ERR_ARG;
-  if (!kv || !kv->len || !kv->pool_sum || !kv->cap || kv->batch < batch) return BUDDY_ERR_ARG;
+  if (!kv || !kv->len || !kv->pool_sum || !kv->cap || kv->batch < batch || !aligned16(kv->pool_sum)) return BUDDY_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   // positions: the cache already holds the newest token (len >= 1)
   launch_route(c, batch, h1, kv->pool_sum, kv->len, 0, k, mask_out, sel_out, scores_out, s, kv);

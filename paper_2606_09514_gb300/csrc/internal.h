@@ -112,6 +112,9 @@ struct RouteCheck {
   int32_t* out;
 };
 
+// Device buffers the kernels read or write with 16-byte vector accesses.
+inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
 // Launch with programmatic stream serialisation when `pdl` is set (the kernel
 // then overlaps its prologue with the predecessor and synchronises with
 // pdl_wait()).

@@ -81,7 +81,8 @@ extern "C" int buddy_route_noalloc(int32_t n_layers, int32_t d_model, int32_t n_
                                    const int32_t* len, const float* h1, const int32_t* k,
                                    int32_t* sel_out, uint8_t* mask_out, float* scores_out,
                                    int32_t* flags_out, void* stream) {
-  if (!dm || !dm->w1 || !dm->b1 || !dm->w2 || !dm->b2 || !pool_sum || !len || !h1 || !k)
+  if (!dm || !dm->w1 || !dm->b1 || !dm->w2 || !dm->b2 || !pool_sum || !len || !h1 || !k || !aligned16(dm->w1) ||
+      !aligned16(pool_sum) || !aligned16(h1))
     return BUDDY_ERR_ARG;
   if (n_layers < 3 || n_layers > kMaxLayers || n_q_heads <= 0 || n_kv_heads <= 0 ||
       (head_dim != 64 && head_dim != 128) || n_q_heads % n_kv_heads != 0 ||

@@ -71,6 +71,16 @@ def test_invalid_configs_rejected_before_any_cuda_call(lib):
     assert lib.buddy_version() >= 1
 
 
+@pytest.mark.parametrize("bad", ["w1", "pool_sum", "h1"])
+def test_noalloc_router_rejects_misaligned_buffers(lib, bad):
+    """Before any CUDA call: the addresses are made up and not read."""
+    from paper_2606_09514_gb300 import binding as B
+    at = {k: 0x10000 + (4 if k == bad else 0) for k in ("w1", "pool_sum", "h1")}
+    dm = B.buddy_dm_weights(at["w1"], 0x20000, 0x20000, 0x20000, None, 0.0)
+    assert lib.buddy_route_noalloc(8, 256, 4, 4, 64, 16, ctypes.byref(dm), 1, at["pool_sum"], 0x20000, at["h1"],
+                                   0x20000, None, None, None, None, None) == B.BUDDY_ERR_ARG
+
+
 def test_ctypes_structs_match_c_layout():
     """sizeof/offsetof of the header's structs (compiled with gcc) equal the
     binding's ctypes layouts."""

@@ -364,6 +364,32 @@ def test_contexts_of_other_shapes_side_by_side():
             assert torch.equal(step(live[i], w), alone[i])
 
 
+def test_misaligned_router_buffers_rejected_on_host():
+    """The Decision Module's and the Budget Predictor's first matrix and the pooled sums, off by 4 bytes."""
+    w = rows_of(C.T_GQA, 3)
+    dw = D.build(w)
+    s = w.shape
+    off = lambda t: torch.cat([t.new_zeros(1), t.reshape(-1)])[1:].view(t.shape)
+    bad = off(dw.dm["w1"])
+    assert bad.data_ptr() % 16 == 4 and bad.is_contiguous()
+    h1, sc = synth.h_in(s, 5, 0, range(3), "cuda"), torch.full((3, s.n_cand), 7.0, device="cuda")
+    dw.kv.len.clamp_(min=1)
+    pred = {k: dw.dm[k] for k in ("b1", "w2", "b2")}
+    pool = dw.kv.state.pool_sum
+    for call in (lambda: dw.ctx.buddy_set_weights(dw.layers, {**dw.dm, "w1": bad}),
+                 lambda: dw.ctx.buddy_set_budget_predictor({**pred, "w1": bad}),
+                 lambda: dw.ctx.buddy_route(dw.kv, h1, dw.k, scores_out=sc)):
+        dw.kv.state.pool_sum = pool + 4
+        with pytest.raises(Bd.BuddyError) as e:
+            call()
+        assert e.value.code == Bd.BUDDY_ERR_ARG
+    dw.kv.state.pool_sum = pool
+    torch.cuda.synchronize()
+    assert bool((sc == 7.0).all())
+    dw.ctx.buddy_route(dw.kv, h1, dw.k, scores_out=sc)
+    assert dw.ctx.buddy_device_status() == 0 and not bool((sc == 7.0).any())
+
+
 def test_panel_wait_limit_runs_out_and_context_recovers():
     """As the other batches' test: 1 ns runs out, the restored limit gives a fresh context's result."""
     w = C.scaled(C.T_GQA, ctx=[5, 200], k=[1, 3], name="t-gqa-b2-timeout")
