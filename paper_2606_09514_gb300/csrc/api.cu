@@ -621,7 +621,8 @@ extern "C" int buddy_route(buddy_ctx* ctx, const buddy_kv_state* kv, int32_t bat
   Ctx& c = ctx->c;
   if (!c.have_weights) return BUDDY_ERR_STATE;
   if (batch < 1 || batch > c.maxB || !h1 || !k || !aligned16(h1)) return BUDDY_ERR_ARG;
-  if (!kv || !kv->len || !kv->pool_sum || !kv->cap || kv->batch < batch || !aligned16(kv->pool_sum)) return BUDDY_ERR_ARG;
+  if (!kv || !kv->len || !kv->pool_sum || !kv->cap || kv->batch < batch || !aligned16(kv->pool_sum))
+    return BUDDY_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   // positions: the cache already holds the newest token (len >= 1)
   launch_route(c, batch, h1, kv->pool_sum, kv->len, 0, k, mask_out, sel_out, scores_out, s, kv);

@@ -129,8 +129,10 @@ bool attention_tc(const Ctx& c) {
 template <int HD>
 static cudaError_t attn_tc_prepare(Ctx& c) {
   const size_t smem = attn_tc_smem_bytes(HD, c.maxB);
-  const cudaError_t e = attn_prepare(attn_tc_kernel<HD, false>, kTcaThreads, smem, kTcaSmemLimit, c.num_sms, &c.attn_grid[0]);
-  return e != cudaSuccess ? e : attn_prepare(attn_tc_kernel<HD, true>, kTcaThreads, smem, kTcaSmemLimit, c.num_sms, &c.attn_grid[1]);
+  const cudaError_t e = attn_prepare(attn_tc_kernel<HD, false>, kTcaThreads, smem, kTcaSmemLimit, c.num_sms,
+                                     &c.attn_grid[0]);
+  return e != cudaSuccess ? e : attn_prepare(attn_tc_kernel<HD, true>, kTcaThreads, smem, kTcaSmemLimit, c.num_sms,
+                                             &c.attn_grid[1]);
 }
 
 cudaError_t attention_prepare(Ctx& c) {

@@ -6,8 +6,9 @@
 // leaves tens of partial results per stream whose merge costs as much as the
 // streaming.  Here a cluster of C CTAs (cl_size: the largest of 16, 8, 4 and 2
 // of which all streams' clusters fit on the GPU at once) takes one stream: CTA r
-// streams positions [r np / C, (r+1) np / C) with its 4 warps (contiguous quarters, 32-position chunks through a
-// 2-buffer cp.async ring per warp; the contractions are those of the
+// streams positions [r np / C, (r+1) np / C) with its 4 warps (contiguous
+// quarters, 32-position chunks through a 2-buffer cp.async ring per warp; the
+// contractions are those of the
 // tensor-core loop in attn_tc.cuh: S^T = K Q^T and O^T += V^T P^T on
 // mma.sync m16n8k16 with the G <= 8 query heads as the 8 columns, base-2
 // online softmax).  The 4 warps' partials are merged in shared memory and
@@ -375,7 +376,8 @@ __global__ void __launch_bounds__(kClThreads) attn_cl_kernel(AttnArgs<bf16> A) {
 template <int HD, bool SPLIT>
 static cudaError_t cl_prepare(int* cap) {
   const size_t smem = attn_cl_smem<HD>();
-  cudaError_t e = cudaFuncSetAttribute(attn_cl_kernel<HD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e =
+      cudaFuncSetAttribute(attn_cl_kernel<HD, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   for (int v = 0; v < kClSizes; ++v) {
     const int C = kClMaxCtas >> v;
